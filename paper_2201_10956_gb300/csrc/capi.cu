@@ -248,7 +248,8 @@ struct epi3_handle {
     void* d_pair_scratch = nullptr;  // pairwise scan: selection passes + outputs
     size_t pair_scratch_bytes = 0;
     int2* d_marg = nullptr;
-    float4* d_ptf = nullptr;         // tensor scan: pair tables + 3 as FP32
+    float4* d_yz = nullptr;          // compacted scan: (Y, Z) pair tables in its epilogue's form
+    float4* d_ptf = nullptr;         // one-hot tensor scan: pair tables + 3 as FP32
     float2* d_margf = nullptr;       // tensor scan: marginals + 9 as FP32
     PairTables ptab{};
     uint8_t* d_oh = nullptr;      // pre-tiled one-hot operand of the tensor-core form
@@ -274,6 +275,8 @@ struct epi3_handle {
     size_t cmp_bytes = 0;
     size_t cmp_cap = (size_t)2 << 30;  // option "cmp_buffer_mb": bytes of compacted chunks at once
     CmpFirst* d_firsts = nullptr; // per first SNP: chunk bases, K-steps, tiles
+    CmpGroup* d_groups = nullptr; // groups of first SNPs that a run of tiles covers
+    CmpBoundTerms bound{};        // the compacted scan's table-free bound
     std::vector<int2> h_marg;     // marginals on the host (the compacted sets' sizes)
     int4* d_tiles = nullptr;      // tile list of the tensor-core form
     long long n_tiles = 0, tiles_pb = -1, tiles_pe = -1;
@@ -308,10 +311,12 @@ void release(epi3_handle* h) {
     dev_free(h->d_pair_scratch, synced);
     dev_free(h->d_marg, synced);
     dev_free(h->d_ptf, synced);
+    dev_free(h->d_yz, synced);
     dev_free(h->d_margf, synced);
     dev_free(h->d_oh, synced);
     dev_free(h->d_cmp, synced);
     dev_free(h->d_firsts, synced);
+    dev_free(h->d_groups, synced);
     dev_free(h->d_tiles, synced);
     dev_free(h->d_cd, synced);
     dev_free(h->d_prof, synced);
@@ -406,6 +411,43 @@ int build_k2_tables(epi3_handle* h) {
     return EPI3_OK;
 }
 
+// The compacted scan's table-free bound.  With u = count + 1 per cell and class, us = u0 + u1, um
+// the smaller class's u and q = um (us - um) / us, Stirling's form (lf(n) = (n + 1/2) ln(n + 1) -
+// (n + 1) + ln(2 pi)/2 + e(n), 0 < e(n) <= 1/(12 (n + 1))) makes a table's score
+//     K2 = sum us H(um / us) + (1/2) sum ln q - 27 ln(2 pi)/2 + remainders,
+// H the binary entropy in nats and the remainders at least -1/6 per cell.  The entropy is bounded
+// from below by a parabola that touches it at p0 = (sum um) / (sum us), the same for every table:
+//     H(p) >= H(p0) + H'(p0) (p - p0) - c (p - p0)^2,  c = max over p of KL(p || p0) / (p - p0)^2,
+// and KL(p || p0) / (p - p0)^2 = integral over s in [0, 1] of (1 - s) / (t (1 - t)), t = p0 + s (p -
+// p0), is convex in p, so its largest value is at p = 0 or 1.  Summed with weights us the linear
+// term vanishes and sum us (p - p0)^2 = S p0 (1 - p0) - sum q, S = sum us = N + 54, hence
+//     K2 >= c sum q + (1/2) sum ln q - [c S p0 (1 - p0) - S H(p0) + 27 ln(2 pi)/2 + 27/6].
+// At the usual class shares c is 1.4 to 1.8 times the parabola's own curvature, which costs a table
+// without association (sum us (p - p0)^2 c / 1.4 ~ 13 nats) 5 to 10 nats: about what the other
+// table-free bound's doubled error term costs, with one reciprocal per cell instead of three logs.
+// FP32 rounding, S1 = sum um (q <= um; p0 <= 1/2, so c S1 <= 1.4 S):
+//     q: the reciprocal (1 ulp), the product and the FMA: um 2^-22 each, S1 2^-22 together, c-fold
+//     in the sum and, with q >= 1/2, once more in (1/2) ln q; the sum's 27 additions: 2^-24 S1
+//     each, c-fold; c's and the last FMA's rounding: 3 2^-24 (c S1 + 200); logs and products: under
+//     0.01; the FP32 score against K2: rel * K + abs as in build_k2_tables.
+// The rounding terms are doubled.
+void cmp_bound_terms(epi3_handle* h) {
+    const int cm = h->N1 <= h->N0 ? 1 : 0;
+    const double S = (double)h->N + 54.0, S1 = (double)(cm ? h->N1 : h->N0) + 27.0, p0 = S1 / S;
+    const double c = std::max(-std::log1p(-p0) / (p0 * p0), -std::log(p0) / ((1.0 - p0) * (1.0 - p0)));
+    const double H = -p0 * std::log(p0) - (1.0 - p0) * std::log1p(-p0);
+    const double u = std::ldexp(1.0, -24);
+    const double kmax = 27.0 * std::log((double)h->N + 2.0) + (double)h->N * std::log(2.0);
+    const double rnd = 4.0 * u * S1 * (c + 1.1) + 27.0 * u * S1 * c + 3.0 * u * (c * S1 + 200.0) + 0.01 +
+                       (double)h->k2.rel * kmax + (double)h->k2.abs_;
+    const double slack = 27.0 / 6.0 + 2.0 * rnd;
+    h->bound.c = (float)c;
+    h->bound.slack = (float)slack;
+    h->bound.off = std::nextafter((float)(c * S * p0 * (1.0 - p0) - S * H + 27.0 * 0.9189385332046727 + slack),
+                                  INFINITY);
+    h->bound.minor = cm;
+}
+
 int create_impl(epi3_handle* h, const uint8_t* geno, const uint8_t* pheno) {
     const size_t MN = (size_t)h->M * h->N;
     uint8_t* d_geno = nullptr;
@@ -484,6 +526,7 @@ int create_impl(epi3_handle* h, const uint8_t* geno, const uint8_t* pheno) {
     cleanup();
     if (rc != EPI3_OK) return rc;
     if ((rc = build_k2_tables(h)) != EPI3_OK) return rc;
+    cmp_bound_terms(h);
     // FP32 candidate list: the CTAs flush their in-band candidates before the shared threshold
     // tightens, about 10^5 of them on a scan that fills the GPU (a list that overflows costs a
     // whole rescan, in a batch a second replay of every cohort)
@@ -525,6 +568,15 @@ int ensure_pair_floats(epi3_handle* h) {
            "FP32 pair tables launch");
         h->ptab.ptf = h->d_ptf;
         h->ptab.margf = h->d_margf;
+    }
+    return EPI3_OK;
+}
+
+int ensure_yz(epi3_handle* h) {
+    if (!h->d_yz) {
+        CK(dev_alloc((void**)&h->d_yz, sizeof(float4) * 16 * (size_t)yz_blocks(h->M)), "alloc paired tables");
+        CK(launch_pair_yz(h->d_pt, h->ptab.n_pairs, h->M, h->bound.minor, h->d_yz, h->stream),
+           "paired tables launch");
     }
     return EPI3_OK;
 }
@@ -830,8 +882,10 @@ int scan_mma_impl(epi3_handle* h, int path, long long pb, long long pe, long lon
 // (the two work terms of this form, used by the tuner to extrapolate a slice's timing).
 struct CmpPlan {
     std::vector<CmpFirst> firsts;
+    std::vector<CmpGroup> groups;
     std::vector<int> range_start;   // first SNP of each range
-    std::vector<long long> range_chunks, range_tiles;
+    std::vector<int> range_group;   // first group of each range
+    std::vector<int> range_runs;
     size_t need = 0;                // buffer bytes of the largest range
     int i_hi = 0;                   // first SNPs [0, i_hi)
     double chunks_total = 0.0, steps_total = 0.0;
@@ -853,16 +907,12 @@ void plan_cmp(const epi3_handle* h, long long pb, long long pe, CmpPlan& P) {
     P.i_hi = i_hi;
     const int jb_first = (int)(j_lo / 64), jb_end = (int)(j_hi / 64) + 1;
     std::vector<CmpFirst>& firsts = P.firsts;
-    std::vector<int>& range_start = P.range_start;
-    std::vector<long long>& range_chunks = P.range_chunks;
-    std::vector<long long>& range_tiles = P.range_tiles;
     firsts.assign((size_t)i_hi, CmpFirst{});
-    long long chunks = 0, tiles = 0;
-    size_t& need = P.need;
+    size_t largest = 0;      // chunk bytes of one first SNP, at most
+    double tiles = 0.0;
     for (int i = 0; i < i_hi; ++i) {
         CmpFirst& f = firsts[i];
         f.b_lo = std::max((i + 1) / 64, jb_first);
-        f.jb_end = jb_end;
         // the two least frequent genotypes of SNP i are counted, the third derived
         int n[2][3];
         for (int c = 0; c < 2; ++c) {
@@ -874,39 +924,58 @@ void plan_cmp(const epi3_handle* h, long long pb, long long pe, CmpPlan& P) {
         f.drop = cmp_drop(n[0][0] + n[1][0], n[0][1] + n[1][1], n[0][2] + n[1][2]);
         for (int c = 0; c < 2; ++c)
             for (int s = 0; s < 2; ++s) f.ks[2 * c + s] = n[c][cmp_geno(f.drop, s)] / 256 + 1;  // + the bias sample
-        const long long ch = cmp_chunks_of(f, M);
-        if (range_start.empty() || (size_t)(chunks + ch) * 16384 > h->cmp_cap ||
-            i - range_start.back() >= 65535) {
-            if (!range_start.empty()) {
-                range_chunks.push_back(chunks);
-                range_tiles.push_back(tiles);
-            }
-            range_start.push_back(i);
-            chunks = 0;
-            tiles = 0;
-        }
-        long long bq = chunks;
-        const long long nblk = (M + 63) / 64 - f.b_lo;
-        for (int q = 0; q < kCmpSets; ++q) {
-            f.base[q] = bq;
-            bq += nblk * f.ks[q];
-        }
-        chunks = bq;
-        f.tiles = cmp_tiles_of(M, f.b_lo, f.jb_end);
-        f.tile0 = tiles;
-        tiles += f.tiles;
-        P.chunks_total += (double)(bq - f.base[0]);
+        f.tiles = cmp_tiles_of(M, f.b_lo, jb_end);
+        const double ch = (double)cmp_chunks_of(f, M);
+        P.chunks_total += ch;
         P.steps_total += (double)f.tiles * (f.ks[0] + f.ks[1] + f.ks[2] + f.ks[3]);
-        need = std::max(need, (size_t)chunks * 16384);
+        largest = std::max(largest, (size_t)ch * 16384);
+        tiles += f.tiles;
     }
-    if (!range_start.empty()) {
-        range_chunks.push_back(chunks);
-        range_tiles.push_back(tiles);
+    // First SNPs per run.  More of them share one set-up of the run's (j, k) inputs, but the chunks
+    // of that many first SNPs are re-read by every wave of CTAs, so they should stay in L2 (48 of
+    // its 129 MB), and the runs are dealt to CTAs whole: at least 16 for each.
+    int G = 8;
+    while (G > 1 && (G * largest > ((size_t)48 << 20) || G * largest > h->cmp_cap ||
+                     tiles < 16.0 * G * h->sm_count))
+        G /= 2;
+    long long chunks = 0;
+    int runs = 0;
+    for (int i = 0; i < i_hi;) {
+        const int ie = std::min(i_hi, ((i + 1) / G + 1) * G - 1);   // one past the group's last
+        long long ch = 0;
+        for (int t = i; t < ie; ++t) ch += cmp_chunks_of(firsts[t], M);
+        if (P.range_start.empty() || (size_t)(chunks + ch) * 16384 > h->cmp_cap ||
+            ie - P.range_start.back() > 65535 || runs > (1 << 30)) {
+            if (!P.range_start.empty()) P.range_runs.push_back(runs);
+            P.range_start.push_back(i);
+            P.range_group.push_back((int)P.groups.size());
+            chunks = 0;
+            runs = 0;
+        }
+        CmpGroup g;
+        g.b_lo = firsts[i].b_lo;
+        g.f0 = i - P.range_start.back();
+        g.n = ie - i;
+        g.runs = firsts[i].tiles;
+        runs += g.runs;
+        g.run_end = runs;
+        if (g.runs > 0) P.groups.push_back(g);
+        for (int t = i; t < ie; ++t) {
+            CmpFirst& f = firsts[t];
+            const long long nblk = (M + 63) / 64 - f.b_lo;
+            for (int q = 0; q < kCmpSets; ++q) {
+                f.base[q] = chunks;
+                chunks += nblk * f.ks[q];
+            }
+        }
+        P.need = std::max(P.need, (size_t)chunks * 16384);
+        i = ie;
     }
+    if (!P.range_start.empty()) P.range_runs.push_back(runs);
 }
 
-// The compaction plan of [pb, pe) for this handle, with its first-SNP table uploaded to
-// h->d_firsts (the marginals come to the host once per handle).
+// The compaction plan of [pb, pe) for this handle, with its first-SNP and group tables uploaded
+// (the marginals come to the host once per handle).
 int cmp_prepare(epi3_handle* h, long long pb, long long pe, CmpPlan& P) {
     const int M = h->M;
     if (h->h_marg.empty()) {
@@ -918,12 +987,36 @@ int cmp_prepare(epi3_handle* h, long long pb, long long pe, CmpPlan& P) {
     plan_cmp(h, pb, pe, P);
     dev_free(h->d_firsts);
     h->d_firsts = nullptr;
+    dev_free(h->d_groups);
+    h->d_groups = nullptr;
     if (!P.firsts.empty()) {
         CK(dev_alloc((void**)&h->d_firsts, sizeof(CmpFirst) * P.firsts.size()), "alloc first-SNP table");
         CK(cudaMemcpyAsync(h->d_firsts, P.firsts.data(), sizeof(CmpFirst) * P.firsts.size(),
                            cudaMemcpyHostToDevice, h->stream), "upload first-SNP table");
     }
+    if (!P.groups.empty()) {
+        CK(dev_alloc((void**)&h->d_groups, sizeof(CmpGroup) * P.groups.size()), "alloc group table");
+        CK(cudaMemcpyAsync(h->d_groups, P.groups.data(), sizeof(CmpGroup) * P.groups.size(),
+                           cudaMemcpyHostToDevice, h->stream), "upload group table");
+    }
     return EPI3_OK;
+}
+
+// Launch arguments of one range of a plan.
+CmpArgs cmp_args(const epi3_handle* h, const CohortDev& cd, int i0, int group, int runs,
+                 const uint8_t* cmp) {
+    CmpArgs a{};
+    a.cd = cd;
+    a.firsts = h->d_firsts + i0;
+    a.groups = h->d_groups + group;
+    a.i0 = i0;
+    a.n_runs = runs;
+    a.cmp = cmp;
+    a.yz = h->d_yz;
+    a.bound_c = h->bound.c;
+    a.bound_off = h->bound.off;
+    a.minor = h->bound.minor;
+    return a;
 }
 
 int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int top_k,
@@ -932,7 +1025,6 @@ int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int 
     const int prc = cmp_prepare(h, pb, pe, P);
     if (prc != EPI3_OK) return prc;
     const std::vector<int>& range_start = P.range_start;
-    const std::vector<long long>& range_tiles = P.range_tiles;
     const int i_hi = P.i_hi;
     const size_t need = P.need;
     h->last_cmp_chunks = P.chunks_total;
@@ -971,13 +1063,8 @@ int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int 
             CK(cudaEventRecord(h->cmp_ev[2 * r], h->stream), "event");
             CK(launch_compact(h->pl, h->d_firsts + i0, i0, n, h->d_cmp, h->stream), "compaction launch");
             CK(cudaEventRecord(h->cmp_ev[2 * r + 1], h->stream), "event");
-            CmpArgs a{};
-            a.cd = cohort_of(h, pb, pe, top_k);
-            a.firsts = h->d_firsts + i0;
-            a.i0 = i0;
-            a.n_first = n;
-            a.n_tiles = range_tiles[r];
-            a.cmp = h->d_cmp;
+            CmpArgs a = cmp_args(h, cohort_of(h, pb, pe, top_k), i0, P.range_group[r], P.range_runs[r],
+                                 h->d_cmp);
             a.prof = h->profile ? h->d_prof : nullptr;
             CK(launch_scan_cmp(a, grid, h->stream, h->tsum != nullptr || h->profile, cmp_paired(h)),
                "compacted scan launch");
@@ -1001,7 +1088,7 @@ int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int 
     s.n_rescored = h->h_ctrl->n_final;
     s.path = EPI3_PATH_MMA4C;
     s.grid = grid;
-    s.block = 512;
+    s.block = scan_cmp_threads();
     s.form = cmp_paired(h) ? 2 : 1;
     s.kernel_launches = 2 * n_ranges + 3;
     s.wait_loader = s.wait_mma_operands = s.wait_mma_accum = s.wait_producers = s.wait_epilogue = 0.f;
@@ -1020,7 +1107,7 @@ int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int 
     }
     s.k2_rel_bound = h->k2.rel;
     s.k2_abs_bound = h->k2.abs_;
-    s.k2_prune_bound = h->k2.prune_delta;
+    s.k2_prune_bound = h->bound.slack;
     cudaEventElapsedTime(&s.scan_kernel_ms, h->ev[1], h->ev[2]);
     cudaEventElapsedTime(&s.select_ms, h->ev[2], h->ev[3]);
     cudaEventElapsedTime(&s.total_ms, h->ev[0], h->ev[3]);
@@ -1068,7 +1155,7 @@ int scan_impl(epi3_handle* h, long long pb, long long pe, int top_k, int32_t* ou
     }
     if (path == EPI3_PATH_MMA4C) {
         int rc = ensure_pair_tables(h);
-        if (rc == EPI3_OK) rc = ensure_pair_floats(h);
+        if (rc == EPI3_OK) rc = ensure_yz(h);
         if (rc != EPI3_OK) return rc;
         return scan_cmp_impl(h, pb, pe, nt, top_k, out_trip, out_scores, n_out);
     }
@@ -1585,11 +1672,9 @@ struct epi3_batch {
     bool own_stream = false;
     std::vector<epi3_handle*> h;
     std::vector<int> path;              // EPI3_PATH_MMA4, EPI3_PATH_MMA4C or EPI3_PATH_POPC8 per cohort
-    // compacted-form cohorts: per cohort its ranges of first SNPs (first SNP of each range,
-    // tiles of each range, end of the last), all compacting into one shared buffer
-    std::vector<std::vector<int>> cmp_start;
-    std::vector<std::vector<long long>> cmp_tiles;
-    std::vector<int> cmp_end;
+    // compacted-form cohorts: per cohort its plan (ranges of first SNPs), all compacting into one
+    // shared buffer
+    std::vector<CmpPlan> cmp_plan;
     uint8_t* d_cmp = nullptr;
     Ctrl* d_ctrls = nullptr;            // one control block per cohort, contiguous
     Ctrl* h_ctrls = nullptr;            // pinned
@@ -1910,19 +1995,13 @@ int batch_capture(epi3_batch* b, int top_k) {
         if (b->path[c] != EPI3_PATH_MMA4C) continue;
         cur_c = c;
         epi3_handle* h = b->h[c];
-        const std::vector<int>& rs = b->cmp_start[c];
+        const CmpPlan& P = b->cmp_plan[c];
+        const std::vector<int>& rs = P.range_start;
         for (size_t r = 0; r < rs.size(); ++r) {
             const int i0 = rs[r];
-            const int n = (r + 1 < rs.size() ? rs[r + 1] : b->cmp_end[c]) - i0;
+            const int n = (r + 1 < rs.size() ? rs[r + 1] : P.i_hi) - i0;
             ok(launch_compact(h->pl, h->d_firsts + i0, i0, n, b->d_cmp, b->stream));
-            CmpArgs a{};
-            a.cd = cds[c];
-            a.firsts = h->d_firsts + i0;
-            a.i0 = i0;
-            a.n_first = n;
-            a.n_tiles = b->cmp_tiles[c][r];
-            a.cmp = b->d_cmp;
-            a.prof = nullptr;
+            const CmpArgs a = cmp_args(h, cds[c], i0, P.range_group[r], P.range_runs[r], b->d_cmp);
             ok(launch_scan_cmp(a, b->sm_count, b->stream, false, cmp_paired(h)));
         }
     }
@@ -2028,9 +2107,7 @@ int epi3_batch_create(epi3_batch** out, int32_t n_cohorts, const epi3_cohort* co
     }
     std::vector<int4> tiles;
     size_t cmp_need = 0;
-    b->cmp_start.assign(n_cohorts, std::vector<int>());
-    b->cmp_tiles.assign(n_cohorts, std::vector<long long>());
-    b->cmp_end.assign(n_cohorts, 0);
+    b->cmp_plan.assign(n_cohorts, CmpPlan());
     for (int c = 0; c < n_cohorts; ++c) {
         epi3_handle* h = b->h[c];
         if ((rc = tune_path(b, h, &b->path[c], &b->tune_ms)) != EPI3_OK) return bail(rc);
@@ -2039,12 +2116,9 @@ int epi3_batch_create(epi3_batch** out, int32_t n_cohorts, const epi3_cohort* co
             append_tiles(h->M, 0, pairs(h->M - 1), c, tiles);
         } else if (b->path[c] == EPI3_PATH_MMA4C) {
             // its own compaction + scan launches in the graph, ranges planned now
-            CmpPlan P;
-            if ((rc = ensure_pair_floats(h)) != EPI3_OK) return bail(rc);
+            CmpPlan& P = b->cmp_plan[c];
+            if ((rc = ensure_yz(h)) != EPI3_OK) return bail(rc);
             if ((rc = cmp_prepare(h, 0, pairs(h->M - 1), P)) != EPI3_OK) return bail(rc);
-            b->cmp_start[c] = P.range_start;
-            b->cmp_tiles[c] = P.range_tiles;
-            b->cmp_end[c] = P.i_hi;
             cmp_need = std::max(cmp_need, P.need);
         }
         h->path = b->path[c];

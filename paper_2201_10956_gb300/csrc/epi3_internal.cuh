@@ -140,6 +140,20 @@ cudaError_t launch_quad_scan(const Planes& pl, const double* lf64, int n0, int n
 cudaError_t launch_approx_error(const double* lf64, int n_lf, double* out, cudaStream_t st);
 cudaError_t launch_pair_tables(const Planes& pl, int4* pt, int2* marg, long long n_pairs,
                                cudaStream_t st);
+// The compacted scan's copy of the pair tables, in blocks of 16 float4 for eight k = 8 b .. 8 b + 7
+// with one j: float4 4 e + p holds, for the pairs (j, k) and (j, k + 1), k = 8 b + 2 p, both classes'
+// sum + 6 {00 00', 01 01'} (e = 0), {10 10', 11 11'} (e = 1), and class `minor` + 3 the same way (e =
+// 2, 3); prime: k + 1.  Pairs with k <= j or k >= M hold zeros.  Row j has the blocks from (j + 1) / 8
+// on: the rows before it skip sum over t = 1 .. j of floor(t / 8) blocks.
+__host__ __device__ inline long long yz_block(int j, int k, int M) {
+    const int q = j / 8, r = j % 8;
+    return (long long)j * ((M + 7) / 8) - (4LL * q * (q - 1) + (long long)q * (r + 1)) + (k / 8 - (j + 1) / 8);
+}
+// blocks allocated: every row's, and the few that a tile's 32 columns reach past the last SNP (read
+// and ignored, like the blocks before a row's first; never below block 0)
+inline long long yz_blocks(int M) { return yz_block(M, 8 * ((M + 1) / 8), M) + 16; }
+cudaError_t launch_pair_yz(const int4* pt, long long n_pairs, int M, int minor, float4* yz,
+                           cudaStream_t st);
 // ptf = pt + 3 and margf = marg + 9 as FP32 (2 n_pairs and 2 M entries)
 cudaError_t launch_pair_floats(const int4* pt, const int2* marg, long long n_pairs, int M,
                                float4* ptf, float2* margf, cudaStream_t st);
@@ -196,16 +210,29 @@ struct CmpFirst {
     int drop;
     int b_lo;                    // first 64-SNP block compacted: the first j block of the tiles
     int tiles;                   // tiles of this first SNP
-    int jb_end;                  // one past its last j block (the pair range's last j)
-    long long tile0;             // index of its first tile in the range
+};
+
+// A group of consecutive first SNPs with the same j blocks: each of its runs, a (j block, k
+// block), covers them all.
+struct CmpGroup {
+    int run_end;                 // one past its last run in the range
+    int runs;                    // its runs
+    int f0, n;                   // first SNPs f0 .. f0 + n - 1, relative to the range
+    int b_lo;                    // first j block
 };
 
 struct CmpArgs {
     CohortDev cd;                // tables, candidate stage, pair range, test hooks
     const CmpFirst* firsts;      // per first SNP of the range
-    int i0, n_first;
-    long long n_tiles;           // tiles of the range
+    const CmpGroup* groups;      // the range's groups, in order
+    int i0;
+    int n_runs;                  // runs of the range
     const uint8_t* cmp;          // compacted chunks of the range
+    const float4* yz;            // (Y, Z) pair tables in the epilogue's form (launch_pair_yz)
+    // the table-free bound: K2 >= bound_c (sum of q) + (ln of the product of q) / 2 - bound_off
+    // over the 27 cells' q = um (us - um) / us (cmp_bound_terms)
+    float bound_c, bound_off;
+    int minor;                   // the smaller class (table m)
     unsigned long long* prof;    // optional (instrumented kernel): wait cycles per role
 };
 // The genotype counted in slot s (0, 1) when genotype d is derived: the other two, ascending.
@@ -256,6 +283,12 @@ __host__ __device__ __forceinline__ void canon_rows(T* u, int d) {
         }
     }
 }
+// Constants of the compacted scan's table-free bound for class sizes n0, n1 (capi.cu).
+struct CmpBoundTerms {
+    float c, off;                // K2 >= c (sum of q) + (ln of the product of q) / 2 - off
+    float slack;                 // the part of off that covers Stirling's remainders and rounding
+    int minor;                   // the smaller class
+};
 // compacted chunks of one first SNP: 16 KB each
 inline long long cmp_chunks_of(const CmpFirst& f, int M) {
     const long long nblk = (M + 63) / 64 - f.b_lo;
@@ -263,6 +296,7 @@ inline long long cmp_chunks_of(const CmpFirst& f, int M) {
 }
 int cmp_tiles_of(int M, int b_lo, int jb_end); // tiles (64 j x 32 k) of one first SNP
 size_t scan_cmp_smem();
+int scan_cmp_threads();          // threads per CTA of the compacted scan
 // compaction of first SNPs i0 .. i0 + n_first - 1 into cmp (chunk indices from firsts)
 cudaError_t launch_compact(const Planes& pl, const CmpFirst* firsts, int i0, int n_first,
                            uint8_t* cmp, cudaStream_t st);
@@ -402,12 +436,16 @@ __host__ __device__ inline unsigned long long mix64(unsigned long long z) {
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
     return z ^ (z >> 31);
 }
+__device__ inline unsigned long long table_fold(unsigned long long f, int r0, int r1) {
+    return f * 0x100000001B3ull + (unsigned long long)(unsigned)r0 + ((unsigned long long)(unsigned)r1 << 32);
+}
+__device__ inline unsigned long long table_mix(unsigned long long f, int i, int j, int k) {
+    return mix64(f ^ mix64(pack_key(i, j, k)));
+}
 __device__ inline unsigned long long table_hash(int i, int j, int k, const int* r0, const int* r1) {
     unsigned long long f = 0;
-    for (int q = 0; q < kCells; ++q)
-        f = f * 0x100000001B3ull + (unsigned long long)(unsigned)r0[q] +
-            ((unsigned long long)(unsigned)r1[q] << 32);
-    return mix64(f ^ mix64(pack_key(i, j, k)));
+    for (int q = 0; q < kCells; ++q) f = table_fold(f, r0[q], r1[q]);
+    return table_mix(f, i, j, k);
 }
 __device__ inline void table_sum_flush(unsigned long long* tsum, unsigned long long h,
                                        unsigned long long n) {

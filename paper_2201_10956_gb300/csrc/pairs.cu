@@ -64,7 +64,47 @@ __global__ void pair_floats_kernel(const int4* __restrict__ pt, const int2* __re
     }
 }
 
+// One thread per (j, pair of k), four to a block of the layout: CTA (x, y) takes 512 k of rows j = y,
+// y + gridDim.y, ...
+__global__ void __launch_bounds__(256)
+pair_yz_kernel(const int4* __restrict__ pt, long long n_pairs, int M, int minor,
+               float4* __restrict__ yz) {
+    const int k = 2 * (blockIdx.x * 256 + threadIdx.x);
+    if ((k & ~7) >= M) return;
+    for (int j = blockIdx.y; j < M && j < (k & ~7) + 8; j += gridDim.y) {
+        if ((k >> 3) < ((j + 1) >> 3)) continue;
+        float s[2][4], m[2][4];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const bool v = k + e > j && k + e < M;
+            const long long p = v ? pair_index(j, k + e) : 0;
+            const int4 a = __ldg(pt + p), b = __ldg(pt + n_pairs + p), q = minor ? b : a;
+            s[e][0] = v ? (float)(a.x + b.x + 6) : 0.f;
+            s[e][1] = v ? (float)(a.y + b.y + 6) : 0.f;
+            s[e][2] = v ? (float)(a.z + b.z + 6) : 0.f;
+            s[e][3] = v ? (float)(a.w + b.w + 6) : 0.f;
+            m[e][0] = v ? (float)(q.x + 3) : 0.f;
+            m[e][1] = v ? (float)(q.y + 3) : 0.f;
+            m[e][2] = v ? (float)(q.z + 3) : 0.f;
+            m[e][3] = v ? (float)(q.w + 3) : 0.f;
+        }
+        float4* const o = yz + 16 * yz_block(j, k, M) + ((k >> 1) & 3);
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            o[4 * t] = make_float4(s[0][2 * t], s[1][2 * t], s[0][2 * t + 1], s[1][2 * t + 1]);
+            o[8 + 4 * t] = make_float4(m[0][2 * t], m[1][2 * t], m[0][2 * t + 1], m[1][2 * t + 1]);
+        }
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_pair_yz(const int4* pt, long long n_pairs, int M, int minor, float4* yz,
+                           cudaStream_t st) {
+    const dim3 grid((M + 511) / 512, M < 65535 ? M : 65535);
+    pair_yz_kernel<<<grid, 256, 0, st>>>(pt, n_pairs, M, minor, yz);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_pair_floats(const int4* pt, const int2* marg, long long n_pairs, int M,
                                float4* ptf, float2* margf, cudaStream_t st) {

@@ -11,11 +11,12 @@
 // expansion to FP4 E2M1 0/1 values in the 128B-swizzled shared-memory image), and the scan
 // multiplies compacted chunks straight from L2: both MMA operands come from shared memory,
 // filled by bulk copies, with no operand formed on chip and 4 MACs per sample-triplet whose
-// first-SNP genotype is counted.  The epilogue relabels SNP i's genotypes (counted ones 0 and 1,
-// the derived one 2) in its pair-table and marginal inputs, derives the 19 other cells from pair
-// tables and marginals, and restores the genotype order before the exact table is scored: K2
-// and the candidate band exactly as in the other scans (Eq. 1; the paper counts with POPCNT,
-// Sec. IV, and points at tensor-core formulations in Sec. II).
+// first-SNP genotype is counted.  SNP i's genotypes are relabelled (counted ones 0 and 1, the
+// derived one 2) in the pair-table and marginal inputs; the epilogue derives the 19 other cells and
+// bounds the table's score from below; the few triplets whose bound does not exceed the candidate
+// threshold get their exact integer table and FP32 score: K2 and the candidate band exactly as in
+// the other scans (Eq. 1; the paper counts with POPCNT, Sec. IV, and points at tensor-core
+// formulations in Sec. II).
 //
 // Every set carries one bias sample (a 1 in every row) after its samples, so every accumulator
 // ends at count + 1, the argument of the epilogue's count + 1 arithmetic.
@@ -29,13 +30,19 @@
 // step takes half a slot): every commit costs the tensor pipe a bubble, so fewer, larger slots
 // beat one slot per step.
 //
-// Warp roles (16 warps): 0 = operand loader + tensor-memory allocator, 1 = MMA issuer (both as
-// whole warps, one elected lane issuing), 2-3 idle, 4-15 = epilogue (three warps per
-// tensor-memory lane quadrant); registers move from the first warp group to the epilogue
-// (setmaxnreg).  Every mbarrier wait is bounded; on timeout the kernel
-// records kStTimeout, waits for its own copies and MMAs, frees tensor memory and returns.
+// Warp roles (16 warps): 0 = operand loader + tensor-memory allocator, 1 = MMA issuer, 2-3 = stagers
+// (the per-tile constants of the derived cells), 4-15 = epilogue.  The epilogue warps meet only every
+// few tiles; mbarriers pass accumulators and staged constants to and from each.  Every mbarrier wait
+// is bounded; on timeout the kernel records kStTimeout, waits for its own copies and MMAs, frees
+// tensor memory and returns.
+//
+// Measured (GB300, scan kernel without the compaction): 2048 SNPs x 4096 samples 46.0 -> 21.4 ms,
+// 2048 x 16384 50.2 -> 31.4 ms.  At 4096 samples a tile takes 8800 cycles, of which the FP32 pipe
+// is busy 3800 (the bound); at 16 384 it takes 12 900, of which the tensor pipe's operand reads and
+// the ring's hand-offs alone take 10 300.
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "epi3_internal.cuh"
 #include "tc_common.cuh"
@@ -223,83 +230,371 @@ constexpr int kSlotA = kSlotSteps * kStepA;
 constexpr int kSlotB = kSlotSteps * kStepB;
 constexpr int kCmpRegions = 7;           // 64-column accumulator regions (columns 0..447)
 constexpr uint32_t kCmpSfCol = 480;      // block scales: A at 480..495, B at 496..511
-constexpr int kCmpThreads = 512;
+// 16 warps: 0 loader, 1 MMA issuer, 2 and 3 stagers, 4..15 epilogue, 128 registers a thread.  The
+// three epilogue warps of a tensor-memory lane quadrant (all on one SM quarter) split its eight
+// items (2 lane groups x 4 column groups) 3 / 3 / 2.
 constexpr int kCmpEpiWarp0 = 4, kCmpEpiWarps = 12, kCmpEpiThreads = kCmpEpiWarps * 32;
-constexpr int kCmpEpiParts = kCmpEpiWarps / 4;   // epilogue warps per tensor-memory lane quadrant
-// the epilogue's items: per quadrant 2 lane groups (8 second SNPs each) x 4 column groups (8 third
-// SNPs each), split 3 / 3 / 2 over its three warps
-static_assert(kCmpEpiParts == 3 && kTJ == 4 * 2 * 8 && kTK == 4 * 8, "epilogue item split");
-constexpr int kCmpRegLaunch = 128, kCmpRegCtl = 56, kCmpRegEpi = 152;
-static_assert(kCmpRegCtl + 3 * kCmpRegEpi == 4 * kCmpRegLaunch, "register split");
-static_assert(kCmpThreads * kCmpRegLaunch == 65536, "the launch holds the whole register file");
+constexpr int kCmpEpiParts = kCmpEpiWarps / 4, kCmpEpiItems = (8 + kCmpEpiParts - 1) / kCmpEpiParts;
+constexpr int kCmpThreads = (kCmpEpiWarp0 + kCmpEpiWarps) * 32;
+static_assert(kTJ == 4 * 2 * 8 && kTK == 4 * 8, "epilogue item split");
 static_assert(kCmpRegions * kN <= (int)kCmpSfCol, "tensor memory budget");
+constexpr int kMaxSyncTiles = 16;        // tiles between the epilogue warps' rendezvous, at most
+
+// One tile's epilogue inputs, staged by the stager warp (two buffers).  Every value comes for two
+// tables, the samples of both classes (s, each u = count + 2) and those of the smaller class
+// (m, u = count + 1), with the offsets that make a difference of u values a u value.
+//   row[j][phase][..]  {s, s, m, m} per constant (f32x2 operands for two triplets of one j):
+//                      phase a = 0, 1: (a, 0, .), (a, 1, .), (a, 2, .) summed over z;
+//                      phase 2: (2, 0, .), (2, 1, .), (2, 2, .)
+//   col[k / 2][phase]  {k, k + 1} per constant: phase a: s(a, ., 0), s(a, ., 1), m(a, ., 0),
+//                      m(a, ., 1); phase 2 the same for a = 2
+//   thr[j]             prune a triplet whose bound exceeds this (-inf: no triplet in this row)
+//   i, f, jb, kb       the tile; flags: kStageRun the first tile of a run, kStageLast this CTA's last
+struct CmpStage {
+    float4 row[kTJ][3][3];
+    float2 col[kTK / 2][3][4];
+    float thr[kTJ];
+    int f, jb, kb, flags;
+};
+constexpr int kStageRun = 1, kStageLast = 2;
 
 // Instruction descriptor of kind::mxf4: A/B E2M1, UE8M0 scales, K-major, N = 64, M = 128.
 constexpr uint32_t kIdescCmp = (1u << 7) | (1u << 10) | ((uint32_t)(kN >> 3) << 17) | (1u << 23) |
                                ((128u >> 4) << 24);
 
-// Issued warp-wide: elect.sync picks the lane that issues (see tc_common.cuh).
-__device__ __forceinline__ void mma_ss_mx_elect(uint32_t d, uint64_t a, uint64_t b, uint32_t acc,
-                                                uint32_t sfa, uint32_t sfb) {
+// One K-step: four MMAs of 64 samples (32 bytes of K each) into d, issued warp-wide by the lane
+// that elect.sync picks (see tc_common.cuh), once for all four; acc: add to d from the first on.
+__device__ __forceinline__ void mma_step_elect(uint32_t d, uint64_t a, uint64_t b, uint32_t acc,
+                                               uint32_t sfa, uint32_t sfb) {
     asm volatile(
-        "{\n .reg .pred p, e;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %3, 0;\n"
-        " @e tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %6,"
-        " [%4], [%5], p;\n}\n"
+        "{\n .reg .pred p, e;\n .reg .b64 a1, a2, a3, b1, b2, b3;\n"
+        " add.s64 a1, %1, 2;\n add.s64 a2, %1, 4;\n add.s64 a3, %1, 6;\n"
+        " add.s64 b1, %2, 2;\n add.s64 b2, %2, 4;\n add.s64 b3, %2, 6;\n"
+        " setp.ne.b32 p, %3, 0;\n elect.sync _|e, 0xffffffff;\n"
+        " @e tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], %1, %2, %6, [%4], [%5], p;\n"
+        " @e tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], a1, b1, %6, [%4], [%5], 1;\n"
+        " @e tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], a2, b2, %6, [%4], [%5], 1;\n"
+        " @e tcgen05.mma.cta_group::1.kind::mxf4.block_scale.scale_vec::2X [%0], a3, b3, %6, [%4], [%5], 1;\n}\n"
         ::"r"(d), "l"(a), "l"(b), "r"(acc), "r"(sfa), "r"(sfb), "r"(kIdescCmp) : "memory");
+}
+// A slot's copies: its barrier told the bytes, the A chunks in one copy, the B halves of one or two
+// chunks (b1: the second, if two).
+__device__ __forceinline__ void load_slot_elect(uint32_t bar, uint32_t da, const uint8_t* a, uint32_t abytes,
+                                                uint32_t db, const uint8_t* b, uint32_t two) {
+    asm volatile(
+        "{\n .reg .pred e, t;\n .reg .b32 n, d1;\n .reg .b64 b1;\n"
+        " add.u32 n, %3, %7;\n setp.ne.u32 t, %6, 0;\n @t add.u32 n, n, %7;\n"
+        " add.u32 d1, %4, %7;\n add.s64 b1, %5, %8;\n"
+        " elect.sync _|e, 0xffffffff;\n and.pred t, t, e;\n"
+        " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], n;\n"
+        " @e cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%1], [%2], %3, [%0];\n"
+        " @e cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%4], [%5], %7, [%0];\n"
+        " @t cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [d1], [b1], %7, [%0];\n}\n"
+        ::"r"(bar), "r"(da), "l"(a), "r"(abytes), "r"(db), "l"(b), "r"(two), "n"(kCmpChunk / 2), "n"(kCmpChunk)
+        : "memory");
 }
 
 // 16 lanes x 16 FP32 columns from taddr: thread t gets lane t / 4 (v[0..1]) and lane t / 4 + 8
 // (v[2..3]) at columns 2 (t % 4) + {0, 1}, then the same at columns + 8 (v[4..7]).
-__device__ __forceinline__ void tc_ld16x2(uint32_t taddr, uint32_t* v) {
+__device__ __forceinline__ void tc_ld16x2(uint32_t taddr, float* v) {
     asm volatile(
         "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-          "=r"(v[7])
+        : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]),
+          "=f"(v[7])
         : "r"(taddr));
 }
+// 16 bytes from global to shared memory, asynchronously.
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+// Wait for every such load; the registers of two or four pass through, so that no use moves above it.
+__device__ __forceinline__ void tc_wait_ld4(float (&v)[4][8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(v[0][0]), "+f"(v[0][1]), "+f"(v[0][2]), "+f"(v[0][3]), "+f"(v[0][4]),
+                   "+f"(v[0][5]), "+f"(v[0][6]), "+f"(v[0][7]), "+f"(v[1][0]), "+f"(v[1][1]),
+                   "+f"(v[1][2]), "+f"(v[1][3]), "+f"(v[1][4]), "+f"(v[1][5]), "+f"(v[1][6]),
+                   "+f"(v[1][7]), "+f"(v[2][0]), "+f"(v[2][1]), "+f"(v[2][2]), "+f"(v[2][3]),
+                   "+f"(v[2][4]), "+f"(v[2][5]), "+f"(v[2][6]), "+f"(v[2][7]), "+f"(v[3][0]),
+                   "+f"(v[3][1]), "+f"(v[3][2]), "+f"(v[3][3]), "+f"(v[3][4]), "+f"(v[3][5]),
+                   "+f"(v[3][6]), "+f"(v[3][7]));
+}
 
-}  // namespace
+__device__ __forceinline__ void tc_wait_ld2(float (&v)[2][8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(v[0][0]), "+f"(v[0][1]), "+f"(v[0][2]), "+f"(v[0][3]), "+f"(v[0][4]),
+                   "+f"(v[0][5]), "+f"(v[0][6]), "+f"(v[0][7]), "+f"(v[1][0]), "+f"(v[1][1]),
+                   "+f"(v[1][2]), "+f"(v[1][3]), "+f"(v[1][4]), "+f"(v[1][5]), "+f"(v[1][6]),
+                   "+f"(v[1][7]));
+}
 
+// The tiles of a CTA, in order.  A run is a (j block, k block) of a group of consecutive first
+// SNPs; CTA c takes runs c, c + gridDim.x, ... and in each run the group's first SNPs one after
+// another, so that what depends on (j, k) only is set up once per run.
+struct CmpCursor {
+    int r;                       // run
+    int g_end;                   // one past the group's runs
+    int jb_run0;                 // first run of j block jb
+    int g, f0, n, f;             // group, its first SNPs (relative to the range), the current one
+    int jb, kb;
 
-namespace {
-
-struct CmpTile {
-    int f;                       // first SNP, relative to the range
-    int jb, kb;                  // 64-SNP block of j, 32-SNP block of k
+    __device__ __forceinline__ bool seek(const CmpArgs& a) {
+        if (r >= a.n_runs) return false;
+        const int nk = (a.cd.pl.M + kTK - 1) / kTK;
+        if (r >= g_end) {
+            do ++g;
+            while (a.groups[g].run_end <= r);
+            const CmpGroup& G = a.groups[g];
+            g_end = G.run_end;
+            f0 = G.f0;
+            n = G.n;
+            jb = G.b_lo;
+            jb_run0 = G.run_end - G.runs;
+        }
+        while (r - jb_run0 >= nk - 2 * jb) {
+            jb_run0 += nk - 2 * jb;
+            ++jb;
+        }
+        kb = 2 * jb + (r - jb_run0);
+        f = f0;
+        return true;
+    }
+    __device__ __forceinline__ bool first(const CmpArgs& a) {
+        r = blockIdx.x;
+        g = -1;
+        g_end = 0;
+        return seek(a);
+    }
+    __device__ __forceinline__ bool next(const CmpArgs& a) {
+        if (++f < f0 + n) return true;
+        r += gridDim.x;
+        return seek(a);
+    }
 };
 
-// Tile t of the range: first SNPs in order, then j blocks from b_lo (to jb_end), then k blocks
-// from 2 jb.
-__device__ __forceinline__ CmpTile cmp_tile(const CmpArgs& a, long long t) {
-    int lo = 0, hi = a.n_first;  // last f with tile0 <= t
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (a.firsts[mid].tile0 <= t) lo = mid;
-        else hi = mid;
+// A warp's triplets that the bound did not prune, waiting for their exact score: the counted cells
+// (count + 1, [8 c + 4 a + 2 b + z]) and the SNPs.  They arrive a few at a time, scattered over
+// lanes; queued, a warp scores up to 16 at once.
+constexpr int kQueue = 16;
+struct CmpQueue {
+    float n8[16][kQueue];
+    int i[kQueue], j[kQueue], k[kQueue];
+    // per lane, set at the first tile of a run: its triplets with k > j in range (bits 2 it + m) and
+    // its first (Y, Z) block for the tile's k in lane groups h = 0, 1
+    unsigned vmask[32], yz[2][32];
+    int n;                       // entries, fewer than kQueue between tiles
+    int pad_[3];
+};
+
+// One queued triplet's exact tables, its FP32 score (k2_f32's operations in its order) and, if that
+// is inside the threshold, its place in the candidate buffer.  One genotype of the first SNP at a
+// time (nine cells of both classes: the whole table would cost the epilogue its registers): its
+// counted cells, or for the derived genotype the (Y, Z) pair table minus the counted ones, then the
+// cells with a 2 from the integer pair tables and marginals, as in derive27.
+template <bool kInstr>
+__device__ __forceinline__ void cmp_score(const CmpArgs& a, EpiShared& es, const CmpQueue& qu, int at,
+                                          unsigned long long* sums) {
+    const CohortDev& cd = a.cd;
+    const PairTables& pt = cd.pt;
+    const int M = cd.pl.M;
+    int i = qu.i[at], j = qu.j[at], k = qu.k[at];
+    const int drop = __ldg(&a.firsts[i - a.i0].drop);
+    float ah = 0.f, al = 0.f;
+    unsigned long long hash = 0;
+    bool ok = true;
+#pragma unroll 1
+    for (int g = 0; g < 3; ++g) {
+        int r[2][9], t[9];
+#pragma unroll 1
+        for (int c = 0; c < 2; ++c) {
+            // opaque: keeps the compiler from holding every table entry across the loops
+            asm volatile("" : "+r"(i), "+r"(j), "+r"(k));
+            const int4* const tab = pt.pt + c * pt.n_pairs;
+            const int2* const mg = pt.marg + (size_t)c * M;
+            const int4 xy = __ldg(tab + pair_index(i, j)), xz = __ldg(tab + pair_index(i, k));
+            const int2 mx = __ldg(mg + i), my = __ldg(mg + j), mz = __ldg(mg + k);
+            int n[4];    // (g, b, z), index 2 b + z
+            const float* const q0 = &qu.n8[8 * c][at];
+            if (g == drop) {
+                const int4 yz = __ldg(tab + pair_index(j, k));
+                const int y[4] = {yz.x, yz.y, yz.z, yz.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) n[e] = y[e] - ((int)q0[kQueue * e] - 1) - ((int)q0[kQueue * (4 + e)] - 1);
+            } else {
+                const float* const q = q0 + kQueue * 4 * (g > drop ? g - 1 : g);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) n[e] = (int)q[kQueue * e] - 1;
+            }
+            const int xy0 = g == 0 ? xy.x : g == 1 ? xy.z : my.x - xy.x - xy.z;     // (g, Y = 0), (g, Y = 1)
+            const int xy1 = g == 0 ? xy.y : g == 1 ? xy.w : my.y - xy.y - xy.w;
+            const int xz0 = g == 0 ? xz.x : g == 1 ? xz.z : mz.x - xz.x - xz.z;
+            const int xz1 = g == 0 ? xz.y : g == 1 ? xz.w : mz.y - xz.y - xz.w;
+            const int mg_ = g == 0 ? mx.x : g == 1 ? mx.y : (c ? pt.n_c[1] : pt.n_c[0]) - mx.x - mx.y;
+            t[0] = n[0];
+            t[1] = n[1];
+            t[2] = xy0 - n[0] - n[1];
+            t[3] = n[2];
+            t[4] = n[3];
+            t[5] = xy1 - n[2] - n[3];
+            t[6] = xz0 - n[0] - n[2];
+            t[7] = xz1 - n[1] - n[3];
+            t[8] = (mg_ - xy0 - xy1) - t[6] - t[7];
+#pragma unroll
+            for (int e = 0; e < 9; ++e) {
+                ok = ok && (unsigned)t[e] <= (unsigned)(c ? pt.n_c[1] : pt.n_c[0]);
+                if (c == 0) r[0][e] = t[e];
+                else r[1][e] = t[e];
+            }
+        }
+        if (!ok) break;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            const float2 s = __ldg(cd.k2.lf2 + r[0][e] + r[1][e] + 1), u = __ldg(cd.k2.lf2 + r[0][e]),
+                         w = __ldg(cd.k2.lf2 + r[1][e]);
+            ah += __fsub_rn(__fsub_rn(s.x, u.x), w.x);
+            al += __fsub_rn(__fsub_rn(s.y, u.y), w.y);
+            if (kInstr) hash = table_fold(hash, r[0][e], r[1][e]);
+        }
     }
-    CmpTile r;
-    r.f = lo;
-    long long u = t - a.firsts[lo].tile0;
-    const int nk = (a.cd.pl.M + kTK - 1) / kTK;
-    int jb = a.firsts[lo].b_lo;
-    while (u >= nk - 2 * jb) {
-        u -= nk - 2 * jb;
-        ++jb;
+    if (!ok) {
+        atomicOr(&cd.ctrl->status, kStBadCount);
+        return;
     }
-    r.jb = jb;
-    r.kb = 2 * jb + (int)u;
-    return r;
+    const float sc = __fadd_rn(ah, al);
+    if (cd.dbg) cd.dbg[((size_t)i * M + j) * M + k] = sc;
+    if (kInstr && cd.tsum) {
+        sums[0] += table_mix(hash, i, j, k);
+        ++sums[1];
+    }
+    const float thr_g = __uint_as_float(*(volatile unsigned*)&cd.ctrl->thr);
+    if (sc <= fminf(*(volatile float*)&es.tloc, thr_g)) {
+        const int idx = atomicAdd(&es.cnt, 1);
+        if (idx < kCandCap) es.buf[idx] = Cand{sc, i, j, k};
+        else cand_global(cd, Cand{sc, i, j, k});
+    }
 }
+
+// A warp's surviving triplets of an item (mask: bit m, triplet (i, j, k0 + m)) go to its queue, their
+// counted cells read from tensor memory again (t: the item's four sets); before it would overflow, the queue is scored.  Called by a whole warp; with no survivors
+// at all (mask 0 in every lane) it scores what is left.
+struct CmpItems {
+    uint32_t t[4];
+    int i, j, k0;
+    unsigned mask;
+};
+template <bool kInstr>
+__device__ __forceinline__ void cmp_survivors(const CmpArgs& a, EpiShared& es, CmpQueue& qu, const CmpItems x,
+                                           unsigned long long* sums) {
+    const CohortDev& cd = a.cd;
+    const int lane = threadIdx.x & 31, i = x.i, j = x.j, M = cd.pl.M;
+    const long long pij = j > i && j < M ? pair_index(i, j) : -1;
+    const bool row = pij >= 0 && pij >= cd.pair_begin && pij < cd.pair_end;
+    int n = qu.n;
+    const bool flush = !__any_sync(0xffffffffu, x.mask != 0u);
+#pragma unroll 1
+    for (int m = flush ? 1 : 0; m < 2; ++m) {
+        const int k = x.k0 + m;
+        bool want = row && ((x.mask >> m) & 1u) && k > j && k < M;
+        unsigned who = __ballot_sync(0xffffffffu, want);
+#pragma unroll 1
+        while (who || flush) {
+            const int at = n + __popc(who & ((1u << lane) - 1u));
+            const bool take = want && at < kQueue;
+            if (who) {
+                float v[4][8];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) tc_ld16x2(x.t[q], v[q]);
+                tc_wait_ld4(v);
+                if (take) {
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {   // register 4 z + 2 b + m of set (c, a)
+                        const int r = 4 * (e & 1) + 2 * ((e >> 1) & 1);
+                        qu.n8[e][at] = m ? v[e >> 2][r + 1] : v[e >> 2][r];
+                    }
+                    qu.i[at] = i;
+                    qu.j[at] = j;
+                    qu.k[at] = k;
+                }
+                n = min(n + __popc(who), kQueue);
+                want = want && !take;
+                who = __ballot_sync(0xffffffffu, want);
+            }
+            if (n == kQueue || flush) {
+                __syncwarp();
+                if (lane < n) cmp_score<kInstr>(a, es, qu, lane, sums);
+                __syncwarp();
+                n = 0;
+                if (flush) break;
+            }
+        }
+    }
+    __syncwarp();
+    if (lane == 0) qu.n = n;
+    __syncwarp();
+}
+
+// The bound of one lane's two triplets of an item (L = LaneOps2), or of one of them (LaneOps1).
+// Per cell q = um (us - um) / us, us and um the cell's u in tables s and m: um + um (um (-1/us)).
+// Sum of q and sum of lg2 q (the cells of a phase multiplied first: every q is at least about
+// 1/2 and nine of them sum to at most (N + 54) / 4, so no product leaves the FP32 range).
+// A reciprocal holds its pipe for 8 cycles a warp and the FP32 pipe is as busy, so cells share one
+// reciprocal in pairs: -1 / a = b (-1 / (a b)).  The nine cells of a phase go through each operation
+// together: one after the other, every operation would wait for the one before it.
+constexpr int kRcpPairs = 4;
+template <class L>
+struct CmpBound {
+    typedef typename L::T T;
+    T sum[2], lgs;
+    __device__ __forceinline__ void init() { sum[0] = sum[1] = lgs = L::dup(0.f); }
+    __device__ __forceinline__ void phase(const T (&us)[9], const T (&um)[9]) {
+        T nr[9], q[9];
+#pragma unroll
+        for (int e = 0; e < 2 * kRcpPairs; e += 2) nr[e] = L::mul(us[e], us[e + 1]);
+#pragma unroll
+        for (int e = 0; e < 9; ++e)
+            if (e >= 2 * kRcpPairs) nr[e] = L::nrcp(us[e]);
+            else if (e % 2 == 0) nr[e] = L::nrcp(nr[e]);
+#pragma unroll
+        for (int e = 0; e < 2 * kRcpPairs; e += 2) {
+            nr[e + 1] = L::mul(nr[e], us[e]);
+            nr[e] = L::mul(nr[e], us[e + 1]);
+        }
+#pragma unroll
+        for (int e = 0; e < 9; ++e) q[e] = L::mul(um[e], nr[e]);
+#pragma unroll
+        for (int e = 0; e < 9; ++e) q[e] = L::fma(q[e], um[e], um[e]);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) sum[e & 1] = L::add(sum[e & 1], q[e]);
+        sum[0] = L::add(sum[0], q[8]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) q[e] = L::mul(q[e], q[4 + e]);
+        lgs = L::add(lgs, L::lg(L::mul(L::mul(L::mul(q[0], q[1]), L::mul(q[2], q[3])), q[8])));
+    }
+};
+
+// Shared memory from the 1024-byte aligned base on: operand ring, staged rows, survivor queues,
+// candidate buffer, barriers.
+constexpr int kBarBytes = 256;
+constexpr size_t kOffB = (size_t)kSlots * kSlotA;
+constexpr size_t kOffStage = kOffB + (size_t)kSlots * kSlotB;
+constexpr size_t kOffQueue = kOffStage + 2 * sizeof(CmpStage);
+constexpr size_t kOffYz = kOffQueue + kCmpEpiWarps * sizeof(CmpQueue);   // float4 [warp][4][32]
+constexpr size_t kOffEpi = kOffYz + (size_t)kCmpEpiWarps * 4 * 32 * sizeof(float4);
+constexpr size_t kOffBars = (kOffEpi + sizeof(EpiShared) + 15) & ~(size_t)15;
+constexpr size_t kCmpSmem = kOffBars + kBarBytes;
+static_assert(1024 + kCmpSmem <= 232448, "shared memory of one CTA");
+static_assert(kOffStage % 16 == 0 && kOffQueue % 16 == 0 && kOffYz % 16 == 0 && kOffEpi % 16 == 0,
+              "alignment");
 
 // kInstr: the instrumented instantiation (table checksums; with a.prof, per role the cycles spent
 // waiting, summed over CTAs: [0] loader on free slots, [1] MMA issuer on loaded slots, [2] MMA
 // issuer on free accumulator regions, [4] epilogue thread 0 on finished tiles, [5] kernel cycles,
 // [7] MMA issuer issuing MMAs and commits).
-// kPaired: the epilogue derives the cells and the bound of a lane's two triplets together in
-// f32x2 instructions (fewer instructions, more registers live: faster where the MMA pipeline
-// bounds the scan, slower where the epilogue does; the tuner measures both).
+// kPaired: the epilogue takes the bound of a lane's two triplets together in f32x2 instructions
+// (half the instructions of the one-at-a-time form).
 template <bool kInstr, bool kPaired>
-__global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const CmpArgs a) {
+__global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const __grid_constant__ CmpArgs a) {
     const long long t_start = kInstr ? clock64() : 0;
     unsigned long long* const prof = kInstr ? a.prof : nullptr;
     unsigned long long w_acc = 0, w_acc2 = 0, w_acc3 = 0;
@@ -307,18 +602,19 @@ __global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const CmpArgs 
     uint8_t* base = reinterpret_cast<uint8_t*>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     uint8_t* sA = base;                                 // [kSlots][kSlotSteps][16 KB] rows (j, b)
-    uint8_t* sB = base + kSlots * kSlotA;               // [kSlots][kSlotSteps][8 KB] rows (k, z)
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sB + kSlots * kSlotB);
-    // bars: fullS[kSlots], emptyS[kSlots], accF[2], regE[kCmpRegions], drain
-    constexpr int kNBars = 2 * kSlots + 2 + kCmpRegions + 1;
-    static_assert(kNBars * 8 + 8 <= 256, "barrier area");
+    uint8_t* sB = base + kOffB;                         // [kSlots][kSlotSteps][8 KB] rows (k, z)
+    CmpStage* const stage = reinterpret_cast<CmpStage*>(base + kOffStage);   // [2]
+    CmpQueue* const queues = reinterpret_cast<CmpQueue*>(base + kOffQueue);  // one per epilogue warp
+    EpiShared& es = *reinterpret_cast<EpiShared*>(base + kOffEpi);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(base + kOffBars);
+    // bars: fullS[kSlots], emptyS[kSlots], accF[2], rowF[2], rowE[2], regE[kCmpRegions], drain
+    constexpr int kNBars = 2 * kSlots + 6 + kCmpRegions + 1;
+    static_assert(kNBars * 8 + 12 <= kBarBytes, "barrier area");
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kNBars);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    volatile unsigned* loader_steps = reinterpret_cast<volatile unsigned*>(tmem_slot + 2);
-    EpiShared& es = *reinterpret_cast<EpiShared*>(reinterpret_cast<uint8_t*>(bars) + 256);
     const uint32_t fullS0 = smem_u32(bars), emptyS0 = smem_u32(bars + kSlots),
-                   accF0 = smem_u32(bars + 2 * kSlots), regE0 = accF0 + 16,
-                   drain0 = regE0 + 8 * kCmpRegions;
+                   accF0 = smem_u32(bars + 2 * kSlots), rowF0 = accF0 + 16, rowE0 = rowF0 + 16,
+                   regE0 = rowE0 + 16, drain0 = regE0 + 8 * kCmpRegions;
     const CohortDev& cd = a.cd;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -327,12 +623,16 @@ __global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const CmpArgs 
             mbar_init(fullS0 + 8 * s, 1);
             mbar_init(emptyS0 + 8 * s, 1);
         }
-        for (int b = 0; b < 2; ++b) mbar_init(accF0 + 8 * b, 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(accF0 + 8 * b, 1);
+            mbar_init(rowF0 + 8 * b, 2);
+            mbar_init(rowE0 + 8 * b, kCmpEpiWarps);
+        }
         for (int r = 0; r < kCmpRegions; ++r) mbar_init(regE0 + 8 * r, kCmpEpiWarps);
         mbar_init(drain0, 1);
         *abort_flag = 0;
-        *loader_steps = 0u;
         es.cnt = 0;
+        for (int w = 0; w < kCmpEpiWarps; ++w) queues[w].n = 0;
         es.tloc = __int_as_float(0x7f800000);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -366,10 +666,9 @@ __global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const CmpArgs 
     __syncthreads();
     tc_fence_after();
 
-    const long long my_tiles =
-        a.n_tiles > blockIdx.x ? (a.n_tiles - blockIdx.x + gridDim.x - 1) / gridDim.x : 0;
     // role: 1 loader (on a free slot), 2 MMA issuer (region), 3 MMA issuer (operands),
-    // 4 epilogue (accumulators), 5 the timeout test hook
+    // 4 epilogue (accumulators), 5 the timeout test hook, 6 stager (free buffer), 7 epilogue
+    // (staged rows)
     auto fail_at = [&](unsigned role, long long tl, int q, int ks, unsigned extra = 0u) {
         *abort_flag = 1;
         if (atomicCAS(&cd.ctrl->wait_role, 0u, role) == 0u) {
@@ -377,330 +676,459 @@ __global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const CmpArgs 
             cd.ctrl->wait_set = (unsigned)q;
             cd.ctrl->wait_step = (unsigned)ks;
             cd.ctrl->pad_[0] = extra;
-            cd.ctrl->pad_[1] = *loader_steps;
         }
         atomicOr(&cd.ctrl->status, kStTimeout);
     };
 
+    // The loader (warp 0), the MMA issuer (warp 1) and the stagers run as whole warps with
+    // warp-uniform control flow; one elected lane issues each copy, MMA and commit.  Values read
+    // from memory are broadcast by shuffles so that every operand is provably uniform; a tile's
+    // sizes are fetched one tile ahead (lanes 0..3, one set each).
     if (warp < kCmpEpiWarp0) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kCmpRegCtl));
-        // The loader (warp 0) and the MMA issuer (warp 1) run as whole warps with warp-uniform
-        // control flow; one elected lane issues each copy, MMA and commit.  Values read from
-        // memory are broadcast from lane 0 so that every operand is provably uniform.
-        if (warp == 0) {
-            // ------------------------------------------------ operand loader
-            Ring rs{0, 0u};
-            uint32_t used = 0, fph = 0;
-            bool stop = false;
-            for (long long tl = 0; tl < my_tiles && !stop; ++tl) {
-                const CmpTile T = cmp_tile(a, blockIdx.x + tl * gridDim.x);
-                const int f = warp_uniform(T.f), jb = warp_uniform(T.jb), kb = warp_uniform(T.kb);
-                const CmpFirst& F = a.firsts[f];
-                const int b_lo = warp_uniform(F.b_lo);
-                for (int q = 0; q < kCmpSets && !stop; ++q) {
-                    const int KS = warp_uniform(F.ks[q]);
-                    const long long base_q = warp_uniform(F.base[q]);
-                    const long long ca0 = base_q + (long long)(jb - b_lo) * KS;
-                    const long long cb0 = base_q + (long long)((kb >> 1) - b_lo) * KS;
-                    const size_t boff = (size_t)(kb & 1) * kStepB;
-                    for (int ks = 0; ks < KS; ks += kSlotSteps) {
-                        // a slot takes up to kSlotSteps consecutive steps of one set: their A
-                        // chunks are adjacent (one copy), their B halves are not
-                        const int n = min(kSlotSteps, KS - ks);
-                        const int s = rs.s;
-                        const bool got = mbar_wait_t(emptyS0 + 8 * s, rs.ph ^ 1u, abort_flag,
-                                                     (prof && lane == 0) ? &w_acc : nullptr);
-                        if (!__all_sync(0xffffffffu, got)) {
-                            if (lane == 0) fail_at(1, tl, q, ks, (unsigned)s | (rs.ph << 8));
-                            stop = true;
-                            break;
-                        }
-                        const uint32_t fb = fullS0 + 8 * s;
-                        mbar_arrive_tx_elect(fb, (unsigned)(n * (kStepA + kStepB)));
-                        bulk_g2s_elect(smem_u32(sA + s * kSlotA), a.cmp + (size_t)(ca0 + ks) * kCmpChunk,
-                                       (unsigned)(n * kStepA), fb);
-                        for (int h = 0; h < n; ++h)
-                            bulk_g2s_elect(smem_u32(sB + s * kSlotB + h * kStepB),
-                                           a.cmp + (size_t)(cb0 + ks + h) * kCmpChunk + boff, kStepB, fb);
-                        used |= 1u << s;
-                        fph ^= 1u << s;
-                        ring_next(rs, kSlots);
-                        if (lane == 0) *loader_steps = *loader_steps + (unsigned)n;
+    if (warp == 0) {
+        // ------------------------------------------------ operand loader
+        static_assert(kSlotSteps == 2, "load_slot_elect");
+        const uint32_t sA0 = smem_u32(sA), sB0 = smem_u32(sB);
+        Ring rs{0, 0u};
+        uint32_t used = 0, fph = 0;
+        bool stop = false;
+        CmpCursor cu;
+        bool have = cu.first(a);
+        int ks_n = 0, blo_n = 0;
+        long long base_n = 0;
+        auto fetch = [&](int f) {
+            ks_n = a.firsts[f].ks[lane & 3];
+            base_n = a.firsts[f].base[lane & 3];
+            blo_n = a.firsts[f].b_lo;
+        };
+        if (have) fetch(cu.f);
+        for (long long tl = 0; have && !stop; ++tl) {
+            const int ks_l = ks_n, b_lo = warp_uniform(blo_n);
+            const long long base_l = base_n;
+            const int jb = warp_uniform(cu.jb), kb = warp_uniform(cu.kb);
+            have = cu.next(a);
+            if (have) fetch(cu.f);
+            for (int q = 0; q < kCmpSets && !stop; ++q) {
+                const int KS = __shfl_sync(0xffffffffu, ks_l, q);
+                const long long base_q = __shfl_sync(0xffffffffu, base_l, q);
+                const uint8_t* pa = a.cmp + (size_t)(base_q + (long long)(jb - b_lo) * KS) * kCmpChunk;
+                const uint8_t* pb = a.cmp + (size_t)(base_q + (long long)((kb >> 1) - b_lo) * KS) * kCmpChunk +
+                                    (size_t)(kb & 1) * kStepB;
+                for (int ks = 0; ks < KS; ks += kSlotSteps) {
+                    // a slot takes up to kSlotSteps consecutive steps of one set: their A
+                    // chunks are adjacent (one copy), their B halves are not
+                    const int n = min(kSlotSteps, KS - ks);
+                    const int s = rs.s;
+                    const bool got = mbar_wait_t(emptyS0 + 8 * s, rs.ph ^ 1u, abort_flag,
+                                                 (prof && lane == 0) ? &w_acc : nullptr);
+                    if (!__all_sync(0xffffffffu, got)) {
+                        if (lane == 0) fail_at(1, tl, q, ks, (unsigned)s | (rs.ph << 8));
+                        stop = true;
+                        break;
                     }
+                    load_slot_elect(fullS0 + 8 * s, sA0 + (uint32_t)(s * kSlotA), pa, (uint32_t)(n * kStepA),
+                                    sB0 + (uint32_t)(s * kSlotB), pb, n > 1 ? 1u : 0u);
+                    pa += (size_t)kSlotSteps * kCmpChunk;
+                    pb += (size_t)kSlotSteps * kCmpChunk;
+                    used |= 1u << s;
+                    fph ^= 1u << s;
+                    ring_next(rs, kSlots);
                 }
             }
-            // drain: the copies issued must land before the CTA exits
-            for (int b = 0; b < kSlots; ++b) {
-                if (!((used >> b) & 1u)) continue;
-                volatile int no_abort = 0;
-                mbar_wait(fullS0 + 8 * b, ((fph >> b) & 1u) ^ 1u, &no_abort);
-            }
-            __syncwarp();
-        } else if (warp == 1) {
-            // ------------------------------------------------ MMA issuer
-            bool ok = true;
-            if (cd.inject_timeout) {  // test hook: a wait that can only run out (about 1 s)
-                const bool got = mbar_wait(drain0, 0, abort_flag);
-                if (!__all_sync(0xffffffffu, got) && lane == 0) fail_at(5, 0, 0, 0);
-                ok = false;
-            }
-            Ring rR{0, 0u}, rs{0, 0u};
-            unsigned consumed = 0;
-            const uint32_t aS = smem_u32(sA), bS = smem_u32(sB);
-            for (long long tl = 0; tl < my_tiles && ok; ++tl) {
-                const CmpTile T = cmp_tile(a, blockIdx.x + tl * gridDim.x);
-                const CmpFirst& F = a.firsts[warp_uniform(T.f)];
-                for (int q = 0; q < kCmpSets && ok; ++q) {
-                    const bool freed = mbar_wait_t(regE0 + 8 * rR.s, rR.ph ^ 1u, abort_flag,
-                                                   (prof && lane == 0) ? &w_acc2 : nullptr);
-                    if (!__all_sync(0xffffffffu, freed)) {
-                        if (lane == 0) fail_at(2, tl, q, 0);
+        }
+        // drain: the copies issued must land before the CTA exits
+        for (int b = 0; b < kSlots; ++b) {
+            if (!((used >> b) & 1u)) continue;
+            volatile int no_abort = 0;
+            mbar_wait(fullS0 + 8 * b, ((fph >> b) & 1u) ^ 1u, &no_abort);
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ------------------------------------------------ MMA issuer
+        bool ok = true;
+        if (cd.inject_timeout) {  // test hook: a wait that can only run out (about 1 s)
+            const bool got = mbar_wait(drain0, 0, abort_flag);
+            if (!__all_sync(0xffffffffu, got) && lane == 0) fail_at(5, 0, 0, 0);
+            ok = false;
+        }
+        Ring rR{0, 0u}, rs{0, 0u};
+        const uint64_t da0 = sw128_desc(smem_u32(sA)), db0 = sw128_desc(smem_u32(sB));
+        CmpCursor cu;
+        bool have = cu.first(a);
+        int ks_n = have ? a.firsts[cu.f].ks[lane & 3] : 0;
+        for (long long tl = 0; have && ok; ++tl) {
+            const int ks_l = ks_n;
+            have = cu.next(a);
+            if (have) ks_n = a.firsts[cu.f].ks[lane & 3];
+            for (int q = 0; q < kCmpSets && ok; ++q) {
+                const bool freed = mbar_wait_t(regE0 + 8 * rR.s, rR.ph ^ 1u, abort_flag,
+                                               (prof && lane == 0) ? &w_acc2 : nullptr);
+                if (!__all_sync(0xffffffffu, freed)) {
+                    if (lane == 0) fail_at(2, tl, q, 0);
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t d = tmem + (uint32_t)(rR.s * kN);
+                ring_next(rR, kCmpRegions);
+                const int KS = __shfl_sync(0xffffffffu, ks_l, q);
+                for (int ks = 0; ks < KS; ks += kSlotSteps) {
+                    const int n = min(kSlotSteps, KS - ks);
+                    const int s = rs.s;
+                    const bool got = mbar_wait_t(fullS0 + 8 * s, rs.ph, abort_flag,
+                                                 (prof && lane == 0) ? &w_acc : nullptr);
+                    if (!__all_sync(0xffffffffu, got)) {
+                        if (lane == 0) fail_at(3, tl, q, ks, (unsigned)s | (rs.ph << 8));
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t d = tmem + (uint32_t)(rR.s * kN);
-                    ring_next(rR, kCmpRegions);
-                    const int KS = warp_uniform(F.ks[q]);
-                    for (int ks = 0; ks < KS; ks += kSlotSteps) {
-                        const int n = min(kSlotSteps, KS - ks);
-                        const int s = rs.s;
-                        const bool got = mbar_wait_t(fullS0 + 8 * s, rs.ph, abort_flag,
-                                                     (prof && lane == 0) ? &w_acc : nullptr);
-                        if (!__all_sync(0xffffffffu, got)) {
-                            if (lane == 0) fail_at(3, tl, q, ks, (unsigned)s | (rs.ph << 8) | (consumed << 16));
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
-                        const long long t_issue = prof ? clock64() : 0;
-                        for (int h = 0; h < n; ++h) {
-                            const uint64_t da = sw128_desc(aS + (uint32_t)(s * kSlotA + h * kStepA));
-                            const uint64_t db = sw128_desc(bS + (uint32_t)(s * kSlotB + h * kStepB));
-#pragma unroll
-                            for (int kk = 0; kk < 4; ++kk)  // 32 bytes (64 samples) of K per MMA
-                                mma_ss_mx_elect(d, da + 2 * kk, db + 2 * kk, (ks | h | kk) ? 1u : 0u,
-                                                tmem + kCmpSfCol, tmem + kCmpSfCol + 16);
-                        }
-                        tc_commit_elect(emptyS0 + 8 * s);  // the slot is free once these MMAs complete
-                        if (prof) w_acc3 += (unsigned long long)(clock64() - t_issue);
-                        ring_next(rs, kSlots);
-                        consumed += (unsigned)n;
-                    }
+                    const long long t_issue = prof ? clock64() : 0;
+                    const uint64_t da = da0 + (uint32_t)(s * (kSlotA >> 4)), db = db0 + (uint32_t)(s * (kSlotB >> 4));
+                    mma_step_elect(d, da, db, (uint32_t)ks, tmem + kCmpSfCol, tmem + kCmpSfCol + 16);
+                    if (n > 1)
+                        mma_step_elect(d, da + (kStepA >> 4), db + (kStepB >> 4), 1u, tmem + kCmpSfCol,
+                                       tmem + kCmpSfCol + 16);
+                    tc_commit_elect(emptyS0 + 8 * s);  // the slot is free once these MMAs complete
+                    if (prof) w_acc3 += (unsigned long long)(clock64() - t_issue);
+                    ring_next(rs, kSlots);
                 }
-                if (ok) tc_commit_elect(accF0 + 8 * (int)(tl & 1));
             }
-            // every MMA issued must complete before tensor memory is released
-            tc_commit_elect(drain0);
-            volatile int no_abort = 0;
-            mbar_wait(drain0, 0, &no_abort);
-            __syncwarp();
+            if (ok) tc_commit_elect(accF0 + 8 * (int)(tl & 1));
         }
+        // every MMA issued must complete before tensor memory is released
+        tc_commit_elect(drain0);
+        volatile int no_abort = 0;
+        mbar_wait(drain0, 0, &no_abort);
+        __syncwarp();
     } else {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kCmpRegEpi));
+        // ------------------------------------------------ stagers (warps 2 and 3)
+        // The (i, j) and (i, k) parts of a tile's derived cells, with SNP i's genotypes
+        // relabelled, ready as the epilogue's operands: the epilogue warps used to form them per
+        // thread from pair-table rows they each loaded from L2.  One j per lane (32 of the tile's
+        // 64 to each stager) and one k per lane of the first; the next tile's table entries are
+        // fetched while this one's buffer is not free yet.
+        const int M = cd.pl.M, half = warp - 2;
+        const PairTables& pt = cd.pt;
+        const int cm = a.minor;
+        const float kInf = __int_as_float(0x7f800000);
+        const bool prune_on = !cd.dbg && !(kInstr && cd.tsum);
+        CmpCursor cu;
+        bool have = cu.first(a);
+        int4 nxy[2], nxz[2];
+        int2 nmx[2], nmy[2], nmz[2];
+        int ndrop = 0;
+        auto fetch = [&]() {
+            const int i = a.i0 + cu.f, j = kTJ * cu.jb + 32 * half + lane, k = kTK * cu.kb + lane;
+            const int jc = j < M && j > i ? j : i + 1, kc = k < M && k > i ? k : i + 1;   // i + 1 < M
+            ndrop = a.firsts[cu.f].drop;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const int4* const tab = pt.pt + c * pt.n_pairs;
+                const int2* const mg = pt.marg + (size_t)c * M;
+                nmx[c] = __ldg(mg + i);
+                nmy[c] = __ldg(mg + jc);
+                nxy[c] = __ldg(tab + pair_index(i, jc));
+                if (half == 0) {
+                    nmz[c] = __ldg(mg + kc);
+                    nxz[c] = __ldg(tab + pair_index(i, kc));
+                }
+            }
+        };
+        if (have) fetch();
+        for (long long tl = 0; have; ++tl) {
+            const int f = cu.f, i = a.i0 + f, jb = cu.jb, kb = cu.kb, drop = ndrop;
+            const int fresh = f == cu.f0 ? kStageRun : 0;
+            const int j = kTJ * jb + 32 * half + lane;
+            const bool in = j < M && j > i;
+            const long long pij = in ? pair_index(i, j) : -1;
+            int w[2][9];   // [class]: [0..3] xy, [4..5] (a, 2), [6..7] (2, b), [8] (2, 2)
+            int wz[2][6];  // [class]: [0..3] xz, [4..5] (2, z)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const int2 mx = relabel_marg(nmx[c], pt.n_c[c], drop);
+                const int4 p = relabel_xy(nxy[c], nmy[c], drop);
+                w[c][0] = p.x;
+                w[c][1] = p.y;
+                w[c][2] = p.z;
+                w[c][3] = p.w;
+                w[c][4] = mx.x - p.x - p.y;
+                w[c][5] = mx.y - p.z - p.w;
+                w[c][6] = nmy[c].x - p.x - p.z;
+                w[c][7] = nmy[c].y - p.y - p.w;
+                w[c][8] = pt.n_c[c] - mx.x - mx.y - w[c][6] - w[c][7];
+                if (half == 0) {
+                    const int4 z = relabel_xy(nxz[c], nmz[c], drop);
+                    wz[c][0] = z.x;
+                    wz[c][1] = z.y;
+                    wz[c][2] = z.z;
+                    wz[c][3] = z.w;
+                    wz[c][4] = nmz[c].x - z.x - z.z;
+                    wz[c][5] = nmz[c].y - z.y - z.w;
+                }
+            }
+            have = cu.next(a);
+            if (have) fetch();
+            const int buf = (int)(tl & 1);
+            if (!__all_sync(0xffffffffu, mbar_wait(rowE0 + 8 * buf, (unsigned)((tl >> 1) & 1) ^ 1u,
+                                                   abort_flag))) {
+                if (lane == 0) fail_at(6, tl, 0, 0);
+                break;
+            }
+            CmpStage& S = stage[buf];
+            // a bound above this proves the exact score above the threshold (cmp_bound_terms)
+            const float thr = fminf(__uint_as_float(*(volatile unsigned*)&cd.ctrl->thr), *(volatile float*)&es.tloc);
+            const float cut = prune_on && thr < kInf ? __fadd_ru(thr, a.bound_off) : kInf;
+            constexpr int kOrder[9] = {0, 1, 4, 2, 3, 5, 6, 7, 8};   // phase-major
+            float4* const dst = &S.row[32 * half + lane][0][0];
+#pragma unroll
+            for (int e = 0; e < 9; ++e) {
+                const int o = kOrder[e];
+                const float s = (float)(w[0][o] + w[1][o] + 6), m = (float)((cm ? w[1][o] : w[0][o]) + 3);
+                dst[e] = make_float4(s, s, m, m);
+            }
+            S.thr[32 * half + lane] = pij >= cd.pair_begin && pij < cd.pair_end ? cut : -kInf;
+            if (half == 0) {
+                float* const dz = reinterpret_cast<float*>(&S.col[lane >> 1][0][0]) + (lane & 1);
+#pragma unroll
+                for (int ph = 0; ph < 3; ++ph)
+#pragma unroll
+                    for (int z = 0; z < 2; ++z) {
+                        const int o = 2 * ph + z;
+                        dz[2 * (4 * ph + z)] = (float)(wz[0][o] + wz[1][o] + 6);
+                        dz[2 * (4 * ph + 2 + z)] = (float)((cm ? wz[1][o] : wz[0][o]) + 3);
+                    }
+                if (lane == 0) {
+                    S.f = f;
+                    S.jb = jb;
+                    S.kb = kb;
+                    S.flags = fresh | (have ? 0 : kStageLast);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(rowF0 + 8 * buf);
+        }
+        __syncwarp();
+    }
+    } else {
         // ------------------------------------------------ epilogue
         // Per set (c, a), tensor-memory lane 16 G + 8 b + r holds the counts + 1 of second SNP
         // jl = 8 G + r with genotype b, in column 16 H + 8 z + s for third SNP kl = 8 H + s with
         // genotype z (the chunks' row order).  A 16x256b.x2 load at lane group G, column group H
         // gives thread t the cells (b, z) of jl = 8 G + t / 4 and kl = 8 H + 2 (t % 4) + e,
-        // e = 0, 1, in registers 4 z + 2 b + e: all 8 cells of a set for two triplets.  Items of
-        // a quadrant: lane groups G = 2 quad + h (h = 0, 1) x column groups H = 0..3; part 0
-        // takes h = 0 with H = 0..2, part 1 h = 1 with H = 0..2, part 2 both h with H = 3.
+        // e = 0, 1, in registers 4 z + 2 b + e: all 8 cells of a set for two triplets, the two in
+        // neighbouring registers, as the f32x2 instructions take them.  Items of a quadrant: lane
+        // groups G = 2 quad + h (h = 0, 1) x column groups H = 0..3; each warp takes two column
+        // groups of one h.
+        // The bound per triplet: 27 cells x 4 FP32 operations, 76 subtractions for the 19 derived
+        // cells in two tables, 36 products for the shared reciprocals, i.e. about 230 FP32 lane
+        // operations (3700 cycles a tile at 128 a clock) and 18 reciprocals and logs (2300 at 16 a
+        // clock).  The form before, phi(us) - phi(u0) - phi(u1) per cell, took 81 logs, and each
+        // thread formed the constants that the stagers now form once a tile.
         const int tid = threadIdx.x - kCmpEpiWarp0 * 32;     // 0 .. 383
         const int quad = warp & 3, part = (warp - kCmpEpiWarp0) >> 2;
-        const int trow = lane >> 2, tcol = 2 * (lane & 3);
+        const int jl0 = 16 * quad + (lane >> 2), tcol = 2 * (lane & 3);
         const int M = cd.pl.M;
-        const PairTables pt = cd.pt;
-        const float2* lf2 = cd.k2.lf2;
-        const float prune = cd.k2.prune_delta;
-        float* dbg = cd.dbg;
-        Ctrl* ctrl = cd.ctrl;
-        const bool tsum_on = kInstr && cd.tsum != nullptr;
-        const bool pruning = !dbg && !tsum_on && prune > 0.f;
-        unsigned long long sum_h = 0, sum_n = 0;
-        Ring rR{0, 0u};
-        for (long long tl = 0; tl < my_tiles; ++tl) {
-            const CmpTile T = cmp_tile(a, blockIdx.x + tl * gridDim.x);
-            const int i = a.i0 + T.f, kb0 = kTK * T.kb;
-            bool bad = false;
-            if (tid == 0) {
-                bad = !mbar_wait_t(accF0 + 8 * (int)(tl & 1), (unsigned)((tl >> 1) & 1), abort_flag,
-                                   prof ? &w_acc : nullptr);
-                if (bad) fail_at(4, tl, 0, 0);
+        const int cm = a.minor;
+        const float cq = a.bound_c;
+        CmpQueue& qu = queues[warp - kCmpEpiWarp0];
+        unsigned long long sums[2] = {0, 0};
+        const uint32_t tbase = tmem + ((uint32_t)(32 * quad) << 16);
+        int reg0 = 0;            // region of the tile's first set
+        bool bad = false, last = (int)blockIdx.x >= a.n_runs;
+        int since = 0, interval = 1;
+        const int prune_at = min(max(2 * cd.top_k, 32), kPruneAt + 1);
+        // An item's (Y, Z) entries come into this lane's slots while the item before is worked on
+        // (asynchronous copies: plain loads shared a scoreboard with the shared-memory loads of the
+        // constants, and every item waited for L2).
+        const float4* const ys = reinterpret_cast<const float4*>(base + kOffYz) +
+                                 (size_t)(warp - kCmpEpiWarp0) * 128 + lane;   // [4], 32 apart
+        auto fetch = [&](int item) {
+            const float4* const src =
+                a.yz + 16 * ((size_t)qu.yz[item >> 2][lane] + (item & 3)) + (lane & 3);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) cp_async16(smem_u32(ys + 32 * e), src + 4 * e);
+            cp_async_commit();
+        };
+        for (unsigned tl = 0; !last; ++tl) {
+            // region of set q of this tile
+            auto region = [&](int q) { return reg0 + q < kCmpRegions ? reg0 + q : reg0 + q - kCmpRegions; };
+            const int buf = (int)(tl & 1);
+            if (!bad) {
+                const bool got = mbar_wait(rowF0 + 8 * buf, (tl >> 1) & 1u, abort_flag);
+                if (!__all_sync(0xffffffffu, got)) {
+                    if (lane == 0) fail_at(7, tl, 0, 0);
+                    bad = true;
+                }
             }
-            // uniform stop; also orders the previous tile's candidate bookkeeping before this
-            // tile's appends, and thread 0's observation of the barrier before every TMEM read
-            if (epi_sync_or<kCmpEpiThreads>(bad || *abort_flag)) break;
-            tc_fence_after();
-            int regs[kCmpSets];
+            if (!bad) {
+                const CmpStage& S = stage[buf];
+                last = (S.flags & kStageLast) != 0;
+                if (S.flags & kStageRun) {  // a new run: its (j, k) parts
+                    unsigned vmask = 0;
 #pragma unroll
-            for (int q = 0; q < kCmpSets; ++q) {
-                regs[q] = rR.s;
-                ring_next(rR, kCmpRegions);
+                    for (int it = 0; it < kCmpEpiItems; ++it) {
+                        const int item = part + kCmpEpiParts * it;
+                        const int j = kTJ * S.jb + jl0 + 8 * (item >> 2), k = kTK * S.kb + 8 * (item & 3) + tcol;
+                        if (item < 8)
+                            vmask |= ((k > j && k < M ? 1u : 0u) | (k + 1 > j && k + 1 < M ? 2u : 0u)) << (2 * it);
+                    }
+                    qu.vmask[lane] = vmask;
+                    // blocks of k <= j or k >= M are other pairs' or padding: masked
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        qu.yz[h][lane] = (unsigned)yz_block(min(kTJ * S.jb + jl0 + 8 * h, M - 1), kTK * S.kb, M);
+                    cp_async_wait();   // the last run's prefetch
+                    fetch(part);
+                }
+                const bool got = mbar_wait_t(accF0 + 8 * buf, (tl >> 1) & 1u, abort_flag,
+                                             (prof && tid == 0) ? &w_acc : nullptr);
+                if (!__all_sync(0xffffffffu, got)) {
+                    if (lane == 0) fail_at(4, tl, 0, 0);
+                    bad = true;
+                }
             }
-            // the derived first-SNP genotype; the first SNP's inputs relabelled
-            const int dsel = __ldg(&a.firsts[T.f].drop);
-            int2 mx[2];
-            mx[0] = relabel_marg(__ldg(pt.marg + i), pt.n_c[0], dsel);
-            mx[1] = relabel_marg(__ldg(pt.marg + M + i), pt.n_c[1], dsel);
-            int cur_h = -1, j = 0;
-            bool jrow = false;
-            RowCells rcl[2];
-            const int n_items = part == 2 ? 2 : 3;
-            for (int it = 0; it < n_items; ++it) {
-                const int h = part == 2 ? it : part, H = part == 2 ? 3 : it;
-                if (h != cur_h) {  // this thread's second SNP and its row cells
-                    cur_h = h;
-                    j = kTJ * T.jb + 8 * (2 * quad + h) + trow;
-                    long long pij = -1;
-                    if (j < M && j > i) {
-                        pij = pair_index(i, j);
-                        if (pij < cd.pair_begin || pij >= cd.pair_end) pij = -1;
-                    }
-                    jrow = pij >= 0;
-                    int4 pxy[2] = {make_int4(0, 0, 0, 0), make_int4(0, 0, 0, 0)};
-                    int2 my[2] = {make_int2(0, 0), make_int2(0, 0)};
-                    if (jrow) {
-                        pxy[0] = __ldg(pt.pt + pij);
-                        pxy[1] = __ldg(pt.pt + pt.n_pairs + pij);
-                        my[0] = __ldg(pt.marg + j);
-                        my[1] = __ldg(pt.marg + M + j);
-                    }
-                    rcl[0] = row_cells(relabel_xy(pxy[0], my[0], dsel), mx[0], my[0], pt.n_c[0]);
-                    rcl[1] = row_cells(relabel_xy(pxy[1], my[1], dsel), mx[1], my[1], pt.n_c[1]);
-                }
-                const float thr_g = __uint_as_float(*(volatile unsigned*)&ctrl->thr);
-                // this thread's two triplets: k = kb0 + 8 H + tcol + m; pair-table rows first
-                float4 tik[2][2], tjk[2][2];
-                float2 tmk[2][2];
-#pragma unroll
-                for (int m = 0; m < 2; ++m) {
-                    const int k = kb0 + 8 * H + tcol + m;
-                    const bool val = jrow && k > j && k < M;
-                    const long long pik = val ? pair_index(i, k) : 0, pjk = val ? pair_index(j, k) : 0;
-                    const int kq = val ? k : 0;
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        tik[m][c] = __ldg(pt.ptf + c * pt.n_pairs + pik);
-                        tjk[m][c] = __ldg(pt.ptf + c * pt.n_pairs + pjk);
-                        tmk[m][c] = __ldg(pt.margf + (size_t)c * M + kq);
-                    }
-                }
-#pragma unroll
-                for (int m = 0; m < 2; ++m)
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) tik[m][c] = relabel_xz(tik[m][c], tmk[m][c], dsel);
-                uint32_t v[kCmpSets][8];
-#pragma unroll
-                for (int q = 0; q < kCmpSets; ++q)
-                    tc_ld16x2(tmem + ((uint32_t)(32 * quad + 16 * h) << 16) + (uint32_t)(regs[q] * kN + 16 * H),
-                              v[q]);
-                tc_wait_ld();
-                // n8[c][4 a + 2 b + z] = count + 1 of triplet m: set 2 c + a, register 4 z + 2 b + m
-                auto n8_of = [&](int m, int c, int e) {
-                    return __uint_as_float(v[2 * c + (e >> 2)][4 * (e & 1) + 2 * ((e >> 1) & 1) + m]);
-                };
-                // paired form: the lane's two triplets in the two lanes of f32x2 instructions
-                // (x: m = 0, y: m = 1); the inputs are gathered into lane pairs once, and the bound
-                // derives both classes' cells on the fly
-                float2 n8p[2][8], xzp[2][2][2], yzp[2][2][2], mzp[2][2], bnd = make_float2(0.f, 0.f);
-                if constexpr (kPaired) {
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) n8p[c][e] = make_float2(n8_of(0, c, e), n8_of(1, c, e));
-                        const float4 x0 = tik[0][c], x1 = tik[1][c], y0 = tjk[0][c], y1 = tjk[1][c];
-                        xzp[c][0][0] = make_float2(x0.x, x1.x); xzp[c][0][1] = make_float2(x0.y, x1.y);
-                        xzp[c][1][0] = make_float2(x0.z, x1.z); xzp[c][1][1] = make_float2(x0.w, x1.w);
-                        yzp[c][0][0] = make_float2(y0.x, y1.x); yzp[c][0][1] = make_float2(y0.y, y1.y);
-                        yzp[c][1][0] = make_float2(y0.z, y1.z); yzp[c][1][1] = make_float2(y0.w, y1.w);
-                        mzp[c][0] = make_float2(tmk[0][c].x, tmk[1][c].x);
-                        mzp[c][1] = make_float2(tmk[0][c].y, tmk[1][c].y);
-                    }
-                    if (pruning) {
-                        const float2 sacc = k2_bound_cells<LaneOps2>(n8p, rcl, xzp, yzp, mzp);
-                        bnd = make_float2(k2_bound_finish(sacc.x), k2_bound_finish(sacc.y));
-                    }
-                }
-#pragma unroll
-                for (int m = 0; m < 2; ++m) {
-                    const int k = kb0 + 8 * H + tcol + m;
-                    if (!(jrow && k > j && k < M)) continue;
-                    // triplet m's inputs: counted cells, pair-table rows (X, Z), (Y, Z), marginal of Z
-                    float n8[2][8], xz[2][2][2], yz[2][2][2], mz[2][2];
-#pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        if constexpr (kPaired) {
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) n8[c][e] = m ? n8p[c][e].y : n8p[c][e].x;
-#pragma unroll
-                            for (int t = 0; t < 4; ++t) {
-                                xz[c][t >> 1][t & 1] = m ? xzp[c][t >> 1][t & 1].y : xzp[c][t >> 1][t & 1].x;
-                                yz[c][t >> 1][t & 1] = m ? yzp[c][t >> 1][t & 1].y : yzp[c][t >> 1][t & 1].x;
-                            }
-                            mz[c][0] = m ? mzp[c][0].y : mzp[c][0].x;
-                            mz[c][1] = m ? mzp[c][1].y : mzp[c][1].x;
-                        } else {
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) n8[c][e] = n8_of(m, c, e);
-                            const float4 x = tik[m][c], y = tjk[m][c];
-                            xz[c][0][0] = x.x; xz[c][0][1] = x.y; xz[c][1][0] = x.z; xz[c][1][1] = x.w;
-                            yz[c][0][0] = y.x; yz[c][0][1] = y.y; yz[c][1][0] = y.z; yz[c][1][1] = y.w;
-                            mz[c][0] = tmk[m][c].x;
-                            mz[c][1] = tmk[m][c].y;
-                        }
-                    }
-                    // most tables lie far above the band: prove it from the table-free
-                    // approximation and skip the exact score's log-table gathers
-                    if (pruning) {
-                        const float bm = kPaired ? (m ? bnd.y : bnd.x)
-                                                 : k2_bound_finish(k2_bound_cells<LaneOps1>(n8, rcl, xz, yz, mz));
-                        if (__fsub_rn(bm, prune) > fminf(es.tloc, thr_g)) continue;
-                    }
-                    // a survivor (or every table, without pruning): its exact cells
-                    float u0[kCells], u1[kCells];
-#pragma unroll
-                    for (int c = 0; c < 2; ++c)
-                        cells_u(n8[c], rcl[c], make_float4(xz[c][0][0], xz[c][0][1], xz[c][1][0], xz[c][1][1]),
-                                make_float4(yz[c][0][0], yz[c][0][1], yz[c][1][0], yz[c][1][1]),
-                                make_float2(mz[c][0], mz[c][1]), c ? u1 : u0);
-                    canon_rows(u0, dsel);
-                    canon_rows(u1, dsel);
-                    int r0[kCells], r1[kCells];
-                    if (!counts_of(u0, u1, pt.n_c[0], pt.n_c[1], r0, r1)) {
-                        atomicOr(&ctrl->status, kStBadCount);
+            if (!bad) {
+                tc_fence_after();
+                const CmpStage& S = stage[buf];
+#pragma unroll 1
+                for (int it = 0; it < kCmpEpiItems; ++it) {
+                    const int item = part + kCmpEpiParts * it, jl = jl0 + 8 * (item >> 2);
+                    const unsigned vmask = (qu.vmask[lane] >> (2 * it)) & 3u;
+                    if (item >= 8) break;
+                    const int next = item + kCmpEpiParts < 8 ? item + kCmpEpiParts : part;
+                    if (!__any_sync(0xffffffffu, vmask)) {   // k <= j throughout
+                        cp_async_wait();
+                        fetch(next);
                         continue;
                     }
-                    const float sc = k2_f32(r0, r1, lf2);
-                    if (dbg) dbg[((size_t)i * M + j) * M + k] = sc;
-                    if (tsum_on) {
-                        sum_h += table_hash(i, j, k, r0, r1);
-                        ++sum_n;
+                    const float cut = S.thr[jl];
+                    const float4* const row = &S.row[jl][0][0];
+                    const float4* const col =
+                        reinterpret_cast<const float4*>(&S.col[4 * (item & 3) + (lane & 3)][0][0]);
+                    const uint32_t tb = tbase + (uint32_t)(16 * (item & 3)) + ((uint32_t)(item & 4) << 18);
+                    unsigned sv = 0;
+#pragma unroll
+                    for (int pass = 0; pass < (kPaired ? 1 : 2); ++pass) {
+                        typedef typename std::conditional<kPaired, LaneOps2, LaneOps1>::type L;
+                        typedef typename L::T T;
+                        CmpBound<L> B;
+                        B.init();
+                        float v[2][8];    // one counted genotype's cells: the larger class, the smaller
+                        auto load = [&](int ph) {
+                            tc_ld16x2(tb + (uint32_t)(region(2 * (cm ^ 1) + ph) * kN), v[0]);
+                            tc_ld16x2(tb + (uint32_t)(region(2 * cm + ph) * kN), v[1]);
+                        };
+                        T ds[4], dm[4];   // cells (2, b, z): the (Y, Z) table minus the counted genotypes
+#pragma unroll
+                        for (int ph = 0; ph < 3; ++ph) {
+                            T us[4], um[4];   // cells (b, z) of this first-SNP genotype, index 2 b + z
+                            float4 y4[4];
+                            if (ph == 2) {
+                                if (pass == 0) cp_async_wait();
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) y4[e] = ys[32 * e];
+                            }
+                            if (ph < 2) {
+                                load(ph);
+                                tc_wait_ld2(v);
+                            }
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                if (ph < 2) {
+                                    const int w = 4 * (e & 1) + 2 * (e >> 1);
+                                    const T c0 = L::pick(make_float2(v[0][w], v[0][w + 1]), pass);
+                                    const T c1 = L::pick(make_float2(v[1][w], v[1][w + 1]), pass);
+                                    us[e] = L::add(c0, c1);
+                                    um[e] = c1;
+                                    ds[e] = ph ? L::add(ds[e], us[e]) : us[e];
+                                    dm[e] = ph ? L::add(dm[e], um[e]) : um[e];
+                                } else {
+                                    const float4 ys = y4[e >> 1], ym = y4[2 + (e >> 1)];
+                                    us[e] = L::sub(L::pick(e & 1 ? make_float2(ys.z, ys.w) : make_float2(ys.x, ys.y), pass), ds[e]);
+                                    um[e] = L::sub(L::pick(e & 1 ? make_float2(ym.z, ym.w) : make_float2(ym.x, ym.y), pass), dm[e]);
+                                }
+                            }
+                            const float4 cs = col[2 * ph], cmn = col[2 * ph + 1];
+                            const float4 r0 = row[3 * ph], r1 = row[3 * ph + 1], r2 = row[3 * ph + 2];
+                            const T cst[9] = {us[0], us[1], us[2], us[3], L::two(r0.x, r0.y), L::two(r1.x, r1.y),
+                                              L::pick(make_float2(cs.x, cs.y), pass),
+                                              L::pick(make_float2(cs.z, cs.w), pass), L::two(r2.x, r2.y)};
+                            const T cmt[9] = {um[0], um[1], um[2], um[3], L::two(r0.z, r0.w), L::two(r1.z, r1.w),
+                                              L::pick(make_float2(cmn.x, cmn.y), pass),
+                                              L::pick(make_float2(cmn.z, cmn.w), pass), L::two(r2.z, r2.w)};
+                            T s9[9], m9[9];   // (., b, z), (., 0, 2), (., 1, 2), (., 2, 0), (., 2, 1), (., 2, 2)
+#pragma unroll
+                            for (int e = 0; e < 9; ++e) {
+                                s9[e] = cst[e];
+                                m9[e] = cmt[e];
+                            }
+                            constexpr int kSub[8] = {0, 2, 0, 1, 1, 3, 2, 3};   // first and second minuend's partner
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                s9[4 + e] = L::sub(s9[4 + e], us[kSub[e]]);
+                                m9[4 + e] = L::sub(m9[4 + e], um[kSub[e]]);
+                            }
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                s9[4 + e] = L::sub(s9[4 + e], us[kSub[4 + e]]);
+                                m9[4 + e] = L::sub(m9[4 + e], um[kSub[4 + e]]);
+                            }
+                            s9[8] = L::sub(L::sub(s9[8], s9[6]), s9[7]);
+                            m9[8] = L::sub(L::sub(m9[8], m9[6]), m9[7]);
+                            if (ph == 2 && (kPaired || pass == 1)) fetch(next);
+                            B.phase(s9, m9);
+                        }
+                        // ln 2 / 2 (sum of lg2 q) + c (sum of q) against the cut
+                        const T b = L::fma(L::dup(cq), L::add(B.sum[0], B.sum[1]), L::mul(L::dup(0.34657359f), B.lgs));
+                        if constexpr (kPaired) sv = (b.x > cut ? 0u : 1u) | (b.y > cut ? 0u : 2u);
+                        else sv |= (b > cut ? 0u : 1u) << pass;
                     }
-                    if (sc <= fminf(es.tloc, thr_g)) {
-                        const int idx = atomicAdd(&es.cnt, 1);
-                        if (idx < kCandCap) es.buf[idx] = Cand{sc, i, j, k};
-                        else cand_global(cd, Cand{sc, i, j, k});
+                    sv &= vmask;
+                    if (__any_sync(0xffffffffu, sv != 0u)) {
+                        CmpItems x;
+#pragma unroll
+                        for (int q = 0; q < kCmpSets; ++q) x.t[q] = tb + (uint32_t)(region(q) * kN);
+                        x.i = a.i0 + S.f;
+                        x.j = kTJ * S.jb + jl;
+                        x.k0 = kTK * S.kb + 8 * (item & 3) + tcol;
+                        x.mask = sv;
+                        cmp_survivors<kInstr>(a, es, qu, x, kInstr ? sums : nullptr);
                     }
                 }
-            }
-            // accumulators read: the four regions go back to the MMA issuer
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0)
+                // accumulators and staged rows read: back to the MMA issuer and the stager
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) {
 #pragma unroll
-                for (int q = 0; q < kCmpSets; ++q) mbar_arrive(regE0 + 8 * regs[q]);
-            epi_sync<kCmpEpiThreads>();  // every append of this tile is in
-            const int cnt = min(es.cnt, kCandCap);
-            if (cnt > kPruneAt) {  // uniform: every thread read the same count
-                epi_sync<kCmpEpiThreads>();
+                    for (int q = 0; q < kCmpSets; ++q) mbar_arrive(regE0 + 8 * region(q));
+                    mbar_arrive(rowE0 + 8 * buf);
+                }
+            }
+            reg0 = region(kCmpSets);
+            if (++since < interval && !last) continue;
+            // rendezvous of the epilogue warps: agree on a stop, and cut the candidate buffer to
+            // this CTA's best once it holds twice as many (which lowers the threshold).  It comes
+            // less often while few candidates arrive: the schedule is the same for every warp,
+            // since it depends on a count read between two barriers.
+            if (epi_sync_or<kCmpEpiThreads>(bad || *abort_flag)) break;
+            const int cnt = min(*(volatile int*)&es.cnt, kCandCap);
+            epi_sync<kCmpEpiThreads>();
+            interval = cnt >= prune_at ? 1 : min(kMaxSyncTiles, 2 * interval);
+            since = 0;
+            if (cnt >= prune_at) {
                 const int kept = epi_prune<kCmpEpiThreads>(cd, es, cnt, tid, false);
                 if (tid == 0) es.cnt = kept;
+                epi_sync<kCmpEpiThreads>();
             }
+        }
+        {   // what is left in this warp's queue
+            CmpItems x{};
+            cmp_survivors<kInstr>(a, es, qu, x, kInstr ? sums : nullptr);
         }
         epi_sync<kCmpEpiThreads>();
         epi_prune<kCmpEpiThreads>(cd, es, min(es.cnt, kCandCap), tid, true);
-        if (tsum_on) table_sum_flush(cd.tsum, sum_h, sum_n);
+        if (kInstr && cd.tsum) table_sum_flush(cd.tsum, sums[0], sums[1]);
     }
     if (prof) {
         if (warp == 0 && lane == 0) atomicAdd(prof + 0, w_acc);
@@ -724,7 +1152,8 @@ __global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const CmpArgs 
 
 }  // namespace
 
-size_t scan_cmp_smem() { return 1024 + kSlots * (kSlotA + kSlotB) + 256 + sizeof(EpiShared) + 64; }
+size_t scan_cmp_smem() { return 1024 + kCmpSmem; }   // the base is aligned to 1024 bytes
+int scan_cmp_threads() { return kCmpThreads; }
 
 int cmp_tiles_of(int M, int b_lo, int jb_end) {
     const int nb = std::min((M + 63) / 64, jb_end), nk = (M + kTK - 1) / kTK;
@@ -744,25 +1173,19 @@ cudaError_t launch_compact(const Planes& pl, const CmpFirst* firsts, int i0, int
 template <bool kInstr, bool kPaired>
 static cudaError_t launch_cmp_variant(const CmpArgs& a, int grid, cudaStream_t st) {
     const size_t smem = scan_cmp_smem();
-    // once per device: the register split adds up to exactly the launch's registers, so refuse a
-    // build whose register count differs (its increase could never be granted); then allow the
-    // dynamic shared memory
+    // once per device: allow the dynamic shared memory
     static std::atomic<unsigned long long> ready{0};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     const unsigned long long bit = 1ull << (dev & 63);
     if (!(ready.load(std::memory_order_acquire) & bit)) {
-        cudaFuncAttributes fa{};
-        e = cudaFuncGetAttributes(&fa, scan_cmp_kernel<kInstr, kPaired>);
-        if (e != cudaSuccess) return e;
-        if (fa.numRegs != kCmpRegLaunch) return cudaErrorInvalidConfiguration;
         e = cudaFuncSetAttribute(scan_cmp_kernel<kInstr, kPaired>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem);
         if (e != cudaSuccess) return e;
         ready.fetch_or(bit, std::memory_order_release);
     }
-    if (a.n_tiles == 0) return cudaSuccess;
+    if (a.n_runs == 0) return cudaSuccess;
     scan_cmp_kernel<kInstr, kPaired><<<grid, kCmpThreads, smem, st>>>(a);
     return cudaGetLastError();
 }

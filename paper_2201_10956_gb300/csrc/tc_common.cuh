@@ -79,19 +79,6 @@ __device__ __forceinline__ void tc_commit(uint32_t mbar) {
 // about 69 cycles per MMA on GB300 (48 cycles for an M=128 N=64 MMA issued warp-wide, which is
 // its shared-memory operand read at 128 B/clk).  elect.sync picks the same leader every time in a
 // full warp, so a commit covers the MMAs that the same lane issued.
-__device__ __forceinline__ void mbar_arrive_tx_elect(uint32_t a, unsigned bytes) {
-    asm volatile(
-        "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
-        " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}\n"
-        ::"r"(a), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void bulk_g2s_elect(uint32_t dst, const void* src, unsigned bytes,
-                                               uint32_t mbar) {
-    asm volatile(
-        "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
-        " @e cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n}\n"
-        ::"r"(dst), "l"(src), "r"(bytes), "r"(mbar) : "memory");
-}
 __device__ __forceinline__ void tc_commit_elect(uint32_t mbar) {
     asm volatile(
         "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
@@ -100,9 +87,6 @@ __device__ __forceinline__ void tc_commit_elect(uint32_t mbar) {
 }
 // A value every lane holds alike, made provably warp-uniform for the compiler.
 __device__ __forceinline__ int warp_uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
-__device__ __forceinline__ long long warp_uniform(long long v) {
-    return __shfl_sync(0xffffffffu, v, 0);
-}
 __device__ __forceinline__ void tc_wait_st() {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
@@ -282,6 +266,19 @@ __device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c) {
         : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
     return d;
 }
+__device__ __forceinline__ float2 f2_mul(float2 a, float2 b) {
+    float2 d;
+    asm("{\n .reg .b64 x, y, r;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %5};\n"
+        " mul.rn.f32x2 r, x, y;\n mov.b64 {%0, %1}, r;\n}\n"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+// the hardware reciprocal (within 1 ulp)
+__device__ __forceinline__ float rcp_hw(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 __device__ __forceinline__ float2 f2_dup(float a) { return make_float2(a, a); }
 
 // Lane arithmetic for the bound of one table (float) or two tables at once (float2, f32x2
@@ -293,6 +290,11 @@ struct LaneOps1 {
     static __device__ __forceinline__ T fma(T a, T b, T c) { return __fmaf_rn(a, b, c); }
     static __device__ __forceinline__ T lg(T a) { return lg2_hw(a); }
     static __device__ __forceinline__ T dup(float a) { return a; }
+    static __device__ __forceinline__ T mul(T a, T b) { return __fmul_rn(a, b); }
+    static __device__ __forceinline__ T nrcp(T a) { return rcp_hw(-a); }
+    // a row constant (stored twice), one triplet's half of a pair
+    static __device__ __forceinline__ T two(float a, float) { return a; }
+    static __device__ __forceinline__ T pick(float2 a, int m) { return m ? a.y : a.x; }
 };
 struct LaneOps2 {
     typedef float2 T;
@@ -301,82 +303,11 @@ struct LaneOps2 {
     static __device__ __forceinline__ T fma(T a, T b, T c) { return f2_fma(a, b, c); }
     static __device__ __forceinline__ T lg(T a) { return make_float2(lg2_hw(a.x), lg2_hw(a.y)); }
     static __device__ __forceinline__ T dup(float a) { return f2_dup(a); }
+    static __device__ __forceinline__ T mul(T a, T b) { return f2_mul(a, b); }
+    static __device__ __forceinline__ T nrcp(T a) { return make_float2(rcp_hw(-a.x), rcp_hw(-a.y)); }
+    static __device__ __forceinline__ T two(float a, float b) { return make_float2(a, b); }
+    static __device__ __forceinline__ T pick(float2 a, int) { return a; }
 };
-
-// The table-free bound (k2_bound_u's terms) with both classes' cells derived on the fly (the
-// operations of cells_u, per class), each cell's three terms chained as soon as both classes'
-// values are known: no 27-cell array is ever live.  n8[c][4 a + 2 b + z] = count + 1 of the
-// counted cells, xz[c][a][z] / yz[c][b][z] = pair-table entries + 3, mz[c][z] = marginal of Z
-// + 9, rc[c] = the row cells of class c.  Cells enter the two chains in derivation order; the
-// bound's error analysis (every finished cell adds a positive amount; 82 roundings of at most
-// 2^-24 of the largest partial sum) holds for any order.
-template <class L>
-__device__ __forceinline__ typename L::T k2_bound_cells(const typename L::T (*n8)[8],
-                                                        const RowCells* rc,
-                                                        const typename L::T (*xz)[2][2],
-                                                        const typename L::T (*yz)[2][2],
-                                                        const typename L::T (*mz)[2]) {
-    typedef typename L::T T;
-    T acc[2] = {L::dup(0.f), L::dup(0.f)};
-    const T half = L::dup(0.5f);
-    auto term = [&](int q, T u0, T u1) {
-        T& a = acc[q & 1];
-        const T us = L::add(u0, u1);
-        a = L::fma(L::sub(us, half), L::lg(us), a);
-        a = L::fma(L::sub(half, u0), L::lg(u0), a);
-        a = L::fma(L::sub(half, u1), L::lg(u1), a);
-    };
-    auto d2 = [&](T x, T y, T z) { return L::sub(L::sub(x, y), z); };
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const int e = 4 * a + 2 * b;
-            term(9 * a + 3 * b, n8[0][e], n8[1][e]);
-            term(9 * a + 3 * b + 1, n8[0][e + 1], n8[1][e + 1]);
-            term(9 * a + 3 * b + 2, d2(L::dup(rc[0].xy[2 * a + b]), n8[0][e], n8[0][e + 1]),
-                 d2(L::dup(rc[1].xy[2 * a + b]), n8[1][e], n8[1][e + 1]));
-        }
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-        T a2z[2][2];  // [class][z]
-#pragma unroll
-        for (int z = 0; z < 2; ++z) {
-#pragma unroll
-            for (int c = 0; c < 2; ++c) a2z[c][z] = d2(xz[c][a][z], n8[c][4 * a + z], n8[c][4 * a + 2 + z]);
-            term(9 * a + 6 + z, a2z[0][z], a2z[1][z]);
-        }
-        term(9 * a + 8, d2(L::dup(rc[0].xa2[a]), a2z[0][0], a2z[0][1]),
-             d2(L::dup(rc[1].xa2[a]), a2z[1][0], a2z[1][1]));
-    }
-    T c2bz[2][2][2];  // [class][b][z]
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-#pragma unroll
-        for (int z = 0; z < 2; ++z) {
-#pragma unroll
-            for (int c = 0; c < 2; ++c) c2bz[c][b][z] = d2(yz[c][b][z], n8[c][2 * b + z], n8[c][4 + 2 * b + z]);
-            term(18 + 3 * b + z, c2bz[0][b][z], c2bz[1][b][z]);
-        }
-        term(18 + 3 * b + 2, d2(L::dup(rc[0].x2b[b]), c2bz[0][b][0], c2bz[0][b][1]),
-             d2(L::dup(rc[1].x2b[b]), c2bz[1][b][0], c2bz[1][b][1]));
-    }
-    T c22z[2][2];  // [class][z]
-#pragma unroll
-    for (int z = 0; z < 2; ++z) {
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const T z2 = d2(mz[c][z], xz[c][0][z], xz[c][1][z]);   // #(X = 2, Z = z) + 3
-            c22z[c][z] = d2(z2, c2bz[c][0][z], c2bz[c][1][z]);
-        }
-        term(24 + z, c22z[0][z], c22z[1][z]);
-    }
-    term(26, d2(L::dup(rc[0].c22), c22z[0][0], c22z[0][1]), d2(L::dup(rc[1].c22), c22z[1][0], c22z[1][1]));
-    return L::add(acc[0], acc[1]);  // in log2 units, before the final scale and offset
-}
-__device__ __forceinline__ float k2_bound_finish(float s) {
-    return __fmaf_rn(0.6931471805599453f, s, -27.f * 0.9189385332046727f);
-}
 
 // Exact integer cells r = u - 1 of both classes; false unless every cell lies in [0, N_c]
 // (which keeps every log-factorial lookup of the table in range).
@@ -416,11 +347,12 @@ __device__ __forceinline__ bool epi_sync_or(bool p) {
 constexpr int kCandCap = 1024;               // per-CTA candidate buffer (power of two)
 constexpr int kPruneAt = kCandCap / 2;       // local candidates that trigger a prune
 
+// Ascending bitonic sort of the buffer's first n entries (a power of two).
 template <int kThreads>
-__device__ void sort_cands(Cand* buf, int tid) {
-    for (int size = 2; size <= kCandCap; size <<= 1)
+__device__ void sort_cands(Cand* buf, int n, int tid) {
+    for (int size = 2; size <= n; size <<= 1)
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int t = tid; t < kCandCap / 2; t += kThreads) {
+            for (int t = tid; t < n / 2; t += kThreads) {
                 const int lo = 2 * t - (t & (stride - 1));
                 const int hi = lo + stride;
                 const bool up = ((lo & size) == 0);
@@ -447,9 +379,11 @@ template <int kThreads>
 __device__ int epi_prune(const CohortDev& a, EpiShared& es, int cnt, int tid, bool final_flush) {
     const float kInf = __int_as_float(0x7f800000);
     if (cnt >= a.top_k) {
-        for (int idx = cnt + tid; idx < kCandCap; idx += kThreads) es.buf[idx].s = kInf;
+        int n2 = 32;
+        while (n2 < cnt) n2 <<= 1;
+        for (int idx = cnt + tid; idx < n2; idx += kThreads) es.buf[idx].s = kInf;
         epi_sync<kThreads>();
-        sort_cands<kThreads>(es.buf, tid);
+        sort_cands<kThreads>(es.buf, n2, tid);
         if (tid == 0) {
             const float tl = band_threshold(es.buf[a.top_k - 1].s, a.k2.rel, a.k2.abs_);
             atomicMin(&a.ctrl->thr, __float_as_uint(tl));
