@@ -1450,23 +1450,44 @@ int epi3_scan_order(epi3_handle* h, int32_t order, int32_t top_k, int32_t* out_s
     if (sel > (size_t)4 << 30)
         return fail(EPI3_ERR_UNSUPPORTED, "%d-SNP scan of %d SNPs with top_k %d needs %zu bytes of "
                     "selection scratch (limit 4 GiB)", order, h->M, top_k, sel);
-    const size_t need = sel + sizeof(double) * (size_t)top_k + sizeof(int32_t) * order * (size_t)top_k;
-    if (h->pair_scratch_bytes < need) {
+    const size_t outs = sizeof(double) * (size_t)top_k + sizeof(int32_t) * order * (size_t)top_k;
+    auto scratch = [&](size_t bytes) -> int {   // kept on the handle; outputs after the first `bytes`
+        if (h->pair_scratch_bytes >= bytes + outs) return EPI3_OK;
         dev_free(h->d_pair_scratch);
         h->d_pair_scratch = nullptr;
         h->pair_scratch_bytes = 0;
-        CK(dev_alloc(&h->d_pair_scratch, need), "alloc k-SNP scan scratch");
-        h->pair_scratch_bytes = need;
-    }
-    double* d_s = reinterpret_cast<double*>(static_cast<char*>(h->d_pair_scratch) + sel);
-    int32_t* d_sets = reinterpret_cast<int32_t*>(d_s + top_k);
+        CK(dev_alloc(&h->d_pair_scratch, bytes + outs), "alloc k-SNP scan scratch");
+        h->pair_scratch_bytes = bytes + outs;
+        return EPI3_OK;
+    };
+    double* d_s = nullptr;
+    int32_t* d_sets = nullptr;
+    auto place = [&](size_t bytes) {
+        d_s = reinterpret_cast<double*>(static_cast<char*>(h->d_pair_scratch) + bytes);
+        d_sets = reinterpret_cast<int32_t*>(d_s + top_k);
+    };
     CK(cudaEventRecord(h->ev[0], h->stream), "event");
-    if (order == 4)
-        CK(launch_quad_scan(h->pl, h->k2.lf64, h->N0, h->N1, top_k, h->d_pair_scratch, d_sets, d_s,
-                            h->stream), "four-SNP scan launch");
-    else
-        CK(launch_order_scan(h->pl, h->k2.lf64, order, top_k, h->d_pair_scratch, d_sets, d_s, h->stream),
-           "k-SNP scan launch");
+    // the counted form, unless its tables are too large (or there is no memory for them) or more
+    // sets tie at the k-th score than it rescores; then the direct form
+    bool done = false;
+    const size_t cnt = set_scan_scratch(h->M, h->N, order);
+    if (cnt && scratch(cnt) == EPI3_OK) {
+        place(cnt);
+        CK(launch_set_scan(h->pl, h->k2.lf64, h->N0, h->N1, order, top_k, h->sm_count, h->d_pair_scratch,
+                           h->h_ctrl, d_sets, d_s, &done, h->stream), "k-SNP scan launch");
+    }
+    if (!done) {
+        g_err.clear();
+        const int rc = scratch(sel);
+        if (rc != EPI3_OK) return rc;
+        place(sel);
+        if (order == 4)
+            CK(launch_quad_scan(h->pl, h->k2.lf64, h->N0, h->N1, top_k, h->d_pair_scratch, d_sets, d_s,
+                                h->stream), "four-SNP scan launch");
+        else
+            CK(launch_order_scan(h->pl, h->k2.lf64, order, top_k, h->d_pair_scratch, d_sets, d_s, h->stream),
+               "k-SNP scan launch");
+    }
     CK(cudaEventRecord(h->ev[1], h->stream), "event");
     const cudaMemcpyKind kind =
         (h->flags & EPI3_DEVICE_PTRS) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;

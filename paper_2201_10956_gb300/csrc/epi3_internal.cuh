@@ -132,6 +132,13 @@ long long order_count(int M, int order);
 size_t order_scan_scratch(int M, int order, int k);
 cudaError_t launch_order_scan(const Planes& pl, const double* lf64, int order, int k, void* scratch,
                               int32_t* out_snps, double* out_s, cudaStream_t st);
+// The counted form of orders 4 to 6: scratch bytes (0: not for this size); *done false: more sets tie
+// at the k-th score than it rescores (the direct form answers).  Reads a few words back into h_ctrl
+// (pinned, at least 16 bytes) and synchronises.
+size_t set_scan_scratch(int M, int N, int order);
+cudaError_t launch_set_scan(const Planes& pl, const double* lf64, int n0, int n1, int order, int k, int sms,
+                            void* scratch, void* h_ctrl, int32_t* out_snps, double* out_s, bool* done,
+                            cudaStream_t st);
 long long quad_count(int M);
 size_t quad_scan_scratch(int M, int k);
 cudaError_t launch_quad_scan(const Planes& pl, const double* lf64, int n0, int n1, int k,

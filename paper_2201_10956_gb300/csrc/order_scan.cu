@@ -17,9 +17,20 @@
 // the FP64 K2 is summed in cell order 0..80 (cell = 27 g_i + 9 g_j + 3 g_k + g_l) like the
 // pairs.  The sets are enumerated in colexicographic order from a linear index.
 //
-// Selection (both): each block scores 2048 consecutive items and keeps its k best (bitonic
+// Orders four to six, the counted form (launch_set_scan): every set is first scored in FP32 from its
+// exact table, and only the sets within that score's error of the k-th best are counted again and
+// scored in FP64.  A thread counts the 2^K cells with genotypes 0 and 1 of its set (AND + POPC) and
+// gets the other 3^K - 2^K from the same counts of all smaller sets, by
+//     #(.., 2, ..) = #(.., any, ..) - #(.., 0, ..) - #(.., 1, ..),
+// both classes in one register and one three-input subtraction per cell.  The direct forms below
+// (81, 243 or 729 cells counted, every set scored in FP64) serve what the counted form refuses:
+// tables of the smaller sets past kSubsetBytes, or more sets tied at the k-th score than it rescores.
+//
+// Selection (pairs and the direct forms): each block scores 2048 consecutive items and keeps its k best (bitonic
 // sort in shared memory); further passes merge 2048 survivors per block until one block
 // remains.  Ties are ordered by a key that sorts like the SNP indices.
+#include <cmath>
+
 #include "epi3_internal.cuh"
 
 namespace epi3 {
@@ -295,15 +306,11 @@ __device__ inline void decode_lex(long long q, int M, int* x) {
         }
 }
 
+// Genotype codes of the cells a lane owns (2 bits per SNP: the genotype of x_t at bits 2 t).
 template <int K>
-__global__ void __launch_bounds__(kOrdThreads)
-order_score_kernel(Planes pl, const double* __restrict__ lf64, long long n_sets, int k,
-                   Item* __restrict__ out) {
+__device__ __forceinline__ void lane_codes(uint32_t* code) {
     constexpr int kCellsK = Pow3<K>::v, kPer = (kCellsK + 31) / 32;
-    __shared__ Item it[kPairBlock];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int M = pl.M;
-    uint32_t code[kPer];   // 2 bits per SNP: the genotype of x_t at bits 2 t
+    const int lane = threadIdx.x & 31;
 #pragma unroll
     for (int m = 0; m < kPer; ++m) {
         int e = lane + 32 * m < kCellsK ? lane + 32 * m : 0;
@@ -315,6 +322,82 @@ order_score_kernel(Planes pl, const double* __restrict__ lf64, long long n_sets,
         }
         code[m] = cd;
     }
+}
+
+// FP64 K2 of one set by one warp (every lane returns it).
+template <int K>
+__device__ double set_score(const Planes& pl, const double* __restrict__ lf64, const int* x,
+                            const uint32_t* code) {
+    constexpr int kCellsK = Pow3<K>::v, kPer = (kCellsK + 31) / 32;
+    const int lane = threadIdx.x & 31;
+    const int M = pl.M;
+    uint32_t cnt[kPer];
+#pragma unroll
+    for (int m = 0; m < kPer; ++m) cnt[m] = 0u;
+#pragma unroll 1
+    for (int c = 0; c < 2; ++c) {
+        const long long coff = c ? pl.coff[1] : pl.coff[0];
+        const int W4 = c ? pl.W4[1] : pl.W4[0];
+        const int sh = 16 * c;
+#pragma unroll 1
+        for (int w4 = 0; w4 < W4; ++w4) {
+            uint4 g0[K], g1[K];
+#pragma unroll
+            for (int v = 0; v < K; ++v) {
+                g0[v] = __ldg(pl.planes + coff + (size_t)w4 * M + x[v]);
+                g1[v] = __ldg(pl.planes + coff + (size_t)(W4 + w4) * M + x[v]);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                uint32_t P[K][3];
+#pragma unroll
+                for (int v = 0; v < K; ++v) {
+                    const uint32_t a0 = e == 0 ? g0[v].x : e == 1 ? g0[v].y : e == 2 ? g0[v].z : g0[v].w;
+                    const uint32_t a1 = e == 0 ? g1[v].x : e == 1 ? g1[v].y : e == 2 ? g1[v].z : g1[v].w;
+                    P[v][0] = a0;
+                    P[v][1] = a1;
+                    P[v][2] = ~(a0 | a1);        // genotype 2, Sec. IV-A (pad bits read 2)
+                }
+#pragma unroll
+                for (int m = 0; m < kPer; ++m) {
+                    uint32_t acc = 0xFFFFFFFFu;
+#pragma unroll
+                    for (int v = 0; v < K; ++v) {
+                        const uint32_t g = (code[m] >> (2 * v)) & 3u;
+                        acc &= g == 0u ? P[v][0] : (g == 1u ? P[v][1] : P[v][2]);
+                    }
+                    cnt[m] += (uint32_t)__popc(acc) << sh;
+                }
+            }
+        }
+    }
+    // pad samples read genotype 2 in every SNP: the last cell only
+    if (lane == (kCellsK - 1) % 32)
+        cnt[(kCellsK - 1) / 32] -= (uint32_t)pl.pad[0] + ((uint32_t)pl.pad[1] << 16);
+    double term[kPer];
+#pragma unroll
+    for (int m = 0; m < kPer; ++m) {
+        const int r0 = (int)(cnt[m] & 0xFFFFu), r1 = (int)(cnt[m] >> 16);
+        term[m] = lane + 32 * m < kCellsK
+                      ? __dsub_rn(__dsub_rn(lf64[r0 + r1 + 1], lf64[r0]), lf64[r1]) : 0.0;
+    }
+    double sc = 0.0;
+#pragma unroll
+    for (int m = 0; m < kPer; ++m)
+#pragma unroll
+        for (int l = 0; l < 32; ++l)
+            if (32 * m + l < kCellsK) sc = __dadd_rn(sc, __shfl_sync(0xffffffffu, term[m], l));
+    return sc;
+}
+
+template <int K>
+__global__ void __launch_bounds__(kOrdThreads)
+order_score_kernel(Planes pl, const double* __restrict__ lf64, long long n_sets, int k,
+                   Item* __restrict__ out) {
+    __shared__ Item it[kPairBlock];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t code[(Pow3<K>::v + 31) / 32];
+    lane_codes<K>(code);
     const long long q0 = (long long)blockIdx.x * kPairBlock;
     for (int t = warp; t < kPairBlock; t += kOrdThreads / 32) {
         const long long q = q0 + t;
@@ -323,63 +406,8 @@ order_score_kernel(Planes pl, const double* __restrict__ lf64, long long n_sets,
             continue;
         }
         int x[K];
-        decode_lex<K>(q, M, x);
-        uint32_t cnt[kPer];
-#pragma unroll
-        for (int m = 0; m < kPer; ++m) cnt[m] = 0u;
-#pragma unroll 1
-        for (int c = 0; c < 2; ++c) {
-            const long long coff = c ? pl.coff[1] : pl.coff[0];
-            const int W4 = c ? pl.W4[1] : pl.W4[0];
-            const int sh = 16 * c;
-#pragma unroll 1
-            for (int w4 = 0; w4 < W4; ++w4) {
-                uint4 g0[K], g1[K];
-#pragma unroll
-                for (int v = 0; v < K; ++v) {
-                    g0[v] = __ldg(pl.planes + coff + (size_t)w4 * M + x[v]);
-                    g1[v] = __ldg(pl.planes + coff + (size_t)(W4 + w4) * M + x[v]);
-                }
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    uint32_t P[K][3];
-#pragma unroll
-                    for (int v = 0; v < K; ++v) {
-                        const uint32_t a0 = e == 0 ? g0[v].x : e == 1 ? g0[v].y : e == 2 ? g0[v].z : g0[v].w;
-                        const uint32_t a1 = e == 0 ? g1[v].x : e == 1 ? g1[v].y : e == 2 ? g1[v].z : g1[v].w;
-                        P[v][0] = a0;
-                        P[v][1] = a1;
-                        P[v][2] = ~(a0 | a1);        // genotype 2, Sec. IV-A (pad bits read 2)
-                    }
-#pragma unroll
-                    for (int m = 0; m < kPer; ++m) {
-                        uint32_t acc = 0xFFFFFFFFu;
-#pragma unroll
-                        for (int v = 0; v < K; ++v) {
-                            const uint32_t g = (code[m] >> (2 * v)) & 3u;
-                            acc &= g == 0u ? P[v][0] : (g == 1u ? P[v][1] : P[v][2]);
-                        }
-                        cnt[m] += (uint32_t)__popc(acc) << sh;
-                    }
-                }
-            }
-        }
-        // pad samples read genotype 2 in every SNP: the last cell only
-        if (lane == (kCellsK - 1) % 32)
-            cnt[(kCellsK - 1) / 32] -= (uint32_t)pl.pad[0] + ((uint32_t)pl.pad[1] << 16);
-        double term[kPer];
-#pragma unroll
-        for (int m = 0; m < kPer; ++m) {
-            const int r0 = (int)(cnt[m] & 0xFFFFu), r1 = (int)(cnt[m] >> 16);
-            term[m] = lane + 32 * m < kCellsK
-                          ? __dsub_rn(__dsub_rn(lf64[r0 + r1 + 1], lf64[r0]), lf64[r1]) : 0.0;
-        }
-        double sc = 0.0;
-#pragma unroll
-        for (int m = 0; m < kPer; ++m)
-#pragma unroll
-            for (int l = 0; l < 32; ++l)
-                if (32 * m + l < kCellsK) sc = __dadd_rn(sc, __shfl_sync(0xffffffffu, term[m], l));
+        decode_lex<K>(q, pl.M, x);
+        const double sc = set_score<K>(pl, lf64, x, code);
         if (lane == 0) it[t] = Item{sc, q};
     }
     __syncthreads();
@@ -424,7 +452,536 @@ cudaError_t order_scan_k(const Planes& pl, const double* lf64, int k, void* scra
     return cudaGetLastError();
 }
 
+
+// ---------------------------------------------------------------- four to six SNPs, counted form
+// Sets are numbered in colexicographic order here: {y_1 < ... < y_t} has rank sum of C(y_s, s).  The
+// counts of every set of t = 1 .. K - 1 SNPs lie at sub[t] + 2^t rank + (genotypes as bits, the
+// smallest SNP's the highest): class 0's count in the low half, class 1's in the high half.
+struct SetArgs {
+    Planes pl;
+    const long long* binom;      // [7][M + 1]: C(x, t)
+    const float* lf;             // [N + 2]
+    int n_lf;
+    uint32_t* sub[6];            // by set size
+    uint32_t total;              // class sizes, packed
+    long long n_sets;
+};
+struct SetCand {
+    long long q;                 // rank
+    float s;
+};
+struct SetCtrl {
+    float thr;
+    unsigned n_cand, n_final;
+};
+
+__device__ __forceinline__ long long binom_at(const SetArgs& a, int x, int t) {
+    return __ldg(a.binom + (size_t)t * (a.pl.M + 1) + x);
+}
+// The set of rank q, ascending.
+template <int T>
+__device__ __forceinline__ void decode_colex(const SetArgs& a, long long q, int* x) {
+    int hi = a.pl.M;
+#pragma unroll
+    for (int t = T; t >= 1; --t) {
+        int lo = t - 1;          // C(t - 1, t) = 0
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (binom_at(a, mid, t) <= q) lo = mid;
+            else hi = mid;
+        }
+        q -= binom_at(a, lo, t);
+        x[t - 1] = lo;
+        hi = lo;
+    }
+}
+
+__global__ void set_tables_kernel(int M, const double* __restrict__ lf64, int n_lf,
+                                  long long* __restrict__ binom, float* __restrict__ lf) {
+    const int n = blockDim.x * gridDim.x, id = blockIdx.x * blockDim.x + threadIdx.x;
+    for (int e = id; e < 7 * (M + 1); e += n) binom[e] = choose_ll(e % (M + 1), e / (M + 1));
+    for (int e = id; e < n_lf; e += n) lf[e] = (float)lf64[e];
+}
+
+// Counts of the cells of x with genotypes 0 and 1, packed; cnt[bits], x[0] the highest bit.
+template <int T>
+__device__ __forceinline__ void count_cells(const Planes& pl, const int* x, uint32_t* cnt) {
+    const int M = pl.M;
+#pragma unroll
+    for (int e = 0; e < (1 << T); ++e) cnt[e] = 0u;
+#pragma unroll 1
+    for (int c = 1; c >= 0; --c) {
+        const uint4* const base = pl.planes + (c ? pl.coff[1] : pl.coff[0]);
+        const int W4 = c ? pl.W4[1] : pl.W4[0];
+#pragma unroll 1
+        for (int w4 = 0; w4 < W4; ++w4) {
+            uint4 g[T][2];
+#pragma unroll
+            for (int v = 0; v < T; ++v) {
+                g[v][0] = __ldg(base + (size_t)w4 * M + x[v]);
+                g[v][1] = __ldg(base + (size_t)(W4 + w4) * M + x[v]);
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                uint32_t p[1 << T];
+                p[0] = 0xFFFFFFFFu;
+#pragma unroll
+                for (int v = 0; v < T; ++v) {
+                    const uint32_t a0 = e == 0 ? g[v][0].x : e == 1 ? g[v][0].y : e == 2 ? g[v][0].z : g[v][0].w;
+                    const uint32_t a1 = e == 0 ? g[v][1].x : e == 1 ? g[v][1].y : e == 2 ? g[v][1].z : g[v][1].w;
+#pragma unroll
+                    for (int b = (1 << v) - 1; b >= 0; --b) {
+                        p[2 * b + 1] = p[b] & a1;
+                        p[2 * b] = p[b] & a0;
+                    }
+                }
+#pragma unroll
+                for (int b = 0; b < (1 << T); ++b) cnt[b] += (uint32_t)__popc(p[b]);
+            }
+        }
+        if (c == 1)
+#pragma unroll
+            for (int e = 0; e < (1 << T); ++e) cnt[e] <<= 16;
+    }
+}
+
+template <int T>
+__global__ void __launch_bounds__(128) set_count_kernel(const SetArgs a, long long n_sets) {
+    for (long long q = (long long)blockIdx.x * 128 + threadIdx.x; q < n_sets; q += (long long)gridDim.x * 128) {
+        int x[T];
+        decode_colex<T>(a, q, x);
+        uint32_t cnt[1 << T];
+        count_cells<T>(a.pl, x, cnt);
+        uint32_t* const o = a.sub[T] + (q << T);
+#pragma unroll
+        for (int e = 0; e < (1 << T); ++e) o[e] = cnt[e];
+    }
+}
+
+// #(positions of the set in `mask` have the genotypes of `bits`, the others any), packed, for the 2^n
+// lowest of those positions' bits (out): the table of that subset, or this set's own counts.
+// Bit K - 1 - p of mask and bits stands for position p.
+template <int K, int NLOW>
+__device__ __forceinline__ void subset_counts(const SetArgs& a, const int* x, const uint32_t* own,
+                                              int mask, int bits, uint32_t* out) {
+    // mask, bits and NLOW are compile-time constants after unrolling
+    if (mask == (1 << K) - 1) {
+#pragma unroll
+        for (int e = 0; e < (1 << NLOW); ++e) out[e] = own[bits + e];
+        return;
+    }
+    if (mask == 0) {
+        out[0] = a.total;
+        return;
+    }
+    long long rank = 0;
+    int t = 0, idx = 0;
+#pragma unroll
+    for (int p = 0; p < K; ++p)
+        if (mask & (1 << (K - 1 - p))) {
+            ++t;
+            rank += binom_at(a, x[p], t);
+            idx = 2 * idx + ((bits >> (K - 1 - p)) & 1);
+        }
+    const uint32_t* const src = a.sub[t] + (rank << t) + idx;
+    if (NLOW == 0) out[0] = __ldg(src);
+    if (NLOW == 1) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2*>(src));
+        out[0] = v.x;
+        out[1] = v.y;
+    }
+    if (NLOW >= 2) {
+#pragma unroll
+        for (int e = 0; e < (1 << NLOW); e += 4) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4*>(src + e));
+            out[e] = v.x;
+            out[e + 1] = v.y;
+            out[e + 2] = v.z;
+            out[e + 3] = v.w;
+        }
+    }
+}
+
+// The 27 cells over the last three positions (index 9 g + 3 h + i) with the positions before them as
+// mask / bits say, positions in mask2 with genotype 2 (each #any - #0 - #1).
+template <int K>
+__device__ __forceinline__ void inner_cells(const SetArgs& a, const int* x, const uint32_t* own,
+                                            int mask, int bits, uint32_t* g) {
+    // {0, 1, any}^3 first: any at digit 2
+    uint32_t v[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {   // which of the last three positions are fixed
+        constexpr int kStep[3] = {9, 3, 1};
+        const int n = (m & 1) + ((m >> 1) & 1) + (m >> 2);
+        if (n == 0) subset_counts<K, 0>(a, x, own, mask | m, bits, v);
+        else if (n == 1) subset_counts<K, 1>(a, x, own, mask | m, bits, v);
+        else if (n == 2) subset_counts<K, 2>(a, x, own, mask | m, bits, v);
+        else subset_counts<K, 3>(a, x, own, mask | m, bits, v);
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if (e < (1 << n)) {
+                int cell = 0, left = n;
+#pragma unroll
+                for (int p = 0; p < 3; ++p) {
+                    if (m & (4 >> p)) cell += ((e >> --left) & 1) * kStep[p];
+                    else cell += 2 * kStep[p];
+                }
+                g[cell] = v[e];
+            }
+    }
+#pragma unroll
+    for (int st = 1; st < 27; st *= 3)
+#pragma unroll
+        for (int e = 0; e < 27; ++e)
+            if ((e / st) % 3 == 2) g[e] = g[e] - g[e - st] - g[e - 2 * st];
+}
+
+// Inner cells with the outer positions' genotypes O (base-3 digits of the first K - 4 positions) and
+// position K - 4 fixed to mid (0, 1) or any (2).
+template <int K>
+__device__ __forceinline__ void outer_cells(const SetArgs& a, const int* x, const uint32_t* own, int outer,
+                                            int mid, uint32_t* g) {
+    // every outer position with genotype 2 expands into any - 0 - 1
+    int mask = 0, bits = 0, n2 = 0, pos2[2] = {0, 0};
+#pragma unroll
+    for (int p = 0; p < K - 4; ++p) {
+        const int d = p == K - 5 ? outer % 3 : outer / 3, bit = 1 << (K - 1 - p);
+        if (d == 2) pos2[n2++] = bit;
+        else {
+            mask |= bit;
+            bits |= d ? bit : 0;
+        }
+    }
+    if (mid < 2) {
+        mask |= 8;
+        bits |= mid ? 8 : 0;
+    }
+    inner_cells<K>(a, x, own, mask, bits, g);
+    uint32_t t[27];
+#pragma unroll
+    for (int c = 1; c < 9; ++c) {
+        const int c0 = c % 3, c1 = c / 3;   // per position with genotype 2: any, 0, 1
+        if (n2 < 2 && c1 > 0) continue;
+        if (n2 < 1) continue;
+        int mk = mask, bt = bits;
+        if (c0) {
+            mk |= pos2[0];
+            bt |= c0 == 2 ? pos2[0] : 0;
+        }
+        if (c1) {
+            mk |= pos2[1];
+            bt |= c1 == 2 ? pos2[1] : 0;
+        }
+        inner_cells<K>(a, x, own, mk, bt, t);
+        const bool minus = ((c0 != 0) != (c1 != 0));
+#pragma unroll
+        for (int e = 0; e < 27; ++e) g[e] = minus ? g[e] - t[e] : g[e] + t[e];
+    }
+}
+
+// Adds the 27 cells' K2 terms in FP32.
+__device__ __forceinline__ float add_terms(const float* lf, const uint32_t* g, float s) {
+#pragma unroll
+    for (int e = 0; e < 27; ++e) {
+        const uint32_t r0 = g[e] & 0xFFFFu, r1 = g[e] >> 16;
+        s += (lf[r0 + r1 + 1] - lf[r0]) - lf[r1];
+    }
+    return s;
+}
+
+// FP32 scores of all sets (or of every stride-th one into `sample`); those at or below the threshold
+// go to the candidate list.  Bound by POPC (2^K a word and set); the lookups of the score come from
+// shared memory where the table fits (kSmemLf).
+constexpr int kSetThreads = 128;
+constexpr int kSetLfMax = 12288;         // log-factorials in shared memory, at most
+template <int K, bool kSmemLf>
+__global__ void __launch_bounds__(kSetThreads)
+set_scan_kernel(const SetArgs a, long long stride, long long n, float* __restrict__ sample,
+                SetCtrl* ctrl, SetCand* __restrict__ cand, unsigned cap) {
+    extern __shared__ float s_lf[];
+    if (kSmemLf) {
+        for (int e = threadIdx.x; e < a.n_lf; e += kSetThreads) s_lf[e] = a.lf[e];
+        __syncthreads();
+    }
+    const float* const lf = kSmemLf ? s_lf : a.lf;
+    const float thr = sample ? 0.f : ctrl->thr;
+    for (long long t = (long long)blockIdx.x * kSetThreads + threadIdx.x; t < n;
+         t += (long long)gridDim.x * kSetThreads) {
+        const long long q = t * stride;
+        int x[K];
+        decode_colex<K>(a, q, x);
+        uint32_t own[1 << K];
+        count_cells<K>(a.pl, x, own);
+        float s = 0.f;
+#pragma unroll 1
+        for (int outer = 0; outer < (K == 4 ? 1 : K == 5 ? 3 : 9); ++outer) {
+            // position K - 4: genotypes 0 and 1, then 2 as what is left of any
+            uint32_t any[27], g[27];
+            auto step = [&](int o) {
+                outer_cells<K>(a, x, own, o, 2, any);
+#pragma unroll
+                for (int mid = 0; mid < 2; ++mid) {
+                    outer_cells<K>(a, x, own, o, mid, g);
+                    s = add_terms(lf, g, s);
+#pragma unroll
+                    for (int e = 0; e < 27; ++e) any[e] -= g[e];
+                }
+                s = add_terms(lf, any, s);
+            };
+            if (K == 4) step(0);
+            else if (K == 5) {
+                if (outer == 0) step(0);
+                else if (outer == 1) step(1);
+                else step(2);
+            } else {
+                switch (outer) {
+                    case 0: step(0); break;
+                    case 1: step(1); break;
+                    case 2: step(2); break;
+                    case 3: step(3); break;
+                    case 4: step(4); break;
+                    case 5: step(5); break;
+                    case 6: step(6); break;
+                    case 7: step(7); break;
+                    default: step(8); break;
+                }
+            }
+        }
+        s = fmaxf(s, 0.f);
+        if (sample) {
+            sample[t] = s;
+        } else if (s <= thr) {
+            const unsigned pos = atomicAdd(&ctrl->n_cand, 1u);
+            if (pos < cap) cand[pos] = SetCand{q, s};
+        }
+    }
+}
+
+// The k-th smallest score (scores are not negative: their bit patterns sort like them) of n floats
+// `step` floats apart; ctrl->thr becomes that + 2 delta, rounded up: no set of the answer scores
+// higher.  One block.
+__global__ void __launch_bounds__(1024)
+set_threshold_kernel(const float* __restrict__ v, int step, long long n, const unsigned* __restrict__ n_dev,
+                     int k, float delta, SetCtrl* ctrl) {
+    __shared__ unsigned hist[256];
+    __shared__ unsigned s_prefix, s_rank;
+    if (n_dev) n = min(n, (long long)*n_dev);
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid == 0) {
+        s_prefix = 0u;
+        s_rank = (unsigned)k;
+    }
+    unsigned mask = 0u;
+    for (int shift = 24; shift >= 0; shift -= 8) {
+        for (int b = tid; b < 256; b += 1024) hist[b] = 0u;
+        __syncthreads();
+        const unsigned prefix = s_prefix, rank = s_rank;
+        for (long long e = tid; e < n; e += 1024) {
+            const unsigned u = __float_as_uint(v[e * step]);
+            if ((u & mask) == prefix) atomicAdd(&hist[(u >> shift) & 255u], 1u);
+        }
+        __syncthreads();
+        if (tid < 32) {   // the bin that holds the rank: eight bins a lane
+            unsigned c[8], sum = 0u;
+#pragma unroll
+            for (int b = 0; b < 8; ++b) sum += c[b] = hist[8 * lane + b];
+            unsigned incl = sum;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const unsigned o = __shfl_up_sync(0xffffffffu, incl, d);
+                if (lane >= d) incl += o;
+            }
+            unsigned before = incl - sum;
+            if (before < rank && rank <= incl) {
+                int b = 0;
+                while (before + c[b] < rank) before += c[b++];
+                s_rank = rank - before;
+                s_prefix = prefix | ((unsigned)(8 * lane + b) << shift);
+            }
+        }
+        mask |= 255u << shift;
+        __syncthreads();
+    }
+    if (tid == 0) {
+        ctrl->thr = __fadd_ru(__uint_as_float(s_prefix), 2.f * delta);
+        if (!n_dev) ctrl->n_cand = 0u;
+        ctrl->n_final = 0u;
+    }
+}
+
+// FP64 scores of the candidates inside the threshold, one warp each.
+template <int K>
+__global__ void __launch_bounds__(kOrdThreads)
+set_rescore_kernel(const SetArgs a, const double* __restrict__ lf64, SetCtrl* ctrl,
+                   const SetCand* __restrict__ cand, unsigned cap, Item* __restrict__ fin, unsigned fin_cap) {
+    uint32_t code[(Pow3<K>::v + 31) / 32];
+    lane_codes<K>(code);
+    const unsigned n = min(ctrl->n_cand, cap);
+    const float thr = ctrl->thr;
+    const int M = a.pl.M;
+    for (unsigned e = blockIdx.x * (kOrdThreads / 32) + (threadIdx.x >> 5); e < n;
+         e += gridDim.x * (kOrdThreads / 32)) {
+        const SetCand cd = cand[e];
+        if (!(cd.s <= thr)) continue;
+        int x[K];
+        decode_colex<K>(a, cd.q, x);
+        const double sc = set_score<K>(a.pl, lf64, x, code);
+        if ((threadIdx.x & 31) == 0) {
+            const unsigned pos = atomicAdd(&ctrl->n_final, 1u);
+            long long lex = a.n_sets - 1;      // rank in lexicographic order, the tie key
+#pragma unroll
+            for (int t = 0; t < K; ++t) lex -= binom_at(a, M - 1 - x[t], K - t);
+            if (pos < fin_cap) fin[pos] = Item{sc, lex};
+        }
+    }
+}
+
+// The k best of at most kPairBlock rescored sets, sorted.
+__global__ void __launch_bounds__(kPairThreads)
+set_final_kernel(const SetCtrl* ctrl, const Item* __restrict__ fin, int k, Item* __restrict__ out) {
+    __shared__ Item it[kPairBlock];
+    const int n = min(ctrl->n_final, (unsigned)kPairBlock);
+    for (int t = threadIdx.x; t < kPairBlock; t += kPairThreads) it[t] = t < n ? fin[t] : pad_item();
+    __syncthreads();
+    sort_items(it);
+    for (int t = threadIdx.x; t < k; t += kPairThreads) out[t] = it[t];
+}
+
+constexpr unsigned kSetCand = 1u << 18;          // candidate list
+constexpr size_t kSubsetBytes = (size_t)16 << 30;   // counts of the smaller sets, at most
+
+struct SetLayout {
+    size_t binom, lf, ctrl, cand, fin, best, sample, sub[6], total;
+    long long n_sample;
+};
+SetLayout set_layout(int M, int N, int order) {
+    SetLayout L{};
+    size_t o = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = o;
+        o += (bytes + 255) & ~(size_t)255;
+        return at;
+    };
+    const long long n = choose_ll(M, order);
+    L.n_sample = n / 256 < 16384 ? (n < 16384 ? n : 16384) : n / 256 < 262144 ? n / 256 : 262144;
+    L.binom = take(sizeof(long long) * 7 * ((size_t)M + 1));
+    L.lf = take(sizeof(float) * ((size_t)N + 2));
+    L.ctrl = take(sizeof(SetCtrl));
+    L.cand = take(sizeof(SetCand) * kSetCand);
+    L.fin = take(sizeof(Item) * kPairBlock);
+    L.best = take(sizeof(Item) * EPI3_MAX_TOPK);
+    L.sample = take(sizeof(float) * (size_t)L.n_sample);
+    for (int t = 1; t < order; ++t) L.sub[t] = take((sizeof(uint32_t) << t) * (size_t)choose_ll(M, t));
+    L.total = o;
+    return L;
+}
+
+template <int T>
+cudaError_t count_subsets(const SetArgs& a, int grid, cudaStream_t st) {
+    const long long n = choose_ll(a.pl.M, T);
+    const long long blocks = (n + 127) / 128;
+    set_count_kernel<T><<<(unsigned)(blocks < grid ? blocks : grid), 128, 0, st>>>(a, n);
+    return cudaGetLastError();
+}
+
+template <int K>
+cudaError_t set_scan_k(const SetArgs& a, const SetLayout& L, const double* lf64, int sms, int k, float delta,
+                       char* base, SetCtrl* h_ctrl, int32_t* out_snps, double* out_s, bool* done,
+                       cudaStream_t st) {
+    *done = false;
+    const bool smem = a.n_lf <= kSetLfMax;
+    const size_t bytes = smem ? sizeof(float) * (size_t)a.n_lf : 0;
+    SetCtrl* const ctrl = reinterpret_cast<SetCtrl*>(base + L.ctrl);
+    SetCand* const cand = reinterpret_cast<SetCand*>(base + L.cand);
+    float* const sample = reinterpret_cast<float*>(base + L.sample);
+    Item* const fin = reinterpret_cast<Item*>(base + L.fin);
+    Item* const best = reinterpret_cast<Item*>(base + L.best);
+    const int grid = 16 * sms;
+    cudaError_t e = cudaSuccess;
+    e = count_subsets<1>(a, grid, st);
+    if (e == cudaSuccess) e = count_subsets<2>(a, grid, st);
+    if (e == cudaSuccess) e = count_subsets<3>(a, grid, st);
+    if (e == cudaSuccess && K > 4) e = count_subsets<4>(a, grid, st);
+    if (e == cudaSuccess && K > 5) e = count_subsets<5>(a, grid, st);
+    if (e != cudaSuccess) return e;
+    auto scan = [&](long long stride, long long n, float* smp) {
+        const long long blocks = (n + kSetThreads - 1) / kSetThreads;
+        const unsigned g = (unsigned)(blocks < grid ? blocks : grid);
+        if (smem) set_scan_kernel<K, true><<<g, kSetThreads, bytes, st>>>(a, stride, n, smp, ctrl, cand, kSetCand);
+        else set_scan_kernel<K, false><<<g, kSetThreads, 0, st>>>(a, stride, n, smp, ctrl, cand, kSetCand);
+        return cudaGetLastError();
+    };
+    e = scan(a.n_sets / L.n_sample, L.n_sample, sample);
+    if (e != cudaSuccess) return e;
+    set_threshold_kernel<<<1, 1024, 0, st>>>(sample, 1, L.n_sample, nullptr, k, delta, ctrl);
+    for (int attempt = 0; attempt < 4; ++attempt) {
+        e = scan(1, a.n_sets, nullptr);
+        if (e != cudaSuccess) return e;
+        // the threshold from the candidates themselves (any set of k of them bounds the k-th)
+        set_threshold_kernel<<<1, 1024, 0, st>>>(&cand->s, sizeof(SetCand) / sizeof(float), kSetCand,
+                                                 &ctrl->n_cand, k, delta, ctrl);
+        set_rescore_kernel<K><<<4 * sms, kOrdThreads, 0, st>>>(a, lf64, ctrl, cand, kSetCand, fin, kPairBlock);
+        set_final_kernel<<<1, kPairThreads, 0, st>>>(ctrl, fin, k, best);
+        order_emit_kernel<K><<<1, 512, 0, st>>>(best, k, a.pl.M, out_snps, out_s);
+        e = cudaMemcpyAsync(h_ctrl, ctrl, sizeof(SetCtrl), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e == cudaSuccess) e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        if (h_ctrl->n_cand <= kSetCand) {
+            *done = h_ctrl->n_final <= (unsigned)kPairBlock;
+            return cudaSuccess;
+        }
+        // the list overflowed: once more with the threshold of what it holds
+        e = cudaMemsetAsync(&ctrl->n_cand, 0, sizeof(unsigned), st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 }  // namespace
+
+// Scratch bytes of the counted form, 0 if it does not serve the size.
+size_t set_scan_scratch(int M, int N, int order) {
+    if (order < 4 || order > 6 || M < order) return 0;
+    double sub = 0.0, c = 1.0;
+    for (int t = 1; t < order; ++t) {
+        c = c * (M - t + 1) / t;
+        sub += c * (4 << t);
+    }
+    if (sub > (double)kSubsetBytes) return 0;
+    return set_layout(M, N, order).total;
+}
+
+cudaError_t launch_set_scan(const Planes& pl, const double* lf64, int n0, int n1, int order, int k, int sms,
+                            void* scratch, void* h_ctrl, int32_t* out_snps, double* out_s, bool* done,
+                            cudaStream_t st) {
+    const int N = n0 + n1;
+    const SetLayout L = set_layout(pl.M, N, order);
+    char* const base = static_cast<char*>(scratch);
+    SetArgs a{};
+    a.pl = pl;
+    a.binom = reinterpret_cast<const long long*>(base + L.binom);
+    a.lf = reinterpret_cast<const float*>(base + L.lf);
+    a.n_lf = N + 2;
+    for (int t = 1; t < order; ++t) a.sub[t] = reinterpret_cast<uint32_t*>(base + L.sub[t]);
+    a.total = (uint32_t)n0 + ((uint32_t)n1 << 16);
+    a.n_sets = choose_ll(pl.M, order);
+    // |FP32 score - K2|: the table's entries and the two subtractions round by 2^-24 of lf(r + 1) at
+    // most, and the cells' lf(r + 1) sum to at most lf(N + 3^K); each addition rounds by 2^-24 of the
+    // score.  Both with a margin, plus the subtraction's own rounding of small terms.
+    const double cells = order == 4 ? 81.0 : order == 5 ? 243.0 : 729.0;
+    const double top = std::lgamma((double)N + cells + 1.0);
+    const double score = (double)N * std::log(2.0) + std::fmin((double)N, cells) * std::log((double)N + 2.0);
+    const float delta = (float)(std::ldexp(1.0, -24) * (6.0 * top + cells * score) * 1.1 + 0.01);
+    set_tables_kernel<<<sms, 256, 0, st>>>(pl.M, lf64, N + 2, reinterpret_cast<long long*>(base + L.binom),
+                                           reinterpret_cast<float*>(base + L.lf));
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    SetCtrl* const hc = static_cast<SetCtrl*>(h_ctrl);
+    if (order == 4) return set_scan_k<4>(a, L, lf64, sms, k, delta, base, hc, out_snps, out_s, done, st);
+    if (order == 5) return set_scan_k<5>(a, L, lf64, sms, k, delta, base, hc, out_snps, out_s, done, st);
+    return set_scan_k<6>(a, L, lf64, sms, k, delta, base, hc, out_snps, out_s, done, st);
+}
 
 long long order_count(int M, int order) { return choose_ll(M, order); }
 
