@@ -431,20 +431,32 @@ int build_k2_tables(epi3_handle* h) {
 //     each, c-fold; c's and the last FMA's rounding: 3 2^-24 (c S1 + 200); logs and products: under
 //     0.01; the FP32 score against K2: rel * K + abs as in build_k2_tables.
 // The rounding terms are doubled.
+// For `cells` cells the S of Sum us and p0 change with the cells' u = count + 1 and Stirling's terms
+// with their number; c is taken for 27 cells and serves 9 as well (a larger value is a weaker bound):
+// the two p0 differ by less than 27 / N, and c is raised to cover both.
 void cmp_bound_terms(epi3_handle* h) {
     const int cm = h->N1 <= h->N0 ? 1 : 0;
-    const double S = (double)h->N + 54.0, S1 = (double)(cm ? h->N1 : h->N0) + 27.0, p0 = S1 / S;
-    const double c = std::max(-std::log1p(-p0) / (p0 * p0), -std::log(p0) / ((1.0 - p0) * (1.0 - p0)));
-    const double H = -p0 * std::log(p0) - (1.0 - p0) * std::log1p(-p0);
+    const double nm = (double)(cm ? h->N1 : h->N0), N = (double)h->N;
+    auto p_of = [&](double cells) { return (nm + cells) / (N + 2.0 * cells); };
+    auto c_of = [](double p) {
+        return std::max(-std::log1p(-p) / (p * p), -std::log(p) / ((1.0 - p) * (1.0 - p)));
+    };
+    const double c = std::max(c_of(p_of(27.0)), c_of(p_of(9.0)));
     const double u = std::ldexp(1.0, -24);
-    const double kmax = 27.0 * std::log((double)h->N + 2.0) + (double)h->N * std::log(2.0);
+    const double kmax = 27.0 * std::log(N + 2.0) + N * std::log(2.0);
+    const double S1 = nm + 27.0;
     const double rnd = 4.0 * u * S1 * (c + 1.1) + 27.0 * u * S1 * c + 3.0 * u * (c * S1 + 200.0) + 0.01 +
                        (double)h->k2.rel * kmax + (double)h->k2.abs_;
-    const double slack = 27.0 / 6.0 + 2.0 * rnd;
-    h->bound.c = (float)c;
-    h->bound.slack = (float)slack;
-    h->bound.off = std::nextafter((float)(c * S * p0 * (1.0 - p0) - S * H + 27.0 * 0.9189385332046727 + slack),
-                                  INFINITY);
+    auto off_of = [&](double cells) {
+        const double S = N + 2.0 * cells, p = p_of(cells);
+        const double H = -p * std::log(p) - (1.0 - p) * std::log1p(-p);
+        const double off = c * S * p * (1.0 - p) - S * H + cells * (0.9189385332046727 + 1.0 / 6.0) + 2.0 * rnd;
+        return std::nextafter((float)off, INFINITY);
+    };
+    h->bound.c = std::nextafter((float)c, INFINITY);
+    h->bound.off = off_of(27.0);
+    h->bound.off2 = off_of(9.0);
+    h->bound.slack = (float)(27.0 / 6.0 + 2.0 * rnd);
     h->bound.minor = cm;
 }
 
@@ -1396,20 +1408,36 @@ int epi3_scan_pairs(epi3_handle* h, int32_t top_k, int32_t* out_pairs, double* o
         return fail(EPI3_ERR_ARG, "top_k %d outside 1..min(%d, %lld)", top_k, EPI3_MAX_TOPK, np);
     int rc = ensure_pair_tables(h);
     if (rc != EPI3_OK) return rc;
-    const size_t sel = (pair_scan_scratch(np, top_k) + 255) & ~(size_t)255;
-    const size_t need = sel + sizeof(double) * (size_t)top_k + sizeof(int32_t) * 2 * (size_t)top_k;
-    if (h->pair_scratch_bytes < need) {
+    const size_t outs = sizeof(double) * (size_t)top_k + sizeof(int32_t) * 2 * (size_t)top_k;
+    auto scratch = [&](size_t bytes) -> int {   // kept on the handle; outputs after the first `bytes`
+        if (h->pair_scratch_bytes >= bytes + outs) return EPI3_OK;
         dev_free(h->d_pair_scratch);
         h->d_pair_scratch = nullptr;
         h->pair_scratch_bytes = 0;
-        CK(dev_alloc(&h->d_pair_scratch, need), "alloc pair-scan scratch");
-        h->pair_scratch_bytes = need;
-    }
-    double* d_s = reinterpret_cast<double*>(static_cast<char*>(h->d_pair_scratch) + sel);
-    int32_t* d_pairs = reinterpret_cast<int32_t*>(d_s + top_k);
+        CK(dev_alloc(&h->d_pair_scratch, bytes + outs), "alloc pair-scan scratch");
+        h->pair_scratch_bytes = bytes + outs;
+        return EPI3_OK;
+    };
+    double* d_s = nullptr;
+    int32_t* d_pairs = nullptr;
+    auto place = [&](size_t bytes) {
+        d_s = reinterpret_cast<double*>(static_cast<char*>(h->d_pair_scratch) + bytes);
+        d_pairs = reinterpret_cast<int32_t*>(d_s + top_k);
+    };
+    const size_t flt = pair_filter_scratch(np);
+    if ((rc = scratch(flt)) != EPI3_OK) return rc;
+    place(flt);
     CK(cudaEventRecord(h->ev[0], h->stream), "event");
-    CK(launch_pair_scan(h->ptab, h->k2.lf64, h->M, top_k, h->d_pair_scratch, d_pairs, d_s,
-                        h->stream), "pair scan launch");
+    bool done = false;
+    CK(launch_pair_filter(h->ptab, h->k2.lf64, h->M, top_k, h->bound, h->sm_count, h->d_pair_scratch, h->h_ctrl,
+                          d_pairs, d_s, &done, h->stream), "pair scan launch");
+    if (!done) {   // thousands of pairs tie at the k-th score: every pair sorted
+        const size_t sel = (pair_scan_scratch(np, top_k) + 255) & ~(size_t)255;
+        if ((rc = scratch(sel)) != EPI3_OK) return rc;
+        place(sel);
+        CK(launch_pair_scan(h->ptab, h->k2.lf64, h->M, top_k, h->d_pair_scratch, d_pairs, d_s,
+                            h->stream), "pair scan launch");
+    }
     CK(cudaEventRecord(h->ev[1], h->stream), "event");
     const cudaMemcpyKind kind =
         (h->flags & EPI3_DEVICE_PTRS) ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;

@@ -86,6 +86,14 @@ struct PairTables {
     const float2* margf;
 };
 
+// Constants of the table-free bound by class sizes (cmp_bound_terms in capi.cu).
+struct CmpBoundTerms {
+    float c, off;                // K2 >= c (sum of q) + (ln of the product of q) / 2 - off, 27 cells
+    float off2;                  // the same for the 9 cells of a pair
+    float slack;                 // the part of off that covers Stirling's remainders and rounding
+    int minor;                   // the smaller class
+};
+
 struct ScanArgs {
     Planes pl;
     K2Tables k2;
@@ -125,6 +133,13 @@ cudaError_t launch_reset(Ctrl* ctrl, cudaStream_t st);
 size_t pair_scan_scratch(long long n_pairs, int k);
 cudaError_t launch_pair_scan(const PairTables& pt, const double* lf64, int M, int k,
                              void* scratch, int32_t* out_pairs, double* out_s, cudaStream_t st);
+// The same by a threshold from a sample of the pairs and a table-free bound; *done false: the direct
+// form must answer (thousands of pairs tie at the k-th score).  Reads a few words back into h_ctrl
+// (pinned) and synchronises.
+size_t pair_filter_scratch(long long n_pairs);
+cudaError_t launch_pair_filter(const PairTables& pt, const double* lf64, int M, int k, const CmpBoundTerms& bound,
+                               int sms, void* scratch, void* h_ctrl, int32_t* out_pairs, double* out_s, bool* done,
+                               cudaStream_t st);
 // Four-SNP scan (Eq. 1 for four SNPs, 81 cells): the k best sets by (FP64 K2, i, j, k, l) from
 // the bit planes; needs both class sizes below 65536 and M below 65536.
 // orders 5 and 6: every set by AND + POPC (one warp per set), FP64 K2 in cell order
@@ -290,12 +305,6 @@ __host__ __device__ __forceinline__ void canon_rows(T* u, int d) {
         }
     }
 }
-// Constants of the compacted scan's table-free bound for class sizes n0, n1 (capi.cu).
-struct CmpBoundTerms {
-    float c, off;                // K2 >= c (sum of q) + (ln of the product of q) / 2 - off
-    float slack;                 // the part of off that covers Stirling's remainders and rounding
-    int minor;                   // the smaller class
-};
 // compacted chunks of one first SNP: 16 KB each
 inline long long cmp_chunks_of(const CmpFirst& f, int M) {
     const long long nblk = (M + 63) / 64 - f.b_lo;

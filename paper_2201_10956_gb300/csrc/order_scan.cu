@@ -50,11 +50,11 @@ __device__ __forceinline__ bool item_before(const Item& a, const Item& b) {
     return a.s < b.s || (a.s == b.s && a.key < b.key);
 }
 
-// Ascending bitonic sort of kPairBlock items in shared memory (all threads of the block).
-__device__ void sort_items(Item* it) {
-    for (int size = 2; size <= kPairBlock; size <<= 1)
+// Ascending bitonic sort of n items (a power of two) in shared memory (all threads of the block).
+__device__ void sort_items(Item* it, int n = kPairBlock) {
+    for (int size = 2; size <= n; size <<= 1)
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int t = threadIdx.x; t < kPairBlock / 2; t += blockDim.x) {
+            for (int t = threadIdx.x; t < n / 2; t += blockDim.x) {
                 const int lo = 2 * t - (t & (stride - 1)), hi = lo + stride;
                 const bool up = (lo & size) == 0;
                 const Item x = it[lo], y = it[hi];
@@ -67,11 +67,51 @@ __device__ void sort_items(Item* it) {
         }
 }
 
+// -1 / x by the hardware reciprocal (within 1 ulp)
+__device__ __forceinline__ float pair_nrcp(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(-x));
+    return y;
+}
+
 __device__ __forceinline__ Item pad_item() {
     return Item{__longlong_as_double(0x7ff0000000000000LL), 0x7fffffffffffffffLL};  // +inf, last
 }
 
-// Pass 1: score pairs [b * 2048, (b + 1) * 2048), keep the block's k best in out[b * k ..].
+// Cells r[c][3 gX + gY] of pair p = (i, j); false if a corrupt table makes one negative.
+__device__ __forceinline__ bool pair_cells(const PairTables& pt, int M, long long p, int i, int j, int (&r)[2][9]) {
+    int neg = 0;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+        const int4 q = __ldg(pt.pt + c * pt.n_pairs + p);        // {n00, n01, n10, n11}
+        const int2 mi = __ldg(pt.marg + (size_t)c * M + i), mj = __ldg(pt.marg + (size_t)c * M + j);
+        r[c][0] = q.x;
+        r[c][1] = q.y;
+        r[c][2] = mi.x - q.x - q.y;     // (0, 2)
+        r[c][3] = q.z;
+        r[c][4] = q.w;
+        r[c][5] = mi.y - q.z - q.w;     // (1, 2)
+        r[c][6] = mj.x - q.x - q.z;     // (2, 0)
+        r[c][7] = mj.y - q.y - q.w;     // (2, 1)
+        r[c][8] = pt.n_c[c] - mi.x - mi.y - r[c][6] - r[c][7];   // (2, 2)
+#pragma unroll
+        for (int cell = 0; cell < 9; ++cell) neg |= r[c][cell];
+    }
+    return neg >= 0;
+}
+// FP64 K2 of a pair in cell order.
+__device__ __forceinline__ double pair_score(const int (&r)[2][9], const double* __restrict__ lf64) {
+    double s = 0.0;
+#pragma unroll
+    for (int cell = 0; cell < 9; ++cell) {
+        const int r0 = r[0][cell], r1 = r[1][cell];
+        s = __dadd_rn(s, __dsub_rn(__dsub_rn(lf64[r0 + r1 + 1], lf64[r0]), lf64[r1]));
+    }
+    return s;
+}
+
+// Pass 1 of the direct form: score pairs [b * 2048, (b + 1) * 2048), keep the block's k best in
+// out[b * k ..].
 __global__ void __launch_bounds__(kPairThreads)
 pair_score_kernel(PairTables pt, const double* __restrict__ lf64, int M, long long n_pairs,
                   int k, Item* __restrict__ out) {
@@ -79,44 +119,12 @@ pair_score_kernel(PairTables pt, const double* __restrict__ lf64, int M, long lo
     const long long p0 = (long long)blockIdx.x * kPairBlock;
     for (int t = threadIdx.x; t < kPairBlock; t += kPairThreads) {
         const long long p = p0 + t;
-        if (p >= n_pairs) {
-            it[t] = pad_item();
-            continue;
-        }
-        int i, j;
+        it[t] = pad_item();
+        if (p >= n_pairs) continue;
+        int i, j, r[2][9];
         decode_pair(p, &i, &j);
-        double s = 0.0;
-        int r[2][9];
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int4 q = __ldg(pt.pt + c * pt.n_pairs + p);        // {n00, n01, n10, n11}
-            const int2 mi = __ldg(pt.marg + (size_t)c * M + i), mj = __ldg(pt.marg + (size_t)c * M + j);
-            r[c][0] = q.x;
-            r[c][1] = q.y;
-            r[c][2] = mi.x - q.x - q.y;     // (0, 2)
-            r[c][3] = q.z;
-            r[c][4] = q.w;
-            r[c][5] = mi.y - q.z - q.w;     // (1, 2)
-            r[c][6] = mj.x - q.x - q.z;     // (2, 0)
-            r[c][7] = mj.y - q.y - q.w;     // (2, 1)
-            r[c][8] = pt.n_c[c] - (r[c][0] + r[c][1] + r[c][2] + r[c][3] + r[c][4] + r[c][5] +
-                                   r[c][6] + r[c][7]);                 // (2, 2)
-        }
         // exact counts cannot be negative; a corrupt table is ranked last, never looked up
-        int neg = 0;
-#pragma unroll
-        for (int cell = 0; cell < 9; ++cell) neg |= r[0][cell] | r[1][cell];
-        if (neg < 0) {
-            it[t] = pad_item();
-            continue;
-        }
-#pragma unroll
-        for (int cell = 0; cell < 9; ++cell) {
-            const int r0 = r[0][cell], r1 = r[1][cell];
-            const double term = __dsub_rn(__dsub_rn(lf64[r0 + r1 + 1], lf64[r0]), lf64[r1]);
-            s = __dadd_rn(s, term);
-        }
-        it[t] = Item{s, (long long)i * M + j};
+        if (pair_cells(pt, M, p, i, j, r)) it[t] = Item{pair_score(r, lf64), (long long)i * M + j};
     }
     __syncthreads();
     sort_items(it);
@@ -841,10 +849,71 @@ __global__ void __launch_bounds__(kPairThreads)
 set_final_kernel(const SetCtrl* ctrl, const Item* __restrict__ fin, int k, Item* __restrict__ out) {
     __shared__ Item it[kPairBlock];
     const int n = min(ctrl->n_final, (unsigned)kPairBlock);
-    for (int t = threadIdx.x; t < kPairBlock; t += kPairThreads) it[t] = t < n ? fin[t] : pad_item();
+    int n2 = 64;
+    while (n2 < n || n2 < k) n2 <<= 1;
+    for (int t = threadIdx.x; t < n2; t += kPairThreads) it[t] = t < n ? fin[t] : pad_item();
     __syncthreads();
-    sort_items(it);
+    sort_items(it, n2);
     for (int t = threadIdx.x; t < k; t += kPairThreads) out[t] = it[t];
+}
+
+// ---------------------------------------------------------------- pairs, thresholded form
+// FP64 scores, rounded up to FP32, of every stride-th pair.
+__global__ void __launch_bounds__(256)
+pair_sample_kernel(PairTables pt, const double* __restrict__ lf64, int M, long long stride, long long n,
+                   float* __restrict__ sample) {
+    for (long long t = (long long)blockIdx.x * 256 + threadIdx.x; t < n; t += (long long)gridDim.x * 256) {
+        const long long p = t * stride;
+        int i, j, r[2][9];
+        decode_pair(p, &i, &j);
+        sample[t] = pair_cells(pt, M, p, i, j, r) ? __double2float_ru(pair_score(r, lf64))
+                                                  : __int_as_float(0x7f800000);
+    }
+}
+// Pairs that may lie at or below the threshold: a table-free bound first (that of the compacted
+// triplet scan with 9 cells, cmp_bound_terms: K2 >= c (sum of q) + (ln of the product of q) / 2 -
+// off), the FP64 score for the few it lets through.  Reads each pair table once (32 bytes a pair, the
+// floor); the direct form sorts every 2048 pairs it scores.  CTA row y: second SNP j = y + 1, ...
+__global__ void __launch_bounds__(256)
+pair_filter_kernel(PairTables pt, const double* __restrict__ lf64, int M, float bound_c, float bound_off,
+                   int minor, SetCtrl* ctrl, SetCand* __restrict__ cand, unsigned cap) {
+    const float thr = ctrl->thr, cut = __fadd_ru(thr, bound_off);
+    for (int j = 1 + blockIdx.y; j < M; j += gridDim.y) {
+        const int i = blockIdx.x * 256 + threadIdx.x;
+        if (i >= j) continue;
+        const long long p = pair_index(i, j);
+        int r[2][9];
+        if (!pair_cells(pt, M, p, i, j, r)) continue;
+        float sum = 0.f, prod = 1.f;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            const float us = (float)(r[0][e] + r[1][e] + 2), um = (float)((minor ? r[1][e] : r[0][e]) + 1);
+            const float q = __fmaf_rn(__fmul_rn(um, pair_nrcp(us)), um, um);
+            sum = __fadd_rn(sum, q);
+            prod = __fmul_rn(prod, q);
+        }
+        if (__fmaf_rn(bound_c, sum, 0.34657359f * lg2_hw(prod)) > cut) continue;
+        const float s = __double2float_ru(pair_score(r, lf64));
+        if (s <= thr) {
+            const unsigned pos = atomicAdd(&ctrl->n_cand, 1u);
+            if (pos < cap) cand[pos] = SetCand{p, s};
+        }
+    }
+}
+__global__ void __launch_bounds__(256)
+pair_rescore_kernel(PairTables pt, const double* __restrict__ lf64, int M, SetCtrl* ctrl,
+                    const SetCand* __restrict__ cand, unsigned cap, Item* __restrict__ fin, unsigned fin_cap) {
+    const unsigned n = min(ctrl->n_cand, cap);
+    const float thr = ctrl->thr;
+    for (unsigned e = blockIdx.x * 256 + threadIdx.x; e < n; e += gridDim.x * 256) {
+        const SetCand cd = cand[e];
+        if (!(cd.s <= thr)) continue;
+        int i, j, r[2][9];
+        decode_pair(cd.q, &i, &j);
+        pair_cells(pt, M, cd.q, i, j, r);
+        const unsigned pos = atomicAdd(&ctrl->n_final, 1u);
+        if (pos < fin_cap) fin[pos] = Item{pair_score(r, lf64), (long long)i * M + j};
+    }
 }
 
 constexpr unsigned kSetCand = 1u << 18;          // candidate list
@@ -1025,6 +1094,70 @@ cudaError_t launch_quad_scan(const Planes& pl, const double* lf64, int n0, int n
     if (e != cudaSuccess) return e;
     quad_emit_kernel<<<1, 512, 0, st>>>(a, k, out_snps, out_s);
     return cudaGetLastError();
+}
+
+namespace {
+struct PairLayout {
+    size_t ctrl, cand, fin, best, sample, total;
+    long long n_sample;
+};
+PairLayout pair_layout(long long n) {
+    PairLayout L{};
+    size_t o = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = o;
+        o += (bytes + 255) & ~(size_t)255;
+        return at;
+    };
+    // evenly spaced pairs for the first threshold: enough that about k n / n_sample candidates are few
+    L.n_sample = n < 32768 ? n : 32768;
+    L.ctrl = take(sizeof(SetCtrl));
+    L.cand = take(sizeof(SetCand) * kSetCand);
+    L.fin = take(sizeof(Item) * kPairBlock);
+    L.best = take(sizeof(Item) * EPI3_MAX_TOPK);
+    L.sample = take(sizeof(float) * (size_t)L.n_sample);
+    L.total = o;
+    return L;
+}
+}  // namespace
+
+size_t pair_filter_scratch(long long n_pairs) { return pair_layout(n_pairs).total; }
+
+cudaError_t launch_pair_filter(const PairTables& pt, const double* lf64, int M, int k, const CmpBoundTerms& bound,
+                               int sms, void* scratch, void* h_ctrl, int32_t* out_pairs, double* out_s, bool* done,
+                               cudaStream_t st) {
+    const PairLayout L = pair_layout(pt.n_pairs);
+    char* const base = static_cast<char*>(scratch);
+    SetCtrl* const ctrl = reinterpret_cast<SetCtrl*>(base + L.ctrl);
+    SetCand* const cand = reinterpret_cast<SetCand*>(base + L.cand);
+    Item* const fin = reinterpret_cast<Item*>(base + L.fin);
+    Item* const best = reinterpret_cast<Item*>(base + L.best);
+    float* const sample = reinterpret_cast<float*>(base + L.sample);
+    SetCtrl* const hc = static_cast<SetCtrl*>(h_ctrl);
+    *done = false;
+    pair_sample_kernel<<<(unsigned)((L.n_sample + 255) / 256), 256, 0, st>>>(pt, lf64, M, pt.n_pairs / L.n_sample,
+                                                                             L.n_sample, sample);
+    set_threshold_kernel<<<1, 1024, 0, st>>>(sample, 1, L.n_sample, nullptr, k, 0.f, ctrl);
+    const dim3 grid((M + 255) / 256, M < 8192 ? M : 8192);
+    for (int attempt = 0; attempt < 4; ++attempt) {
+        pair_filter_kernel<<<grid, 256, 0, st>>>(pt, lf64, M, bound.c, bound.off2, bound.minor, ctrl, cand, kSetCand);
+        set_threshold_kernel<<<1, 1024, 0, st>>>(&cand->s, sizeof(SetCand) / sizeof(float), kSetCand,
+                                                 &ctrl->n_cand, k, 0.f, ctrl);
+        pair_rescore_kernel<<<sms, 256, 0, st>>>(pt, lf64, M, ctrl, cand, kSetCand, fin, kPairBlock);
+        set_final_kernel<<<1, kPairThreads, 0, st>>>(ctrl, fin, k, best);
+        pair_emit_kernel<<<1, 512, 0, st>>>(best, k, M, out_pairs, out_s);
+        cudaError_t e = cudaMemcpyAsync(hc, ctrl, sizeof(SetCtrl), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e == cudaSuccess) e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        if (hc->n_cand <= kSetCand) {
+            *done = hc->n_final <= (unsigned)kPairBlock;
+            return cudaSuccess;
+        }
+        e = cudaMemsetAsync(&ctrl->n_cand, 0, sizeof(unsigned), st);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 size_t pair_scan_scratch(long long n_pairs, int k) {
