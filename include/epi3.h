@@ -292,8 +292,10 @@ int epi3_get_stats(const epi3_handle* h, epi3_stats* out);
  *   top_k, out_triplets, out_scores   as epi3_scan, but the outputs are device pointers.
  *   cuda_stream            stream to run on (NULL = the legacy default stream).
  *
- * It counts with the 27-cell POPC scan (EPI3_PATH_POPC, about 5 T sample-triplets/s on
- * GB300), not the tensor-core form epi3_scan uses by default, and its candidate list has a
+ * It counts with the 8-cell POPC scan (EPI3_PATH_POPC8, about 18 T sample-triplets/s on
+ * GB300) where the pair tables fit the scratch too (up to some 600 SNPs), with the 27-cell one
+ * (EPI3_PATH_POPC, about 5 T) beyond, not with the tensor-core form epi3_scan uses by default,
+ * and its candidate list has a
  * fixed 65536 entries with no retry: a data set with more near-tied FP32 candidates gives
  * EPI3_ERR_OVERFLOW where epi3_scan would grow the list.  The answer is the one epi3_scan
  * gives.

@@ -225,6 +225,24 @@ long long triplets_in_pairs(long long M, long long pb, long long pe) {
 
 }  // namespace
 
+namespace {
+
+// The compaction plan of the pair range [pb, pe): per first SNP its chunks and tiles, grouped
+// into ranges whose chunks fit the handle's buffer; totals of compacted chunks and MMA K-steps
+// (the two work terms of this form, used by the tuner to extrapolate a slice's timing).
+struct CmpPlan {
+    std::vector<CmpFirst> firsts;
+    std::vector<CmpGroup> groups;
+    std::vector<int> range_start;   // first SNP of each range
+    std::vector<int> range_group;   // first group of each range
+    std::vector<int> range_runs;
+    size_t need = 0;                // buffer bytes of the largest range
+    int i_hi = 0;                   // first SNPs [0, i_hi)
+    double chunks_total = 0.0, steps_total = 0.0;
+};
+
+}  // namespace
+
 struct epi3_handle {
     int device = 0, sm_count = 0;
     cudaStream_t stream = nullptr;
@@ -276,6 +294,9 @@ struct epi3_handle {
     size_t cmp_cap = (size_t)2 << 30;  // option "cmp_buffer_mb": bytes of compacted chunks at once
     CmpFirst* d_firsts = nullptr; // per first SNP: chunk bases, K-steps, tiles
     CmpGroup* d_groups = nullptr; // groups of first SNPs that a run of tiles covers
+    CmpPlan plan;                 // the compacted scan's plan for pairs [plan_pb, plan_pe) ...
+    long long plan_pb = -1, plan_pe = -1;
+    size_t plan_cap = 0;          // ... at this cmp_cap
     CmpBoundTerms bound{};        // the compacted scan's table-free bound
     std::vector<int2> h_marg;     // marginals on the host (the compacted sets' sizes)
     int4* d_tiles = nullptr;      // tile list of the tensor-core form
@@ -711,15 +732,25 @@ int resolve_path(const epi3_handle* h) {
 }
 int tune_handle(epi3_handle* h);
 
-// Candidate stage + result read-back shared by both scan forms.  Returns 1 to retry with a
-// larger candidate list, EPI3_OK, or an error.
-int finish_scan(epi3_handle* h, int top_k, int attempt) {
-    CK(launch_select(h->d_ctrl, h->d_cand, h->cand_cap, top_k, h->k2.rel, h->k2.abs_, h->stream),
-       "select launch");
-    CK(launch_rescore(h->pl, h->k2, h->d_ctrl, h->d_cand, h->cand_cap, h->d_fin, h->sm_count * 8,
-                      h->stream), "rescore launch");
-    CK(launch_final(h->d_ctrl, h->d_fin, top_k, h->d_out_scores, h->d_out_trip, h->stream),
-       "final launch");
+// Start of a scan of [pb, pe): control block, threshold, checksum slots (a retried scan counts every
+// table again).
+int start_scan(epi3_handle* h, long long pb, long long pe, int top_k) {
+    CK(launch_seed(h->pl, h->k2, h->d_ctrl, h->d_cand, h->cand_cap, pb, pe, top_k, h->stream), "seed launch");
+    if (h->tsum)
+        CK(cudaMemsetAsync(h->tsum, 0, 2 * kTsumSlots * sizeof(unsigned long long), h->stream),
+           "clear checksum slots");
+    return EPI3_OK;
+}
+
+// Candidate stage + result read-back shared by all scan forms.  The caller's device outputs are
+// written by the candidate stage itself; the scans of the tuner and of the debug calls keep their
+// answer in the handle's buffers.  Returns 1 to retry with a larger candidate list, EPI3_OK, or an
+// error.
+int finish_scan(epi3_handle* h, int top_k, int attempt, int32_t* out_trip, double* out_scores) {
+    const bool direct = (h->flags & EPI3_DEVICE_PTRS) && !h->tuning && !h->dbg && !h->tsum;
+    CK(launch_answer(h->pl, h->k2, h->d_ctrl, h->d_cand, h->cand_cap, top_k, h->d_fin,
+                     direct ? out_scores : h->d_out_scores, direct ? out_trip : h->d_out_trip, h->stream),
+       "candidate stage launch");
     CK(cudaEventRecord(h->ev[3], h->stream), "event");
     CK(cudaMemcpyAsync(h->h_ctrl, h->d_ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream),
        "read status");
@@ -756,20 +787,13 @@ int finish_scan(epi3_handle* h, int top_k, int attempt) {
     return EPI3_OK;
 }
 
-int copy_out(epi3_handle* h, int32_t* out_trip, double* out_scores, int32_t* n_out) {
+void copy_out(epi3_handle* h, int32_t* out_trip, double* out_scores, int32_t* n_out) {
     const int nout = (int)h->h_ctrl->n_out;
-    if (h->flags & EPI3_DEVICE_PTRS) {
-        CK(cudaMemcpyAsync(out_scores, h->d_out_scores, sizeof(double) * nout,
-                           cudaMemcpyDeviceToDevice, h->stream), "copy scores");
-        CK(cudaMemcpyAsync(out_trip, h->d_out_trip, sizeof(int) * 3 * nout,
-                           cudaMemcpyDeviceToDevice, h->stream), "copy triplets");
-        CK(cudaStreamSynchronize(h->stream), "copy outputs");
-    } else {
+    if (!(h->flags & EPI3_DEVICE_PTRS)) {
         memcpy(out_scores, h->h_scores, sizeof(double) * nout);
         memcpy(out_trip, h->h_trip, sizeof(int) * 3 * nout);
     }
     if (n_out) *n_out = nout;
-    return EPI3_OK;
 }
 
 // Register-split or plain form of the tensor scan for this handle (option "mma_form").
@@ -827,10 +851,8 @@ int scan_mma_impl(epi3_handle* h, int path, long long pb, long long pe, long lon
     for (int attempt = 0;; ++attempt) {
         if (inject("launch")) return fail(EPI3_ERR_CUDA, "injected launch failure");
         CK(cudaEventRecord(h->ev[0], h->stream), "event");
-        CK(launch_reset(h->d_ctrl, h->stream), "reset launch");
-        if (h->tsum)  // a retried scan counts every table again: the checksum restarts with it
-            CK(cudaMemsetAsync(h->tsum, 0, 2 * kTsumSlots * sizeof(unsigned long long), h->stream),
-               "clear checksum slots");
+        const int src = start_scan(h, pb, pe, top_k);
+        if (src != EPI3_OK) return src;
         CK(cudaEventRecord(h->ev[1], h->stream), "event");
         const CohortDev cd = cohort_of(h, pb, pe, top_k);
         CK(cudaMemcpyAsync(h->d_cd, &cd, sizeof(cd), cudaMemcpyHostToDevice, h->stream),
@@ -843,13 +865,12 @@ int scan_mma_impl(epi3_handle* h, int path, long long pb, long long pe, long lon
                            h->profile ? h->d_prof : nullptr, mma_split(h, kind), h->tsum != nullptr),
            "mma scan launch");
         CK(cudaEventRecord(h->ev[2], h->stream), "event");
-        const int rc = finish_scan(h, top_k, attempt);
+        const int rc = finish_scan(h, top_k, attempt, out_trip, out_scores);
         if (rc == 1) continue;
         if (rc != EPI3_OK) return rc;
         break;
     }
-    const int rc = copy_out(h, out_trip, out_scores, n_out);
-    if (rc != EPI3_OK) return rc;
+    copy_out(h, out_trip, out_scores, n_out);
     epi3_stats& s = h->stats;
     s.n_triplets = nt;
     s.n_candidates = h->h_ctrl->n_cand;
@@ -858,7 +879,7 @@ int scan_mma_impl(epi3_handle* h, int path, long long pb, long long pe, long lon
     s.grid = grid;
     s.block = mma_threads(mma_split(h, kind_of_path(path)));
     s.form = mma_split(h, kind_of_path(path)) ? 2 : 1;
-    s.kernel_launches = 5;
+    s.kernel_launches = 3;
     s.wait_loader = s.wait_mma_operands = s.wait_mma_accum = s.wait_producers = s.wait_epilogue = 0.f;
     s.wait_producers_tmem = s.mma_issue = 0.f;
     if (h->profile && h->d_prof) {
@@ -889,19 +910,7 @@ int scan_mma_impl(epi3_handle* h, int path, long long pb, long long pe, long lon
 // the handle's buffer; per range one compaction launch, then one scan launch over the range's
 // tiles (the candidate stage carries over from range to range).
 
-// The compaction plan of the pair range [pb, pe): per first SNP its chunks and tiles, grouped
-// into ranges whose chunks fit the handle's buffer; totals of compacted chunks and MMA K-steps
-// (the two work terms of this form, used by the tuner to extrapolate a slice's timing).
-struct CmpPlan {
-    std::vector<CmpFirst> firsts;
-    std::vector<CmpGroup> groups;
-    std::vector<int> range_start;   // first SNP of each range
-    std::vector<int> range_group;   // first group of each range
-    std::vector<int> range_runs;
-    size_t need = 0;                // buffer bytes of the largest range
-    int i_hi = 0;                   // first SNPs [0, i_hi)
-    double chunks_total = 0.0, steps_total = 0.0;
-};
+// The compaction plan of the pair range [pb, pe) (CmpPlan).
 
 void plan_cmp(const epi3_handle* h, long long pb, long long pe, CmpPlan& P) {
     const int M = h->M;
@@ -986,10 +995,15 @@ void plan_cmp(const epi3_handle* h, long long pb, long long pe, CmpPlan& P) {
     if (!P.range_start.empty()) P.range_runs.push_back(runs);
 }
 
-// The compaction plan of [pb, pe) for this handle, with its first-SNP and group tables uploaded
-// (the marginals come to the host once per handle).
-int cmp_prepare(epi3_handle* h, long long pb, long long pe, CmpPlan& P) {
+// The compaction plan of [pb, pe) for this handle (h->plan, kept until another range or buffer size
+// is asked for), with its first-SNP and group tables uploaded (the marginals come to the host once
+// per handle).
+int cmp_prepare(epi3_handle* h, long long pb, long long pe) {
+    if (h->plan_pb == pb && h->plan_pe == pe && h->plan_cap == h->cmp_cap) return EPI3_OK;
     const int M = h->M;
+    h->plan_pb = -1;
+    h->plan = CmpPlan();
+    CmpPlan& P = h->plan;
     if (h->h_marg.empty()) {
         h->h_marg.resize(2 * (size_t)M);
         CK(cudaMemcpyAsync(h->h_marg.data(), h->d_marg, sizeof(int2) * 2 * (size_t)M,
@@ -1011,6 +1025,9 @@ int cmp_prepare(epi3_handle* h, long long pb, long long pe, CmpPlan& P) {
         CK(cudaMemcpyAsync(h->d_groups, P.groups.data(), sizeof(CmpGroup) * P.groups.size(),
                            cudaMemcpyHostToDevice, h->stream), "upload group table");
     }
+    h->plan_pb = pb;
+    h->plan_pe = pe;
+    h->plan_cap = h->cmp_cap;
     return EPI3_OK;
 }
 
@@ -1033,9 +1050,9 @@ CmpArgs cmp_args(const epi3_handle* h, const CohortDev& cd, int i0, int group, i
 
 int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int top_k,
                   int32_t* out_trip, double* out_scores, int32_t* n_out) {
-    CmpPlan P;
-    const int prc = cmp_prepare(h, pb, pe, P);
+    const int prc = cmp_prepare(h, pb, pe);
     if (prc != EPI3_OK) return prc;
+    const CmpPlan& P = h->plan;
     const std::vector<int>& range_start = P.range_start;
     const int i_hi = P.i_hi;
     const size_t need = P.need;
@@ -1059,10 +1076,8 @@ int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int 
     for (int attempt = 0;; ++attempt) {
         if (inject("launch")) return fail(EPI3_ERR_CUDA, "injected launch failure");
         CK(cudaEventRecord(h->ev[0], h->stream), "event");
-        CK(launch_reset(h->d_ctrl, h->stream), "reset launch");
-        if (h->tsum)  // a retried scan counts every table again: the checksum restarts with it
-            CK(cudaMemsetAsync(h->tsum, 0, 2 * kTsumSlots * sizeof(unsigned long long), h->stream),
-               "clear checksum slots");
+        const int src = start_scan(h, pb, pe, top_k);
+        if (src != EPI3_OK) return src;
         if (h->profile) {
             if (!h->d_prof) CK(dev_alloc((void**)&h->d_prof, 8 * sizeof(unsigned long long)), "alloc profile");
             CK(cudaMemsetAsync(h->d_prof, 0, 8 * sizeof(unsigned long long), h->stream), "clear profile");
@@ -1082,7 +1097,7 @@ int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int 
                "compacted scan launch");
         }
         CK(cudaEventRecord(h->ev[2], h->stream), "event");
-        const int rc = finish_scan(h, top_k, attempt);
+        const int rc = finish_scan(h, top_k, attempt, out_trip, out_scores);
         if (rc == 1) continue;
         if (rc != EPI3_OK) return rc;
         break;
@@ -1092,8 +1107,7 @@ int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int 
         cudaEventElapsedTime(&ms, h->cmp_ev[2 * r], h->cmp_ev[2 * r + 1]);
         compact_ms += ms;
     }
-    const int rc = copy_out(h, out_trip, out_scores, n_out);
-    if (rc != EPI3_OK) return rc;
+    copy_out(h, out_trip, out_scores, n_out);
     epi3_stats& s = h->stats;
     s.n_triplets = nt;
     s.n_candidates = h->h_ctrl->n_cand;
@@ -1102,7 +1116,7 @@ int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int 
     s.grid = grid;
     s.block = scan_cmp_threads();
     s.form = cmp_paired(h) ? 2 : 1;
-    s.kernel_launches = 2 * n_ranges + 3;
+    s.kernel_launches = 2 * n_ranges + 2;
     s.wait_loader = s.wait_mma_operands = s.wait_mma_accum = s.wait_producers = s.wait_epilogue = 0.f;
     s.wait_producers_tmem = s.mma_issue = 0.f;
     s.compact_ms = compact_ms;
@@ -1185,10 +1199,8 @@ int scan_impl(epi3_handle* h, long long pb, long long pe, int top_k, int32_t* ou
     for (int attempt = 0;; ++attempt) {
         if (inject("launch")) return fail(EPI3_ERR_CUDA, "injected launch failure");
         CK(cudaEventRecord(h->ev[0], h->stream), "event");
-        CK(launch_reset(h->d_ctrl, h->stream), "reset launch");
-        if (h->tsum)  // a retried scan counts every table again: the checksum restarts with it
-            CK(cudaMemsetAsync(h->tsum, 0, 2 * kTsumSlots * sizeof(unsigned long long), h->stream),
-               "clear checksum slots");
+        const int src = start_scan(h, pb, pe, top_k);
+        if (src != EPI3_OK) return src;
         ScanArgs a;
         a.pl = h->pl;
         a.k2 = h->k2;
@@ -1205,53 +1217,12 @@ int scan_impl(epi3_handle* h, long long pb, long long pe, int top_k, int32_t* ou
         if (path == EPI3_PATH_POPC8) CK(launch_scan_popc8(a, grid, block, smem, h->stream), "scan launch");
         else CK(launch_scan_popc(a, grid, block, smem, h->stream), "scan launch");
         CK(cudaEventRecord(h->ev[2], h->stream), "event");
-        CK(launch_select(h->d_ctrl, h->d_cand, h->cand_cap, top_k, h->k2.rel, h->k2.abs_, h->stream),
-           "select launch");
-        CK(launch_rescore(h->pl, h->k2, h->d_ctrl, h->d_cand, h->cand_cap, h->d_fin,
-                          h->sm_count * 8, h->stream),
-           "rescore launch");
-        CK(launch_final(h->d_ctrl, h->d_fin, top_k, h->d_out_scores, h->d_out_trip, h->stream),
-           "final launch");
-        CK(cudaEventRecord(h->ev[3], h->stream), "event");
-        CK(cudaMemcpyAsync(h->h_ctrl, h->d_ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream),
-           "read status");
-        if (!(h->flags & EPI3_DEVICE_PTRS)) {
-            CK(cudaMemcpyAsync(h->h_scores, h->d_out_scores, sizeof(double) * top_k,
-                               cudaMemcpyDeviceToHost, h->stream), "read scores");
-            CK(cudaMemcpyAsync(h->h_trip, h->d_out_trip, sizeof(int) * 3 * top_k,
-                               cudaMemcpyDeviceToHost, h->stream), "read triplets");
-        }
-        CK(cudaStreamSynchronize(h->stream), "scan");
-        const int st = h->h_ctrl->status;
-        if (st & kStCandOverflow) {
-            if (h->cand_cap >= (1LL << 24) || attempt >= 3)
-                return fail(EPI3_ERR_OVERFLOW, "more than %lld FP32 candidates", h->cand_cap);
-            dev_free(h->d_cand);
-            h->d_cand = nullptr;
-            h->cand_cap *= 8;
-            CK(dev_alloc((void**)&h->d_cand, sizeof(Cand) * h->cand_cap), "grow candidates");
-            continue;
-        }
-        if (st & kStFinalOverflow)
-            return fail(EPI3_ERR_OVERFLOW,
-                        "more than %d triplets lie within the FP32 error band of the k-th best",
-                        kFinalCap);
-        if (st & (kStInternal | kStBadIndex))
-            return fail(EPI3_ERR_CUDA, "internal error in the candidate stage (status %d)", st);
+        const int rc = finish_scan(h, top_k, attempt, out_trip, out_scores);
+        if (rc == 1) continue;
+        if (rc != EPI3_OK) return rc;
         break;
     }
-    const int nout = (int)h->h_ctrl->n_out;
-    if (h->flags & EPI3_DEVICE_PTRS) {
-        CK(cudaMemcpyAsync(out_scores, h->d_out_scores, sizeof(double) * nout,
-                           cudaMemcpyDeviceToDevice, h->stream), "copy scores");
-        CK(cudaMemcpyAsync(out_trip, h->d_out_trip, sizeof(int) * 3 * nout,
-                           cudaMemcpyDeviceToDevice, h->stream), "copy triplets");
-        CK(cudaStreamSynchronize(h->stream), "copy outputs");
-    } else {
-        memcpy(out_scores, h->h_scores, sizeof(double) * nout);
-        memcpy(out_trip, h->h_trip, sizeof(int) * 3 * nout);
-    }
-    if (n_out) *n_out = nout;
+    copy_out(h, out_trip, out_scores, n_out);
     epi3_stats& s = h->stats;
     s.n_triplets = nt;
     s.n_candidates = h->h_ctrl->n_cand;
@@ -1259,7 +1230,7 @@ int scan_impl(epi3_handle* h, long long pb, long long pe, int top_k, int32_t* ou
     s.path = path;
     s.grid = grid;
     s.block = block;
-    s.kernel_launches = 5;
+    s.kernel_launches = 3;
     s.k2_rel_bound = h->k2.rel;
     s.k2_abs_bound = h->k2.abs_;
     s.k2_prune_bound = h->k2.prune_delta;
@@ -1721,9 +1692,8 @@ struct epi3_batch {
     bool own_stream = false;
     std::vector<epi3_handle*> h;
     std::vector<int> path;              // EPI3_PATH_MMA4, EPI3_PATH_MMA4C or EPI3_PATH_POPC8 per cohort
-    // compacted-form cohorts: per cohort its plan (ranges of first SNPs), all compacting into one
+    // compacted-form cohorts (ranges of first SNPs in their handles' plans) all compact into one
     // shared buffer
-    std::vector<CmpPlan> cmp_plan;
     uint8_t* d_cmp = nullptr;
     Ctrl* d_ctrls = nullptr;            // one control block per cohort, contiguous
     Ctrl* h_ctrls = nullptr;            // pinned
@@ -1994,10 +1964,11 @@ int batch_capture(epi3_batch* b, int top_k) {
             where_c = cur_c;
         }
     };
-    cur = "reset";
+    cur = "seed";
     for (int c = 0; c < b->n; ++c) {
         cur_c = c;
-        ok(launch_reset(b->h[c]->d_ctrl, b->stream));
+        epi3_handle* h = b->h[c];
+        ok(launch_seed(h->pl, h->k2, h->d_ctrl, h->d_cand, h->cand_cap, 0, pairs(h->M - 1), top_k, b->stream));
     }
     cur = "tensor scan";
     cur_c = -1;
@@ -2044,7 +2015,7 @@ int batch_capture(epi3_batch* b, int top_k) {
         if (b->path[c] != EPI3_PATH_MMA4C) continue;
         cur_c = c;
         epi3_handle* h = b->h[c];
-        const CmpPlan& P = b->cmp_plan[c];
+        const CmpPlan& P = h->plan;
         const std::vector<int>& rs = P.range_start;
         for (size_t r = 0; r < rs.size(); ++r) {
             const int i0 = rs[r];
@@ -2058,11 +2029,9 @@ int batch_capture(epi3_batch* b, int top_k) {
     for (int c = 0; c < b->n; ++c) {
         cur_c = c;
         epi3_handle* h = b->h[c];
-        ok(launch_select(h->d_ctrl, h->d_cand, h->cand_cap, top_k, h->k2.rel, h->k2.abs_, b->stream));
-        ok(launch_rescore(h->pl, h->k2, h->d_ctrl, h->d_cand, h->cand_cap, h->d_fin,
-                          b->sm_count * 8, b->stream));
-        ok(launch_final(h->d_ctrl, h->d_fin, top_k, b->d_scores + (size_t)c * EPI3_MAX_TOPK,
-                        b->d_trip + (size_t)c * 3 * EPI3_MAX_TOPK, b->stream));
+        ok(launch_answer(h->pl, h->k2, h->d_ctrl, h->d_cand, h->cand_cap, top_k, h->d_fin,
+                         b->d_scores + (size_t)c * EPI3_MAX_TOPK, b->d_trip + (size_t)c * 3 * EPI3_MAX_TOPK,
+                         b->stream));
     }
     cur = "read-back";
     cur_c = -1;
@@ -2137,6 +2106,8 @@ int epi3_batch_create(epi3_batch** out, int32_t n_cohorts, const epi3_cohort* co
         if ((e = cudaEventCreate(&ev)) != cudaSuccess) return bail(cuda_fail(e, "event create"));
     if ((e = dev_alloc((void**)&b->d_ctrls, sizeof(Ctrl) * n_cohorts)) != cudaSuccess)
         return bail(cuda_fail(e, "alloc control blocks"));
+    for (int c = 0; c < n_cohorts; ++c)
+        if ((e = launch_reset(b->d_ctrls + c, b->stream)) != cudaSuccess) return bail(cuda_fail(e, "reset"));
     if ((e = host_alloc((void**)&b->h_ctrls, sizeof(Ctrl) * n_cohorts)) != cudaSuccess)
         return bail(cuda_fail(e, "pinned control blocks"));
     b->h.assign(n_cohorts, nullptr);
@@ -2156,7 +2127,6 @@ int epi3_batch_create(epi3_batch** out, int32_t n_cohorts, const epi3_cohort* co
     }
     std::vector<int4> tiles;
     size_t cmp_need = 0;
-    b->cmp_plan.assign(n_cohorts, CmpPlan());
     for (int c = 0; c < n_cohorts; ++c) {
         epi3_handle* h = b->h[c];
         if ((rc = tune_path(b, h, &b->path[c], &b->tune_ms)) != EPI3_OK) return bail(rc);
@@ -2165,10 +2135,9 @@ int epi3_batch_create(epi3_batch** out, int32_t n_cohorts, const epi3_cohort* co
             append_tiles(h->M, 0, pairs(h->M - 1), c, tiles);
         } else if (b->path[c] == EPI3_PATH_MMA4C) {
             // its own compaction + scan launches in the graph, ranges planned now
-            CmpPlan& P = b->cmp_plan[c];
             if ((rc = ensure_yz(h)) != EPI3_OK) return bail(rc);
-            if ((rc = cmp_prepare(h, 0, pairs(h->M - 1), P)) != EPI3_OK) return bail(rc);
-            cmp_need = std::max(cmp_need, P.need);
+            if ((rc = cmp_prepare(h, 0, pairs(h->M - 1))) != EPI3_OK) return bail(rc);
+            cmp_need = std::max(cmp_need, h->plan.need);
         }
         h->path = b->path[c];
     }
@@ -2301,7 +2270,7 @@ int epi3_batch_scan(epi3_batch* b, int32_t top_k, int32_t* out_triplets, double*
     s.path = n_mma == b->n ? EPI3_PATH_MMA4 : (n_mma == 0 ? EPI3_PATH_POPC8 : EPI3_PATH_AUTO);
     s.grid = b->sm_count;
     s.block = mma_threads(b->split);
-    s.kernel_launches = b->n + (b->n_tiles > 0 ? 1 : 0) + (b->n - n_mma) + 3 * b->n;
+    s.kernel_launches = b->n + (b->n_tiles > 0 ? 1 : 0) + (b->n - n_mma) + b->n;
     // device time of the whole graph replay (scan kernels + candidate stages + read-back);
     // the scan kernels are > 99 % of it
     cudaEventElapsedTime(&s.total_ms, b->ev[0], b->ev[4]);

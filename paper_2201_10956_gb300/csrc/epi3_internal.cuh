@@ -39,7 +39,9 @@ struct Ctrl {
     // first bounded wait that ran out (0 = none): role + 1, then the tile, set and step it
     // was on (diagnostics of EPI3_ERR_TIMEOUT)
     unsigned int wait_role, wait_tile, wait_set, wait_step;
-    unsigned int pad_[3];
+    unsigned int pad_[2];
+    unsigned int seeds_done, answers_done;   // blocks of seed / answer that are done, zero between them
+    unsigned int pad2_[1];
 };
 
 struct Cand {                     // one FP32 candidate
@@ -119,12 +121,14 @@ cudaError_t launch_pack(const uint8_t* geno, const uint8_t* pheno, int M, int N,
 cudaError_t launch_scan_popc(const ScanArgs& a, int grid, int block, size_t smem, cudaStream_t st);
 size_t scan_popc_smem(const Planes& pl);
 cudaError_t scan_popc_occupancy(int block, size_t smem, int* ctas_per_sm);
-cudaError_t launch_select(Ctrl* ctrl, const Cand* cand, long long cand_cap, int top_k,
-                          float rel, float abs_, cudaStream_t st);
-cudaError_t launch_rescore(const Planes& pl, const K2Tables& k2, Ctrl* ctrl, const Cand* cand,
-                           long long cand_cap, Final* fin, int grid, cudaStream_t st);
-cudaError_t launch_final(Ctrl* ctrl, const Final* fin, int top_k, double* out_scores,
-                         int* out_trip, cudaStream_t st);
+// Starts a scan of pairs [pair_begin, pair_end): control block cleared, threshold from a sample (+inf
+// where that is shorter than the answer).  Writes into `cand`; the block's counters must be zero
+// (launch_reset once after allocation).
+cudaError_t launch_seed(const Planes& pl, const K2Tables& k2, Ctrl* ctrl, Cand* cand, long long cap,
+                        long long pair_begin, long long pair_end, int top_k, cudaStream_t st);
+// The candidate stage: the answer from the scan's candidates.
+cudaError_t launch_answer(const Planes& pl, const K2Tables& k2, Ctrl* ctrl, const Cand* cand, long long cap,
+                          int top_k, Final* fin, double* out_scores, int* out_trip, cudaStream_t st);
 cudaError_t launch_tables(const Planes& pl, const PairTables* pt, const K2Tables* k2, long long n,
                           const int* trip, int* out_counts, float* out_s32, double* out_s64,
                           Ctrl* ctrl, cudaStream_t st);

@@ -3,11 +3,12 @@
 // Some callers cannot call cudaMalloc: real-time or embedded hosts with a fixed memory
 // budget, and frameworks whose caching allocator owns the device memory (a raw
 // cudaMalloc/cudaFree there can fail or implicitly synchronise the device).  For them this
-// entry point runs the class split, the packing, the 27-cell POPC scan (the counting kernel
-// of the popc path, about 5 T sample-triplets/s on GB300; not the tensor-core form that
+// entry point runs the class split, the packing, a POPC scan (8 cells counted and 19 derived where
+// the pair tables fit the scratch beside the rest -- up to some 600 SNPs --, about 18 T
+// sample-triplets/s on GB300; else all 27 cells, about 5 T; not the tensor-core form that
 // epi3_scan picks by default), the candidate band, FP64 rescoring and the final order, with
-// every piece of scratch memory (class counts, packed bit planes, log-factorial tables,
-// control block, candidate lists) in one file-scope device array of kScratchBytes;
+// every piece of scratch memory (class counts, packed bit planes, pair tables, log-factorial
+// tables, control block, candidate lists) in one file-scope device array of kScratchBytes;
 // the log-factorial tables are staged in file-scope host arrays.  The caller passes device
 // inputs and device outputs.  The candidate list has a fixed 65536 entries and is not
 // grown: a data set with more FP32 candidates gets EPI3_ERR_OVERFLOW (epi3_scan would retry
@@ -59,6 +60,8 @@ size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct Layout {
     size_t ctrl, counts, planes, lf2, lf64, cand, fin, total;
+    size_t pt, marg;
+    bool eight;                  // the pair tables fit: count 8 cells, derive 19
 };
 
 // Offsets inside the scratch array; the planes are sized for the worst class split.
@@ -74,6 +77,10 @@ Layout layout(long long M, long long N) {
     L.cand = o;   o += up256((size_t)kNoAllocCandCap * sizeof(Cand));
     L.fin = o;    o += up256((size_t)kFinalCap * sizeof(Final));
     L.total = o;
+    const size_t np = (size_t)M * (size_t)(M - 1) / 2;
+    L.pt = o;     o += up256(2 * np * sizeof(int4));
+    L.marg = o;   o += up256((size_t)2 * M * sizeof(int2));
+    L.eight = o <= kScratchBytes;
     return L;
 }
 
@@ -172,9 +179,10 @@ int scan_noalloc(const uint8_t* geno, const uint8_t* pheno, int M, int N, int to
     k2.abs_ = std::ldexp(1.0f, -(g + 13));
 
     // scan, candidate band, FP64 rescoring, final order
-    const size_t smem = scan_popc_smem(pl);
+    const size_t smem = L.eight ? scan_popc8_smem(pl) : scan_popc_smem(pl);
     int occ = 0;
-    NA_CK(scan_popc_occupancy(128, smem, &occ), "scan occupancy");
+    if (L.eight) NA_CK(scan_popc8_occupancy(128, smem, &occ), "scan occupancy");
+    else NA_CK(scan_popc_occupancy(128, smem, &occ), "scan occupancy");
     if (occ < 1) return err(EPI3_ERR_UNSUPPORTED, "scan kernel does not fit");
     ScanArgs a{};
     a.pl = pl;
@@ -186,11 +194,21 @@ int scan_noalloc(const uint8_t* geno, const uint8_t* pheno, int M, int N, int to
     a.pair_end = (long long)(M - 1) * (M - 2) / 2;
     a.top_k = top_k;
     a.dbg = nullptr;
-    NA_CK(launch_reset(ctrl, st), "reset launch");
-    NA_CK(launch_scan_popc(a, sms * occ, 128, smem, st), "scan launch");
-    NA_CK(launch_select(ctrl, cand, kNoAllocCandCap, top_k, k2.rel, k2.abs_, st), "select launch");
-    NA_CK(launch_rescore(pl, k2, ctrl, cand, kNoAllocCandCap, fin, sms * 8, st), "rescore launch");
-    NA_CK(launch_final(ctrl, fin, top_k, out_scores, out_trip, st), "final launch");
+    if (L.eight) {
+        int4* const pt = reinterpret_cast<int4*>(base + L.pt);
+        int2* const marg = reinterpret_cast<int2*>(base + L.marg);
+        a.pt.pt = pt;
+        a.pt.marg = marg;
+        a.pt.n_pairs = (long long)M * (M - 1) / 2;
+        a.pt.n_c[0] = hc[0];
+        a.pt.n_c[1] = hc[1];
+        NA_CK(launch_pair_tables(pl, pt, marg, a.pt.n_pairs, st), "pair tables launch");
+    }
+    NA_CK(launch_seed(pl, k2, ctrl, cand, kNoAllocCandCap, 0, a.pair_end, top_k, st), "seed launch");
+    if (L.eight) NA_CK(launch_scan_popc8(a, sms * occ, 128, smem, st), "scan launch");
+    else NA_CK(launch_scan_popc(a, sms * occ, 128, smem, st), "scan launch");
+    NA_CK(launch_answer(pl, k2, ctrl, cand, kNoAllocCandCap, top_k, fin, out_scores, out_trip, st),
+          "candidate stage launch");
     NA_CK(cudaMemcpyAsync(&hctrl, ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st), "read status");
     NA_CK(cudaStreamSynchronize(st), "scan");
     if (hctrl.status & kStCandOverflow)

@@ -1,14 +1,16 @@
 // Candidate stage of the scan and the per-triplet debug kernels.
 //
 //   reset    : zero the control block, threshold = +inf.
-//   select   : exact k-th smallest FP32 score among the global candidates (radix select
-//              on the float bit patterns, which order like the non-negative values), then
-//              the rescoring band T = band_threshold(k-th).
-//   rescore  : one warp per candidate inside the band: recount its 2 x 27 table (lanes
-//              split the sample groups, warp-shuffle sums of the 54 counts), FP64 K2
-//              (Eq. 1, cell order 0..26).
-//   final    : one CTA sorts the rescored candidates by (K2, i, j, k) and writes the
-//              first top_k (Sec. III: the lowest K2 is the solution).
+//   seed     : zero the control block; threshold = band of the k-th smallest FP32 score of up to
+//              2048 triplets spread over the scan's pairs, so that the scan's first tiles need not
+//              keep everything they score.
+//   answer   : one launch for the whole candidate stage.  Every CTA finds the exact k-th smallest
+//              FP32 score among the global candidates (radix select on the float bit patterns,
+//              which order like the non-negative values) and the rescoring band; one warp per
+//              candidate inside the band recounts its 2 x 27 table (lanes split the sample groups,
+//              warp-shuffle sums of the 54 counts) and takes its FP64 K2 (Eq. 1, cell order
+//              0..26); the last CTA to finish sorts them by (K2, i, j, k) and writes the first
+//              top_k (Sec. III: the lowest K2 is the solution).
 //   tables   : warp per listed triplet, tables and/or FP32 and FP64 K2.
 #include "epi3_internal.cuh"
 
@@ -16,8 +18,10 @@ namespace epi3 {
 
 namespace {
 
-constexpr int kSelThreads = 1024;
-constexpr int kFinThreads = 1024;
+constexpr int kAnsThreads = 512;
+constexpr int kAnsCtas = 32;
+constexpr int kSeedThreads = 256;
+constexpr int kSeedMax = 2048;        // seed triplets, at most
 
 __device__ __forceinline__ int popc4(uint4 a, uint4 b, uint4 c) {
     return __popc(a.x & b.x & c.x) + __popc(a.y & b.y & c.y) + __popc(a.z & b.z & c.z) +
@@ -114,73 +118,126 @@ __global__ void reset_kernel(Ctrl* ctrl) {
     *ctrl = z;
 }
 
-__global__ void __launch_bounds__(kSelThreads)
-select_kernel(Ctrl* ctrl, const Cand* __restrict__ cand, long long cap, int top_k, float rel,
-              float abs_) {
+// The rank-th smallest (1-based) of n non-negative floats `stride` floats apart, by all threads of
+// the block: four passes over eight bits each, the bin of a pass found by one warp (a single thread
+// walking 256 bins took four microseconds a pass).
+__device__ float block_kth(const float* v, int stride, long long n, unsigned rank) {
     __shared__ unsigned hist[256];
     __shared__ unsigned s_prefix, s_rank;
-    const int tid = threadIdx.x;
-    const long long n = min((long long)ctrl->n_cand, cap);
-    if (n < top_k) {
-        if (tid == 0) atomicOr(&ctrl->status, kStInternal);
-        return;
-    }
+    const int tid = threadIdx.x, lane = tid & 31;
     if (tid == 0) {
         s_prefix = 0u;
-        s_rank = (unsigned)top_k;  // 1-based rank still to find inside the current prefix
+        s_rank = rank;
     }
     unsigned mask = 0u;
     for (int shift = 24; shift >= 0; shift -= 8) {
-        for (int b = tid; b < 256; b += kSelThreads) hist[b] = 0u;
+        for (int b = tid; b < 256; b += blockDim.x) hist[b] = 0u;
         __syncthreads();
-        const unsigned prefix = s_prefix;
-        for (long long idx = tid; idx < n; idx += kSelThreads) {
-            const unsigned u = __float_as_uint(cand[idx].s);
+        const unsigned prefix = s_prefix, want = s_rank;
+        for (long long e = tid; e < n; e += blockDim.x) {
+            const unsigned u = __float_as_uint(v[e * stride]);
             if ((u & mask) == prefix) atomicAdd(&hist[(u >> shift) & 255u], 1u);
         }
         __syncthreads();
-        if (tid == 0) {
-            unsigned cum = 0u, rank = s_rank;
-            int digit = 255;
-            for (int b = 0; b < 256; ++b) {
-                if (cum + hist[b] >= rank) {
-                    digit = b;
-                    break;
-                }
-                cum += hist[b];
+        if (tid < 32) {
+            unsigned c[8], sum = 0u;
+#pragma unroll
+            for (int b = 0; b < 8; ++b) sum += c[b] = hist[8 * lane + b];
+            unsigned incl = sum;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const unsigned o = __shfl_up_sync(0xffffffffu, incl, d);
+                if (lane >= d) incl += o;
             }
-            s_rank = rank - cum;
-            s_prefix = prefix | ((unsigned)digit << shift);
+            unsigned before = incl - sum;
+            if (before < want && want <= incl) {
+                int b = 0;
+#pragma unroll
+                for (int t = 0; t < 7; ++t)
+                    if (b == t && before + c[t] < want) {
+                        before += c[t];
+                        ++b;
+                    }
+                s_rank = want - before;
+                s_prefix = prefix | ((unsigned)(8 * lane + b) << shift);
+            }
         }
         mask |= 255u << shift;
         __syncthreads();
     }
-    if (tid == 0) {
-        const float kth = __uint_as_float(s_prefix);
-        ctrl->kth = kth;
-        ctrl->t_final = band_threshold(kth, rel, abs_);
-    }
+    return __uint_as_float(s_prefix);
 }
 
-__global__ void __launch_bounds__(256)
-rescore_kernel(Planes pl, K2Tables k2, Ctrl* ctrl, const Cand* __restrict__ cand, long long cap,
-               Final* __restrict__ fin) {
-    const long long n = min((long long)ctrl->n_cand, cap);
-    const float t = ctrl->t_final;
+// This lane's cell of a table every lane holds.
+__device__ __forceinline__ void lane_cell(const int* r0, const int* r1, int* a, int* b) {
     const int lane = threadIdx.x & 31;
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long idx = warp; idx < n; idx += nwarps) {
-        const Cand e = cand[idx];
-        if (!(e.s <= t)) continue;
-        int r0[kCells], r1[kCells];
-        warp_table(pl, e.i, e.j, e.k, r0, r1);
-        if (lane == 0) {
-            const double s = k2_f64(r0, r1, k2.lf64);
-            const unsigned pos = atomicAdd(&ctrl->n_final, 1u);
-            if (pos < (unsigned)kFinalCap) fin[pos] = Final{s, pack_key(e.i, e.j, e.k)};
-            else atomicOr(&ctrl->status, kStFinalOverflow);
+    *a = 0;
+    *b = 0;
+#pragma unroll
+    for (int q = 0; q < kCells; ++q)
+        if (q == lane) {
+            *a = r0[q];
+            *b = r1[q];
         }
+}
+// k2_f64 and k2_f32 by one warp: a lane looks up its cell, the terms are added in cell order.
+__device__ double warp_k2_f64(const int* r0, const int* r1, const double* lf64) {
+    int a, b;
+    lane_cell(r0, r1, &a, &b);
+    const double t = __dsub_rn(__dsub_rn(lf64[a + b + 1], lf64[a]), lf64[b]);
+    double s = 0.0;
+#pragma unroll
+    for (int q = 0; q < kCells; ++q) s = __dadd_rn(s, __shfl_sync(0xffffffffu, t, q));
+    return s;
+}
+__device__ float warp_k2_f32(const int* r0, const int* r1, const float2* lf2) {
+    int a, b;
+    lane_cell(r0, r1, &a, &b);
+    const float2 u = __ldg(lf2 + a + b + 1), v = __ldg(lf2 + a), w = __ldg(lf2 + b);
+    const float th = __fsub_rn(__fsub_rn(u.x, v.x), w.x), tl = __fsub_rn(__fsub_rn(u.y, v.y), w.y);
+    float ah = 0.f, al = 0.f;
+#pragma unroll
+    for (int q = 0; q < kCells; ++q) {
+        ah = __fadd_rn(ah, __shfl_sync(0xffffffffu, th, q));
+        al = __fadd_rn(al, __shfl_sync(0xffffffffu, tl, q));
+    }
+    return __fadd_rn(ah, al);
+}
+
+// True in every thread of the last block of the grid to get here (*count: zero before, and after).
+__device__ bool last_block(unsigned* count) {
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_last = atomicAdd(count, 1u) == gridDim.x - 1;
+        if (s_last) *count = 0u;
+    }
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last;
+}
+
+// Warp w takes the pair pb + w step and one third SNP of it: distinct triplets.
+__global__ void __launch_bounds__(kSeedThreads)
+seed_kernel(Planes pl, K2Tables k2, Ctrl* ctrl, float* __restrict__ scores, long long pb, long long step, int n,
+            int top_k) {
+    const int w = blockIdx.x * (kSeedThreads / 32) + (threadIdx.x >> 5);
+    if (w < n) {
+        int i, j;
+        decode_pair(pb + w * step, &i, &j);
+        const int k = j + 1 + (int)((unsigned)w * 2654435761u % (unsigned)(pl.M - 1 - j));
+        int r0[kCells], r1[kCells];
+        warp_table(pl, i, j, k, r0, r1);
+        const float s = warp_k2_f32(r0, r1, k2.lf2);
+        if ((threadIdx.x & 31) == 0) scores[w] = s;
+    }
+    if (!last_block(&ctrl->seeds_done)) return;
+    const float kth = block_kth(scores, 1, n, (unsigned)top_k);
+    if (threadIdx.x == 0) {
+        Ctrl z = {};
+        z.thr = __float_as_uint(band_threshold(kth, k2.rel, k2.abs_));
+        *ctrl = z;
     }
 }
 
@@ -188,20 +245,45 @@ __device__ __forceinline__ bool fin_less(const Final& a, const Final& b) {
     return a.s < b.s || (a.s == b.s && a.key < b.key);
 }
 
-__global__ void __launch_bounds__(kFinThreads)
-final_kernel(Ctrl* ctrl, const Final* __restrict__ fin, int top_k, double* out_scores,
-             int* out_trip) {
+__global__ void __launch_bounds__(kAnsThreads)
+answer_kernel(Planes pl, K2Tables k2, Ctrl* ctrl, const Cand* __restrict__ cand, long long cap, int top_k,
+              Final* __restrict__ fin, double* __restrict__ out_scores, int* __restrict__ out_trip) {
+    const long long n = min((long long)ctrl->n_cand, cap);
+    const int lane = threadIdx.x & 31, tid = threadIdx.x;
+    if (n < top_k) {
+        if (tid == 0 && blockIdx.x == 0) atomicOr(&ctrl->status, kStInternal);
+    } else {
+        const float kth = block_kth(&cand->s, sizeof(Cand) / sizeof(float), n, (unsigned)top_k);
+        const float t = band_threshold(kth, k2.rel, k2.abs_);
+        if (tid == 0 && blockIdx.x == 0) {
+            ctrl->kth = kth;
+            ctrl->t_final = t;
+        }
+        const long long nwarps = (long long)gridDim.x * (kAnsThreads / 32);
+        for (long long idx = blockIdx.x + (long long)gridDim.x * (tid >> 5); idx < n; idx += nwarps) {
+            const Cand e = cand[idx];
+            if (!(e.s <= t)) continue;
+            int r0[kCells], r1[kCells];
+            warp_table(pl, e.i, e.j, e.k, r0, r1);
+            const double s = warp_k2_f64(r0, r1, k2.lf64);
+            if (lane == 0) {
+                const unsigned pos = atomicAdd(&ctrl->n_final, 1u);
+                if (pos < (unsigned)kFinalCap) fin[pos] = Final{s, pack_key(e.i, e.j, e.k)};
+                else atomicOr(&ctrl->status, kStFinalOverflow);
+            }
+        }
+    }
+    if (!last_block(&ctrl->answers_done)) return;
     extern __shared__ Final sf[];
-    const int tid = threadIdx.x;
-    const int n = (int)min(ctrl->n_final, (unsigned)kFinalCap);
-    int size = 64;
-    while (size < n) size <<= 1;
-    for (int idx = tid; idx < size; idx += kFinThreads)
-        sf[idx] = (idx < n) ? fin[idx] : Final{__longlong_as_double(0x7ff0000000000000LL), ~0ULL};
+    const int nf = (int)min(*(volatile unsigned*)&ctrl->n_final, (unsigned)kFinalCap);
+    int size = 32;
+    while (size < nf) size <<= 1;
+    const Final last = Final{__longlong_as_double(0x7ff0000000000000LL), ~0ULL};
+    for (int idx = tid; idx < size; idx += kAnsThreads) sf[idx] = idx < nf ? fin[idx] : last;
     __syncthreads();
     for (int sz = 2; sz <= size; sz <<= 1) {
         for (int stride = sz >> 1; stride > 0; stride >>= 1) {
-            for (int t = tid; t < size / 2; t += kFinThreads) {
+            for (int t = tid; t < size / 2; t += kAnsThreads) {
                 const int lo = 2 * t - (t & (stride - 1));
                 const int hi = lo + stride;
                 const bool up = ((lo & sz) == 0);
@@ -214,8 +296,10 @@ final_kernel(Ctrl* ctrl, const Final* __restrict__ fin, int top_k, double* out_s
             __syncthreads();
         }
     }
-    const int nout = min(top_k, n);
-    for (int r = tid; r < nout; r += kFinThreads) {
+    // a failed scan (or one that runs again with a longer list) leaves the outputs alone
+    const int status = *(volatile int*)&ctrl->status;
+    const int nout = status ? 0 : min(top_k, nf);
+    for (int r = tid; r < nout; r += kAnsThreads) {
         const Final e = sf[r];
         out_scores[r] = e.s;
         out_trip[3 * r + 0] = (int)(e.key >> 42);
@@ -224,7 +308,7 @@ final_kernel(Ctrl* ctrl, const Final* __restrict__ fin, int top_k, double* out_s
     }
     if (tid == 0) {
         ctrl->n_out = (unsigned)nout;
-        if (n < top_k) atomicOr(&ctrl->status, kStInternal);
+        if (nf < top_k) atomicOr(&ctrl->status, kStInternal);
     }
 }
 
@@ -294,25 +378,25 @@ cudaError_t launch_approx_error(const double* lf64, int n_lf, double* out, cudaS
     return cudaGetLastError();
 }
 
-cudaError_t launch_select(Ctrl* ctrl, const Cand* cand, long long cap, int top_k, float rel,
-                          float abs_, cudaStream_t st) {
-    select_kernel<<<1, kSelThreads, 0, st>>>(ctrl, cand, cap, top_k, rel, abs_);
+cudaError_t launch_seed(const Planes& pl, const K2Tables& k2, Ctrl* ctrl, Cand* cand, long long cap,
+                        long long pair_begin, long long pair_end, int top_k, cudaStream_t st) {
+    // the scores go where the candidates will: the scan has not started
+    long long n = pair_end - pair_begin;
+    if (n > kSeedMax) n = kSeedMax;
+    if (n > cap) n = cap;
+    if (n < top_k) return launch_reset(ctrl, st);
+    const int per = kSeedThreads / 32;
+    seed_kernel<<<(unsigned)((n + per - 1) / per), kSeedThreads, 0, st>>>(
+        pl, k2, ctrl, reinterpret_cast<float*>(cand), pair_begin, (pair_end - pair_begin) / n, (int)n, top_k);
     return cudaGetLastError();
 }
 
-cudaError_t launch_rescore(const Planes& pl, const K2Tables& k2, Ctrl* ctrl, const Cand* cand,
-                           long long cap, Final* fin, int grid, cudaStream_t st) {
-    rescore_kernel<<<grid, 256, 0, st>>>(pl, k2, ctrl, cand, cap, fin);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_final(Ctrl* ctrl, const Final* fin, int top_k, double* out_scores,
-                         int* out_trip, cudaStream_t st) {
+cudaError_t launch_answer(const Planes& pl, const K2Tables& k2, Ctrl* ctrl, const Cand* cand, long long cap,
+                          int top_k, Final* fin, double* out_scores, int* out_trip, cudaStream_t st) {
     const size_t smem = (size_t)kFinalCap * sizeof(Final);
-    cudaError_t e = cudaFuncSetAttribute(final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    cudaError_t e = cudaFuncSetAttribute(answer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    final_kernel<<<1, kFinThreads, smem, st>>>(ctrl, fin, top_k, out_scores, out_trip);
+    answer_kernel<<<kAnsCtas, kAnsThreads, smem, st>>>(pl, k2, ctrl, cand, cap, top_k, fin, out_scores, out_trip);
     return cudaGetLastError();
 }
 
