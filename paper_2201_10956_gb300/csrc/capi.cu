@@ -237,6 +237,7 @@ struct CmpPlan {
     std::vector<int> range_group;   // first group of each range
     std::vector<int> range_runs;
     size_t need = 0;                // buffer bytes of the largest range
+    int most = 0;                   // first SNPs of the longest range
     int i_hi = 0;                   // first SNPs [0, i_hi)
     double chunks_total = 0.0, steps_total = 0.0;
 };
@@ -291,6 +292,9 @@ struct epi3_handle {
     unsigned long long* d_prof = nullptr;
     uint8_t* d_cmp = nullptr;     // compacted chunks of the sample-compacted tensor form
     size_t cmp_bytes = 0;
+    uint4* d_rows = nullptr;      // what each sample contributes to each 64-SNP block
+    uint32_t* d_list = nullptr;   // the counted samples of a range's first SNPs
+    size_t list_len = 0;
     size_t cmp_cap = (size_t)2 << 30;  // option "cmp_buffer_mb": bytes of compacted chunks at once
     CmpFirst* d_firsts = nullptr; // per first SNP: chunk bases, K-steps, tiles
     CmpGroup* d_groups = nullptr; // groups of first SNPs that a run of tiles covers
@@ -336,6 +340,8 @@ void release(epi3_handle* h) {
     dev_free(h->d_margf, synced);
     dev_free(h->d_oh, synced);
     dev_free(h->d_cmp, synced);
+    dev_free(h->d_rows, synced);
+    dev_free(h->d_list, synced);
     dev_free(h->d_firsts, synced);
     dev_free(h->d_groups, synced);
     dev_free(h->d_tiles, synced);
@@ -605,11 +611,16 @@ int ensure_pair_floats(epi3_handle* h) {
     return EPI3_OK;
 }
 
-int ensure_yz(epi3_handle* h) {
+// Inputs of the compacted form that depend on the data set only.
+int ensure_cmp(epi3_handle* h) {
     if (!h->d_yz) {
         CK(dev_alloc((void**)&h->d_yz, sizeof(float4) * 16 * (size_t)yz_blocks(h->M)), "alloc paired tables");
         CK(launch_pair_yz(h->d_pt, h->ptab.n_pairs, h->M, h->bound.minor, h->d_yz, h->stream),
            "paired tables launch");
+    }
+    if (!h->d_rows) {
+        CK(dev_alloc((void**)&h->d_rows, sample_rows_bytes(h->pl)), "alloc sample rows");
+        CK(launch_sample_rows(h->pl, h->d_rows, h->stream), "sample rows launch");
     }
     return EPI3_OK;
 }
@@ -944,7 +955,10 @@ void plan_cmp(const epi3_handle* h, long long pb, long long pe, CmpPlan& P) {
         }
         f.drop = cmp_drop(n[0][0] + n[1][0], n[0][1] + n[1][1], n[0][2] + n[1][2]);
         for (int c = 0; c < 2; ++c)
-            for (int s = 0; s < 2; ++s) f.ks[2 * c + s] = n[c][cmp_geno(f.drop, s)] / 256 + 1;  // + the bias sample
+            for (int s = 0; s < 2; ++s) {
+                f.cnt[2 * c + s] = n[c][cmp_geno(f.drop, s)];
+                f.ks[2 * c + s] = f.cnt[2 * c + s] / 256 + 1;  // + the bias sample
+            }
         f.tiles = cmp_tiles_of(M, f.b_lo, jb_end);
         const double ch = (double)cmp_chunks_of(f, M);
         P.chunks_total += ch;
@@ -990,6 +1004,7 @@ void plan_cmp(const epi3_handle* h, long long pb, long long pe, CmpPlan& P) {
             }
         }
         P.need = std::max(P.need, (size_t)chunks * 16384);
+        P.most = std::max(P.most, ie - P.range_start.back());
         i = ie;
     }
     if (!P.range_start.empty()) P.range_runs.push_back(runs);
@@ -1065,6 +1080,14 @@ int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int 
         CK(dev_alloc((void**)&h->d_cmp, need), "alloc compacted chunks");
         h->cmp_bytes = need;
     }
+    const size_t len = (size_t)P.most * h->N;
+    if (h->list_len < len) {
+        dev_free(h->d_list);
+        h->d_list = nullptr;
+        h->list_len = 0;
+        CK(dev_alloc((void**)&h->d_list, sizeof(uint32_t) * len), "alloc sample lists");
+        h->list_len = len;
+    }
     const int grid = h->sm_count;
     const int n_ranges = (int)range_start.size();
     float compact_ms = 0.f;
@@ -1088,7 +1111,8 @@ int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int 
             const int i0 = range_start[r];
             const int n = (r + 1 < n_ranges ? range_start[r + 1] : i_hi) - i0;
             CK(cudaEventRecord(h->cmp_ev[2 * r], h->stream), "event");
-            CK(launch_compact(h->pl, h->d_firsts + i0, i0, n, h->d_cmp, h->stream), "compaction launch");
+            CK(launch_compact(h->pl, h->d_rows, h->d_firsts + i0, i0, n, h->N0, h->N, h->d_list, h->d_cmp, h->stream),
+               "compaction launch");
             CK(cudaEventRecord(h->cmp_ev[2 * r + 1], h->stream), "event");
             CmpArgs a = cmp_args(h, cohort_of(h, pb, pe, top_k), i0, P.range_group[r], P.range_runs[r],
                                  h->d_cmp);
@@ -1116,7 +1140,7 @@ int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int 
     s.grid = grid;
     s.block = scan_cmp_threads();
     s.form = cmp_paired(h) ? 2 : 1;
-    s.kernel_launches = 2 * n_ranges + 2;
+    s.kernel_launches = 3 * n_ranges + 2;
     s.wait_loader = s.wait_mma_operands = s.wait_mma_accum = s.wait_producers = s.wait_epilogue = 0.f;
     s.wait_producers_tmem = s.mma_issue = 0.f;
     s.compact_ms = compact_ms;
@@ -1181,7 +1205,7 @@ int scan_impl(epi3_handle* h, long long pb, long long pe, int top_k, int32_t* ou
     }
     if (path == EPI3_PATH_MMA4C) {
         int rc = ensure_pair_tables(h);
-        if (rc == EPI3_OK) rc = ensure_yz(h);
+        if (rc == EPI3_OK) rc = ensure_cmp(h);
         if (rc != EPI3_OK) return rc;
         return scan_cmp_impl(h, pb, pe, nt, top_k, out_trip, out_scores, n_out);
     }
@@ -1695,6 +1719,7 @@ struct epi3_batch {
     // compacted-form cohorts (ranges of first SNPs in their handles' plans) all compact into one
     // shared buffer
     uint8_t* d_cmp = nullptr;
+    uint32_t* d_list = nullptr;
     Ctrl* d_ctrls = nullptr;            // one control block per cohort, contiguous
     Ctrl* h_ctrls = nullptr;            // pinned
     CohortDev* d_cds = nullptr;
@@ -1729,6 +1754,7 @@ void batch_release(epi3_batch* b) {
     dev_free(b->d_cds, synced);
     dev_free(b->d_tiles, synced);
     dev_free(b->d_cmp, synced);
+    dev_free(b->d_list, synced);
     dev_free(b->d_scores, synced);
     dev_free(b->d_trip, synced);
     host_free(b->h_scores);
@@ -2020,7 +2046,7 @@ int batch_capture(epi3_batch* b, int top_k) {
         for (size_t r = 0; r < rs.size(); ++r) {
             const int i0 = rs[r];
             const int n = (r + 1 < rs.size() ? rs[r + 1] : P.i_hi) - i0;
-            ok(launch_compact(h->pl, h->d_firsts + i0, i0, n, b->d_cmp, b->stream));
+            ok(launch_compact(h->pl, h->d_rows, h->d_firsts + i0, i0, n, h->N0, h->N, b->d_list, b->d_cmp, b->stream));
             const CmpArgs a = cmp_args(h, cds[c], i0, P.range_group[r], P.range_runs[r], b->d_cmp);
             ok(launch_scan_cmp(a, b->sm_count, b->stream, false, cmp_paired(h)));
         }
@@ -2126,7 +2152,7 @@ int epi3_batch_create(epi3_batch** out, int32_t n_cohorts, const epi3_cohort* co
         if ((rc = ensure_pair_tables(h)) != EPI3_OK) return bail(rc);
     }
     std::vector<int4> tiles;
-    size_t cmp_need = 0;
+    size_t cmp_need = 0, list_need = 0;
     for (int c = 0; c < n_cohorts; ++c) {
         epi3_handle* h = b->h[c];
         if ((rc = tune_path(b, h, &b->path[c], &b->tune_ms)) != EPI3_OK) return bail(rc);
@@ -2135,14 +2161,17 @@ int epi3_batch_create(epi3_batch** out, int32_t n_cohorts, const epi3_cohort* co
             append_tiles(h->M, 0, pairs(h->M - 1), c, tiles);
         } else if (b->path[c] == EPI3_PATH_MMA4C) {
             // its own compaction + scan launches in the graph, ranges planned now
-            if ((rc = ensure_yz(h)) != EPI3_OK) return bail(rc);
+            if ((rc = ensure_cmp(h)) != EPI3_OK) return bail(rc);
             if ((rc = cmp_prepare(h, 0, pairs(h->M - 1))) != EPI3_OK) return bail(rc);
             cmp_need = std::max(cmp_need, h->plan.need);
+            list_need = std::max(list_need, (size_t)h->plan.most * h->N);
         }
         h->path = b->path[c];
     }
     if (cmp_need && (e = dev_alloc((void**)&b->d_cmp, cmp_need)) != cudaSuccess)
         return bail(cuda_fail(e, "alloc compacted chunks"));
+    if (list_need && (e = dev_alloc((void**)&b->d_list, sizeof(uint32_t) * list_need)) != cudaSuccess)
+        return bail(cuda_fail(e, "alloc sample lists"));
     b->n_tiles = (long long)tiles.size();
     // the tensor launch's form (plain or register-split) is measured on the first scan, unless
     // EPI3_BATCH_FORM forces one

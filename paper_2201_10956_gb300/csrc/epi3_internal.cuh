@@ -233,6 +233,7 @@ constexpr int kCmpSets = 4;      // (class, one of the two counted genotypes of 
 struct CmpFirst {
     long long base[kCmpSets];
     int ks[kCmpSets];
+    int cnt[kCmpSets];           // samples of each set
     int drop;
     int b_lo;                    // first 64-SNP block compacted: the first j block of the tiles
     int tiles;                   // tiles of this first SNP
@@ -317,9 +318,13 @@ inline long long cmp_chunks_of(const CmpFirst& f, int M) {
 int cmp_tiles_of(int M, int b_lo, int jb_end); // tiles (64 j x 32 k) of one first SNP
 size_t scan_cmp_smem();
 int scan_cmp_threads();          // threads per CTA of the compacted scan
-// compaction of first SNPs i0 .. i0 + n_first - 1 into cmp (chunk indices from firsts)
-cudaError_t launch_compact(const Planes& pl, const CmpFirst* firsts, int i0, int n_first,
-                           uint8_t* cmp, cudaStream_t st);
+// what each sample contributes to each 64-SNP block (built once per data set)
+size_t sample_rows_bytes(const Planes& pl);
+cudaError_t launch_sample_rows(const Planes& pl, uint4* rows, cudaStream_t st);
+// compaction of first SNPs i0 .. i0 + n_first - 1 into cmp (chunk indices from firsts); n0 controls of
+// n samples; list: n_first * n entries of scratch
+cudaError_t launch_compact(const Planes& pl, const uint4* rows, const CmpFirst* firsts, int i0, int n_first,
+                           int n0, int n, uint32_t* list, uint8_t* cmp, cudaStream_t st);
 // instrumented: table checksums / wait profile; paired: the two-triplets-per-lane epilogue
 cudaError_t launch_scan_cmp(const CmpArgs& a, int grid, cudaStream_t st, bool instrumented, bool paired);
 

@@ -46,176 +46,166 @@
 
 #include "epi3_internal.cuh"
 #include "tc_common.cuh"
-#include "bit_compress.cuh"
 
 namespace epi3 {
 
 namespace {
 
 constexpr int kCmpChunk = 16384;         // one compacted chunk: 128 rows (m, z) x 256 samples
-constexpr int kMaskWords = 128;          // selection words staged per pass of the compaction
-constexpr int kSlabBytes = 32 * 128;     // one warp's 32 rows of a chunk: 4 KB, contiguous
 
-}  // namespace
-
-namespace {
-
-// One compacted output stream of a thread: 32-bit words of compacted samples, written one at
-// a time as 16 E2M1 bytes into unit (word % 8) of the thread's row in step (word / 8).
-struct CmpStream {
-    unsigned long long acc;     // pending bits, low first
-    int fill;                   // pending bit count
-    int word;                   // words written
-};
-
-// A word goes to the warp's shared-memory image of its 32 rows of the current chunk (the same
-// 128B-swizzled layout); when the K-step's eighth word is in, the warp writes the 4 KB slab out
-// with contiguous 16-byte stores (every thread of the CTA emits at the same points: the bit
-// counts per word are the CTA's).
-__device__ __forceinline__ void cmp_emit(uint8_t* set_base, uint8_t* slab, int row, CmpStream& st,
-                                         uint32_t w) {
-    uint4 v;
-    v.x = byte_to_e2m1(w);
-    v.y = byte_to_e2m1(w >> 8);
-    v.z = byte_to_e2m1(w >> 16);
-    v.w = byte_to_e2m1(w >> 24);
-    const uint32_t u = (uint32_t)(st.word & 7);
-    *reinterpret_cast<uint4*>(slab + sw128_off((uint32_t)(row & 31), u)) = v;
-    if (u == 7) {  // uniform across the warp
-        __syncwarp();
-        uint8_t* const dst = set_base + (size_t)(st.word >> 3) * kCmpChunk + (size_t)(row & ~31) * 128;
-        const int lane = row & 31;
+// 32 x 32 bit transpose across a warp: bit t of lane r's x becomes bit r of lane t's.
+__device__ __forceinline__ uint32_t warp_transpose(uint32_t x) {
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-        for (int j = 0; j < kSlabBytes / 512; ++j) {
-            const int off = 16 * (lane + 32 * j);
-            *reinterpret_cast<uint4*>(dst + off) = *reinterpret_cast<const uint4*>(slab + off);
-        }
-        __syncwarp();
+    for (int k = 16; k >= 1; k >>= 1) {
+        const uint32_t m = k == 16 ? 0x0000FFFFu : k == 8 ? 0x00FF00FFu : k == 4 ? 0x0F0F0F0Fu
+                         : k == 2 ? 0x33333333u : 0x55555555u;
+        const uint32_t y = __shfl_xor_sync(0xffffffffu, x, k);
+        x = lane & k ? (x & ~m) | ((y >> k) & m) : (x & m) | ((y << k) & ~m);
     }
-    ++st.word;
+    return x;
 }
 
-__device__ __forceinline__ void cmp_push(uint8_t* set_base, uint8_t* slab, int row, CmpStream& st,
-                                         uint32_t bits, int n) {
-    st.acc |= (unsigned long long)bits << st.fill;
-    st.fill += n;
-    if (st.fill >= 32) {
-        cmp_emit(set_base, slab, row, st, (uint32_t)st.acc);
-        st.acc >>= 32;
-        st.fill -= 32;
-    }
-}
-
-constexpr int kCompactThreads = 128;     // one row (SNP, genotype) of the 64-SNP block per thread
-
-// Push the bits of one 32-sample word selected by a set's mask: compress by the mask (Hacker's
-// Delight 7-4, masks prepared once per word by cmp_masks), append to the stream, emit each full
-// word.
-__device__ __forceinline__ void cmp_word(uint8_t* set_base, uint8_t* slab, int row, CmpStream& st,
-                                         uint32_t x, uint32_t mask, const uint32_t* mv, int n) {
-    if (n == 0) return;
-    cmp_push(set_base, slab, row, st, n == 32 ? x : cmp_bits(x, mask, mv), n);
-}
-
-// One selection word's masks for both sets, read with four 16-byte shared-memory loads:
-// {mask0, mask1, pop0, pop1}, mv0[0..3], mv1[0..3], {mv0[4], mv1[4], -, -}.
-struct MaskWord {
-    uint4 q[4];
-};
-
-// Rows of a chunk come in 16-row groups: row 16 G + 8 z + r holds SNP m = 64 b + 8 G + r with
-// genotype z (8 SNPs of genotype 0, then the same 8 of genotype 1), so that a 16x256b
-// tensor-memory load hands a thread both genotype rows of one SNP (see the epilogue).
-// CTA (b, i - i0, c), 128 threads: thread r writes row r of every chunk of block b for the two
-// sets (c, 0) and (c, 1) of first SNP i: the bits [g_m = z] of the class-c samples whose g_i is
-// the set's counted genotype, in sample order, then the bias sample, then zeros to the set's
-// K-steps.
-// Plane words come four at a time (one 16-byte load per 128 samples, the next one in flight
-// while the current one is compressed); each word's masks of both sets come in four 16-byte
-// shared-memory loads.
-__global__ void __launch_bounds__(kCompactThreads)
-compact_kernel(Planes pl, const CmpFirst* __restrict__ firsts, int i0, uint8_t* __restrict__ cmp) {
-    __shared__ MaskWord s_w[kMaskWords];
-    __shared__ __align__(128) uint8_t s_slab[2][kCompactThreads / 32][kSlabBytes];
-    const int b = blockIdx.x, i = i0 + (int)blockIdx.y, c = (int)blockIdx.z;
-    // the fields this CTA needs, read in place (a local copy indexed by the class would live in
-    // local memory)
-    const CmpFirst* const fp = firsts + blockIdx.y;
-    const int b_lo = fp->b_lo;
-    if (b < b_lo) return;  // whole CTA: no block before the first SNP's successors
-    const int ks0 = fp->ks[2 * c], ks1 = fp->ks[2 * c + 1];
-    const long long fb0 = fp->base[2 * c], fb1 = fp->base[2 * c + 1];
-    const int drop = fp->drop;
+// ------------------------------------------------------------------ compaction
+// The compaction gathers samples: what one sample contributes to a 64-SNP block is 16 bytes, the
+// genotype-0 and genotype-1 bits of the block's SNPs (rows[c][b][s], built once per data set), and
+// 32 gathered samples turn into a K-step unit of all 128 operand rows by four bit transposes across
+// a warp (80 instructions for 128 words).  Extracting the selected bits of every row's plane words
+// instead cost 40 instructions a source word and set, for 0.19 output words.
+//
+// Warp: one 32-sample word of class c, one block: planes -> rows.
+__global__ void __launch_bounds__(256)
+sample_rows_kernel(Planes pl, int nblk, uint4* __restrict__ rows) {
+    const int lane = threadIdx.x & 31;
+    const int words0 = 4 * pl.W4[0], words = words0 + 4 * pl.W4[1];
+    const long long n = (long long)words * nblk;
     const int M = pl.M;
-    const int r = threadIdx.x, z = (r >> 3) & 1;
-    const int m = 64 * b + 8 * (r >> 4) + (r & 7);
-    const long long coff = c ? pl.coff[1] : pl.coff[0];
-    const int W4 = c ? pl.W4[1] : pl.W4[0];
-    const int W = 4 * W4;                       // 32-sample words of the class
-    const int Nc = 128 * W4 - (c ? pl.pad[1] : pl.pad[0]);
-    uint8_t* const base0 = cmp + (size_t)(fb0 + (long long)(b - b_lo) * ks0) * kCmpChunk;
-    uint8_t* const base1 = cmp + (size_t)(fb1 + (long long)(b - b_lo) * ks1) * kCmpChunk;
-    CmpStream s0{0ull, 0, 0}, s1{0ull, 0, 0};   // sets (c, 0) and (c, 1)
-    uint8_t* const slab0 = s_slab[0][r >> 5];
-    uint8_t* const slab1 = s_slab[1][r >> 5];
-    const uint4* const pc = pl.planes + coff;   // [plane][group][SNP] of 4 words
-    const uint32_t* const prow = reinterpret_cast<const uint32_t*>(pc);
-    const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
-    for (int w0 = 0; w0 < W; w0 += kMaskWords) {
-        const int nw = min(kMaskWords, W - w0);   // a multiple of 4
-        __syncthreads();  // the previous pass's masks are no longer read
-        for (int w = threadIdx.x; w < nw; w += blockDim.x) {
-            // word w0 + w of planes 0 and 1 of SNP i: group (w0 + w) / 4, word (w0 + w) % 4
-            const int ww = w0 + w;
-            const uint32_t g0 = prow[((size_t)(ww >> 2) * M + i) * 4 + (ww & 3)];
-            const uint32_t g1 = prow[((size_t)(W4 + (ww >> 2)) * M + i) * 4 + (ww & 3)];
+    for (long long t = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); t < n; t += (long long)gridDim.x * 8) {
+        const int b = (int)(t / words), ww = (int)(t % words);
+        const int c = ww >= words0 ? 1 : 0, w = c ? ww - words0 : ww;
+        const int W4 = c ? pl.W4[1] : pl.W4[0];
+        const uint32_t* const p =
+            reinterpret_cast<const uint32_t*>(pl.planes + (c ? pl.coff[1] : pl.coff[0])) + (w & 3);
+        uint32_t x[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {   // genotype e / 2, SNP half e % 2
+            const int m = 64 * b + 32 * (e & 1) + lane;
+            x[e] = m < M ? __ldg(p + ((size_t)((e >> 1) * W4 + (w >> 2)) * M + m) * 4) : 0u;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[e] = warp_transpose(x[e]);
+        rows[((size_t)b * words + ww) * 32 + lane] = make_uint4(x[0], x[1], x[2], x[3]);
+    }
+}
+
+// CTA (f, c): the class-c samples of each counted genotype of first SNP i0 + f, ascending, into
+// list + f N + (class 1: N0): slot 0's, then slot 1's.
+__global__ void __launch_bounds__(256)
+sample_list_kernel(Planes pl, const CmpFirst* __restrict__ firsts, int i0, int n0, int n,
+                   uint32_t* __restrict__ list) {
+    __shared__ uint32_t s_warp[8];
+    const int f = blockIdx.x, c = blockIdx.y, i = i0 + f, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int W4 = c ? pl.W4[1] : pl.W4[0], W = 4 * W4, Nc = c ? n - n0 : n0, M = pl.M;
+    const int drop = firsts[f].drop;
+    uint32_t* const l0 = list + (size_t)f * n + (c ? n0 : 0);
+    uint32_t* const l1 = l0 + firsts[f].cnt[2 * c];
+    const uint32_t* const p = reinterpret_cast<const uint32_t*>(pl.planes + (c ? pl.coff[1] : pl.coff[0]));
+    uint32_t at0 = 0, at1 = 0;
+    for (int w0 = 0; w0 < W; w0 += 256) {
+        const int w = w0 + tid;
+        uint32_t m0 = 0u, m1 = 0u;
+        if (w < W) {
+            const uint32_t g0 = __ldg(p + ((size_t)(w >> 2) * M + i) * 4 + (w & 3));
+            const uint32_t g1 = __ldg(p + ((size_t)(W4 + (w >> 2)) * M + i) * 4 + (w & 3));
             // genotype 2 by NOR, without the pad positions past the class's last sample
-            const int nv = Nc - 32 * ww;
+            const int nv = Nc - 32 * w;
             const uint32_t valid = nv >= 32 ? 0xFFFFFFFFu : (nv <= 0 ? 0u : (1u << nv) - 1u);
             const uint32_t g2 = ~(g0 | g1) & valid;
-            // the two counted genotypes, ascending (cmp_geno)
-            const uint32_t mk0 = drop == 0 ? g1 : g0;
-            const uint32_t mk1 = drop == 2 ? g1 : g2;
-            uint32_t v0[5], v1[5];
-            cmp_masks(mk0, v0);
-            cmp_masks(mk1, v1);
-            MaskWord e;
-            e.q[0] = make_uint4(mk0, mk1, (uint32_t)__popc(mk0), (uint32_t)__popc(mk1));
-            e.q[1] = make_uint4(v0[0], v0[1], v0[2], v0[3]);
-            e.q[2] = make_uint4(v1[0], v1[1], v1[2], v1[3]);
-            e.q[3] = make_uint4(v0[4], v1[4], 0u, 0u);
-            s_w[w] = e;
+            m0 = drop == 0 ? g1 : g0;       // the two counted genotypes, ascending (cmp_geno)
+            m1 = drop == 2 ? g1 : g2;
         }
-        __syncthreads();
-        const int g0 = w0 >> 2, ng = nw >> 2;
-        const uint4* const src = pc + (size_t)(z * W4 + g0) * M + m;   // this row's plane
-        uint4 vn = m < M ? __ldg(src) : zero4;
-        for (int g = 0; g < ng; ++g) {
-            const uint4 v = vn;
-            if (g + 1 < ng) vn = m < M ? __ldg(src + (size_t)(g + 1) * M) : zero4;
-            const uint32_t xs[4] = {v.x, v.y, v.z, v.w};
+        const uint32_t own = (uint32_t)__popc(m0) | ((uint32_t)__popc(m1) << 16);   // at most 8192 each
+        uint32_t incl = own;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const MaskWord& mw = s_w[4 * g + e];
-                const uint4 h = mw.q[0], a0 = mw.q[1], a1 = mw.q[2], a4 = mw.q[3];
-                const uint32_t mv0[5] = {a0.x, a0.y, a0.z, a0.w, a4.x};
-                const uint32_t mv1[5] = {a1.x, a1.y, a1.z, a1.w, a4.y};
-                cmp_word(base0, slab0, r, s0, xs[e], h.x, mv0, (int)h.z);
-                cmp_word(base1, slab1, r, s1, xs[e], h.y, mv1, (int)h.w);
-            }
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t o = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += o;
+        }
+        if (lane == 31) s_warp[wid] = incl;
+        __syncthreads();
+        uint32_t before = incl - own, all = 0;
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+            const uint32_t o = s_warp[v];
+            before += v < wid ? o : 0u;
+            all += o;
+        }
+        uint32_t* o0 = l0 + at0 + (before & 0xFFFFu);
+        uint32_t* o1 = l1 + at1 + (before >> 16);
+        for (; m0; m0 &= m0 - 1) *o0++ = (uint32_t)(32 * w + __ffs(m0) - 1);
+        for (; m1; m1 &= m1 - 1) *o1++ = (uint32_t)(32 * w + __ffs(m1) - 1);
+        at0 += all & 0xFFFFu;
+        at1 += all >> 16;
+        __syncthreads();
+    }
+}
+
+// CTA (b, f, c): block b's chunks of the two sets of class c of first SNP f.  Rows of a chunk come in
+// 16-row groups: row 16 G + 8 z + r holds SNP m = 64 b + 8 G + r with genotype z (8 SNPs of genotype
+// 0, then the same 8 of genotype 1), so that a 16x256b tensor-memory load hands a thread both genotype
+// rows of one SNP (see the epilogue).  Warp u makes unit u (32 samples) of every K-step: the samples
+// in list order, then the bias sample (a 1 in every row), then zeros.  The 16 KB image is put together
+// in shared memory and leaves in one bulk copy, two images in flight.  Bound by the chunks' writes
+// (2048 x 16384: 14.2 GB).
+constexpr int kCompactThreads = 256;
+__global__ void __launch_bounds__(kCompactThreads)
+compact_kernel(const uint4* __restrict__ rows, int words0, int words, const CmpFirst* __restrict__ firsts,
+               const uint32_t* __restrict__ list, int n0, int n, uint8_t* __restrict__ cmp) {
+    __shared__ __align__(128) uint8_t s_img[2][kCmpChunk];
+    const int b = blockIdx.x, f = blockIdx.y, c = blockIdx.z;
+    const CmpFirst* const fp = firsts + f;
+    const int b_lo = fp->b_lo;
+    if (b < b_lo) return;  // whole CTA: no block before the first SNP's successors
+    const int tid = threadIdx.x, lane = tid & 31, u = tid >> 5;
+    const uint4* const src = rows + ((size_t)b * words + (c ? words0 : 0)) * 32;
+    const int ks[2] = {fp->ks[2 * c], fp->ks[2 * c + 1]}, cnt[2] = {fp->cnt[2 * c], fp->cnt[2 * c + 1]};
+    const uint32_t* const l0 = list + (size_t)f * n + (c ? n0 : 0);
+    const int steps = ks[0] + ks[1];
+    auto gather = [&](int q) {   // this lane's sample of K-step q (both sets' steps in a row)
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (q >= steps) return v;
+        const int s = q >= ks[0] ? 1 : 0, p = 256 * (s ? q - ks[0] : q) + 32 * u + lane, m = s ? cnt[1] : cnt[0];
+        if (p < m) v = __ldg(src + __ldg(l0 + (s ? cnt[0] : 0) + p));
+        else if (p == m) v = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+        return v;
+    };
+    uint4 next = gather(0);
+    for (int q = 0; q < steps; ++q) {
+        const uint4 v = next;
+        next = gather(q + 1);
+        const uint32_t x[4] = {warp_transpose(v.x), warp_transpose(v.y), warp_transpose(v.z), warp_transpose(v.w)};
+        uint8_t* const img = s_img[q & 1];
+        // the copy two K-steps ago has read this image
+        if (tid == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {   // genotype e / 2, SNP 32 (e % 2) + lane
+            const uint32_t w = x[e];
+            const int m = 32 * (e & 1) + lane, row = 16 * (m >> 3) + 8 * (e >> 1) + (m & 7);
+            *reinterpret_cast<uint4*>(img + sw128_off((uint32_t)row, (uint32_t)u)) =
+                make_uint4(byte_to_e2m1(w), byte_to_e2m1(w >> 8), byte_to_e2m1(w >> 16), byte_to_e2m1(w >> 24));
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncthreads();
+        if (tid == 0) {
+            const int s = q >= ks[0] ? 1 : 0;
+            const long long chunk = fp->base[2 * c + s] + (long long)(b - b_lo) * ks[s] + (s ? q - ks[0] : q);
+            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;"
+                         ::"l"(cmp + (size_t)chunk * kCmpChunk), "r"(smem_u32(img)), "r"(kCmpChunk) : "memory");
+            asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         }
     }
-    // the bias sample, then zeros up to the set's K-steps (8 words each)
-    cmp_push(base0, slab0, r, s0, 1u, 1);
-    cmp_push(base1, slab1, r, s1, 1u, 1);
-    for (const int words = 8 * ks0; s0.word < words;) {
-        cmp_emit(base0, slab0, r, s0, (uint32_t)s0.acc);
-        s0.acc >>= 32;
-    }
-    for (const int words = 8 * ks1; s1.word < words;) {
-        cmp_emit(base1, slab1, r, s1, (uint32_t)s1.acc);
-        s1.acc >>= 32;
-    }
+    if (tid == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
 // ------------------------------------------------------------------ the scan kernel
@@ -1162,11 +1152,26 @@ int cmp_tiles_of(int M, int b_lo, int jb_end) {
     return t;
 }
 
-cudaError_t launch_compact(const Planes& pl, const CmpFirst* firsts, int i0, int n_first,
-                           uint8_t* cmp, cudaStream_t st) {
+size_t sample_rows_bytes(const Planes& pl) {
+    return (size_t)((pl.M + 63) / 64) * 128 * (size_t)(pl.W4[0] + pl.W4[1]) * sizeof(uint4);
+}
+
+cudaError_t launch_sample_rows(const Planes& pl, uint4* rows, cudaStream_t st) {
+    const int nblk = (pl.M + 63) / 64;
+    const long long warps = 4LL * (pl.W4[0] + pl.W4[1]) * nblk, blocks = (warps + 7) / 8;
+    sample_rows_kernel<<<(unsigned)std::min<long long>(blocks, 65535), 256, 0, st>>>(pl, nblk, rows);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_compact(const Planes& pl, const uint4* rows, const CmpFirst* firsts, int i0, int n_first,
+                           int n0, int n, uint32_t* list, uint8_t* cmp, cudaStream_t st) {
     if (n_first == 0) return cudaSuccess;
+    sample_list_kernel<<<dim3(n_first, 2), 256, 0, st>>>(pl, firsts, i0, n0, n, list);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     const dim3 grid((pl.M + 63) / 64, n_first, 2);
-    compact_kernel<<<grid, kCompactThreads, 0, st>>>(pl, firsts, i0, cmp);
+    compact_kernel<<<grid, kCompactThreads, 0, st>>>(rows, 4 * pl.W4[0], 4 * (pl.W4[0] + pl.W4[1]), firsts, list,
+                                                     n0, n, cmp);
     return cudaGetLastError();
 }
 
