@@ -90,8 +90,8 @@ struct PairTables {
 
 // Constants of the table-free bound by class sizes (cmp_bound_terms in capi.cu).
 struct CmpBoundTerms {
-    float c, off;                // K2 >= c (sum of q) + (ln of the product of q) / 2 - off, 27 cells
-    float off2;                  // the same for the 9 cells of a pair
+    float c, off;                // K2 >= (sum of ln us) / 2 - c (sum of um^2 / us) - off, 27 cells
+    float off2;                  // K2 >= c (sum of q) + (sum of ln q) / 2 - off2, the 9 cells of a pair
     float slack;                 // the part of off that covers Stirling's remainders and rounding
     int minor;                   // the smaller class
 };
@@ -256,8 +256,7 @@ struct CmpArgs {
     int n_runs;                  // runs of the range
     const uint8_t* cmp;          // compacted chunks of the range
     const float4* yz;            // (Y, Z) pair tables in the epilogue's form (launch_pair_yz)
-    // the table-free bound: K2 >= bound_c (sum of q) + (ln of the product of q) / 2 - bound_off
-    // over the 27 cells' q = um (us - um) / us (cmp_bound_terms)
+    // the table-free bound (cmp_bound_terms)
     float bound_c, bound_off;
     int minor;                   // the smaller class (table m)
     unsigned long long* prof;    // optional (instrumented kernel): wait cycles per role

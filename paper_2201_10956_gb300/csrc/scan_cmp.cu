@@ -524,42 +524,34 @@ __device__ __forceinline__ void cmp_survivors(const CmpArgs& a, EpiShared& es, C
     __syncwarp();
 }
 
-// The bound of one lane's two triplets of an item (L = LaneOps2), or of one of them (LaneOps1).
-// Per cell q = um (us - um) / us, us and um the cell's u in tables s and m: um + um (um (-1/us)).
-// Sum of q and sum of lg2 q (the cells of a phase multiplied first: every q is at least about
-// 1/2 and nine of them sum to at most (N + 54) / 4, so no product leaves the FP32 range).
-// A reciprocal holds its pipe for 8 cycles a warp and the FP32 pipe is as busy, so cells share one
-// reciprocal in pairs: -1 / a = b (-1 / (a b)).  The nine cells of a phase go through each operation
-// together: one after the other, every operation would wait for the one before it.
-constexpr int kRcpPairs = 4;
+// The bound of one lane's two triplets of an item (L = LaneOps2), or of one of them (LaneOps1): the sum
+// of um^2 / us and of lg2 us over the cells, us and um the cell's u in tables s and m (cmp_bound_terms).
+// Two cells a, b share a reciprocal and its argument is their factor of the product:
+//     um_a^2 / us_a + um_b^2 / us_b = (um_a^2 us_b + um_b^2 us_a) / (us_a us_b),
+// seven FP32 operations for two cells and half a reciprocal each.  The nine cells of a phase go
+// through each operation together: one after the other, every operation would wait for the one
+// before it.  (The us of nine cells sum to at most N + 54, so their product stays in FP32 range.)
 template <class L>
 struct CmpBound {
     typedef typename L::T T;
     T sum[2], lgs;
     __device__ __forceinline__ void init() { sum[0] = sum[1] = lgs = L::dup(0.f); }
     __device__ __forceinline__ void phase(const T (&us)[9], const T (&um)[9]) {
-        T nr[9], q[9];
+        T w[5], r[5], n[9];
 #pragma unroll
-        for (int e = 0; e < 2 * kRcpPairs; e += 2) nr[e] = L::mul(us[e], us[e + 1]);
+        for (int e = 0; e < 4; ++e) w[e] = L::mul(us[2 * e], us[2 * e + 1]);
+        w[4] = us[8];
 #pragma unroll
-        for (int e = 0; e < 9; ++e)
-            if (e >= 2 * kRcpPairs) nr[e] = L::nrcp(us[e]);
-            else if (e % 2 == 0) nr[e] = L::nrcp(nr[e]);
+        for (int e = 0; e < 5; ++e) r[e] = L::rcp(w[e]);
 #pragma unroll
-        for (int e = 0; e < 2 * kRcpPairs; e += 2) {
-            nr[e + 1] = L::mul(nr[e], us[e]);
-            nr[e] = L::mul(nr[e], us[e + 1]);
-        }
+        for (int e = 0; e < 9; ++e) n[e] = L::mul(um[e], um[e]);
 #pragma unroll
-        for (int e = 0; e < 9; ++e) q[e] = L::mul(um[e], nr[e]);
+        for (int e = 0; e < 4; ++e) n[2 * e] = L::mul(n[2 * e], us[2 * e + 1]);
 #pragma unroll
-        for (int e = 0; e < 9; ++e) q[e] = L::fma(q[e], um[e], um[e]);
+        for (int e = 0; e < 4; ++e) n[2 * e] = L::fma(n[2 * e + 1], us[2 * e], n[2 * e]);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) sum[e & 1] = L::add(sum[e & 1], q[e]);
-        sum[0] = L::add(sum[0], q[8]);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) q[e] = L::mul(q[e], q[4 + e]);
-        lgs = L::add(lgs, L::lg(L::mul(L::mul(L::mul(q[0], q[1]), L::mul(q[2], q[3])), q[8])));
+        for (int e = 0; e < 5; ++e) sum[e & 1] = L::fma(n[2 * e], r[e], sum[e & 1]);
+        lgs = L::add(lgs, L::lg(L::mul(L::mul(L::mul(w[0], w[1]), L::mul(w[2], w[3])), w[4])));
     }
 };
 
@@ -910,10 +902,9 @@ __global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const __grid_c
         // neighbouring registers, as the f32x2 instructions take them.  Items of a quadrant: lane
         // groups G = 2 quad + h (h = 0, 1) x column groups H = 0..3; each warp takes two column
         // groups of one h.
-        // The bound per triplet: 27 cells x 4 FP32 operations, 76 subtractions for the 19 derived
-        // cells in two tables, 36 products for the shared reciprocals, i.e. about 230 FP32 lane
-        // operations (3700 cycles a tile at 128 a clock) and 18 reciprocals and logs (2300 at 16 a
-        // clock).  The form before, phi(us) - phi(u0) - phi(u1) per cell, took 81 logs, and each
+        // The bound per triplet: 93 FP32 operations for the 27 cells and 76 subtractions for the 19
+        // derived cells in two tables, about 185 lane operations in all (3000 cycles a tile at 128 a
+        // clock), and 18 reciprocals and logs (2300 at 16 a clock).  The form before, phi(us) - phi(u0) - phi(u1) per cell, took 81 logs, and each
         // thread formed the constants that the stagers now form once a tile.
         const int tid = threadIdx.x - kCmpEpiWarp0 * 32;     // 0 .. 383
         const int quad = warp & 3, part = (warp - kCmpEpiWarp0) >> 2;
@@ -1069,8 +1060,8 @@ __global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const __grid_c
                             if (ph == 2 && (kPaired || pass == 1)) fetch(next);
                             B.phase(s9, m9);
                         }
-                        // ln 2 / 2 (sum of lg2 q) + c (sum of q) against the cut
-                        const T b = L::fma(L::dup(cq), L::add(B.sum[0], B.sum[1]), L::mul(L::dup(0.34657359f), B.lgs));
+                        // ln 2 / 2 (sum of lg2 us) - c (sum of um^2 / us) against the cut
+                        const T b = L::fma(L::dup(-cq), L::add(B.sum[0], B.sum[1]), L::mul(L::dup(0.34657359f), B.lgs));
                         if constexpr (kPaired) sv = (b.x > cut ? 0u : 1u) | (b.y > cut ? 0u : 2u);
                         else sv |= (b > cut ? 0u : 1u) << pass;
                     }

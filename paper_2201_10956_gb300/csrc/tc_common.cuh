@@ -291,7 +291,7 @@ struct LaneOps1 {
     static __device__ __forceinline__ T lg(T a) { return lg2_hw(a); }
     static __device__ __forceinline__ T dup(float a) { return a; }
     static __device__ __forceinline__ T mul(T a, T b) { return __fmul_rn(a, b); }
-    static __device__ __forceinline__ T nrcp(T a) { return rcp_hw(-a); }
+    static __device__ __forceinline__ T rcp(T a) { return rcp_hw(a); }
     // a row constant (stored twice), one triplet's half of a pair
     static __device__ __forceinline__ T two(float a, float) { return a; }
     static __device__ __forceinline__ T pick(float2 a, int m) { return m ? a.y : a.x; }
@@ -304,7 +304,7 @@ struct LaneOps2 {
     static __device__ __forceinline__ T lg(T a) { return make_float2(lg2_hw(a.x), lg2_hw(a.y)); }
     static __device__ __forceinline__ T dup(float a) { return f2_dup(a); }
     static __device__ __forceinline__ T mul(T a, T b) { return f2_mul(a, b); }
-    static __device__ __forceinline__ T nrcp(T a) { return make_float2(rcp_hw(-a.x), rcp_hw(-a.y)); }
+    static __device__ __forceinline__ T rcp(T a) { return make_float2(rcp_hw(a.x), rcp_hw(a.y)); }
     static __device__ __forceinline__ T two(float a, float b) { return make_float2(a, b); }
     static __device__ __forceinline__ T pick(float2 a, int) { return a; }
 };
