@@ -293,6 +293,12 @@ __device__ __forceinline__ void tc_ld16x2(uint32_t taddr, float* v) {
           "=f"(v[7])
         : "r"(taddr));
 }
+// A shared-memory load that stays where it is written: the compiler moves plain ones to their use,
+// where their latency shows (2048 x 4096: 7740 -> 7310 cycles a tile with the next phase's constants
+// loaded before a phase's work).
+__device__ __forceinline__ void lds128(float4& v, const float4* p) {
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(smem_u32(p)));
+}
 // 16 bytes from global to shared memory, asynchronously.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -526,9 +532,10 @@ __device__ __forceinline__ void cmp_survivors(const CmpArgs& a, EpiShared& es, C
 
 // The bound of one lane's two triplets of an item (L = LaneOps2), or of one of them (LaneOps1): the sum
 // of um^2 / us and of lg2 us over the cells, us and um the cell's u in tables s and m (cmp_bound_terms).
-// Two cells a, b share a reciprocal and its argument is their factor of the product:
+// Two cells a, b share a denominator that is also their factor of the product:
 //     um_a^2 / us_a + um_b^2 / us_b = (um_a^2 us_b + um_b^2 us_a) / (us_a us_b),
-// seven FP32 operations for two cells and half a reciprocal each.  The nine cells of a phase go
+// six FP32 operations, and two such pairs share a reciprocal (a reciprocal holds its pipe for 8 cycles
+// a warp, a product the FP32 pipe for 2).  The nine cells of a phase go
 // through each operation together: one after the other, every operation would wait for the one
 // before it.  (The us of nine cells sum to at most N + 54, so their product stays in FP32 range.)
 template <class L>
@@ -541,17 +548,23 @@ struct CmpBound {
 #pragma unroll
         for (int e = 0; e < 4; ++e) w[e] = L::mul(us[2 * e], us[2 * e + 1]);
         w[4] = us[8];
-#pragma unroll
-        for (int e = 0; e < 5; ++e) r[e] = L::rcp(w[e]);
+        const T p0 = L::mul(w[0], w[1]), p1 = L::mul(w[2], w[3]);
+        const T q0 = L::rcp(p0), q1 = L::rcp(p1);
+        r[4] = L::rcp(w[4]);
+        const T all = L::mul(L::mul(p0, p1), w[4]);
 #pragma unroll
         for (int e = 0; e < 9; ++e) n[e] = L::mul(um[e], um[e]);
 #pragma unroll
         for (int e = 0; e < 4; ++e) n[2 * e] = L::mul(n[2 * e], us[2 * e + 1]);
 #pragma unroll
         for (int e = 0; e < 4; ++e) n[2 * e] = L::fma(n[2 * e + 1], us[2 * e], n[2 * e]);
+        r[0] = L::mul(q0, w[1]);
+        r[1] = L::mul(q0, w[0]);
+        r[2] = L::mul(q1, w[3]);
+        r[3] = L::mul(q1, w[2]);
 #pragma unroll
         for (int e = 0; e < 5; ++e) sum[e & 1] = L::fma(n[2 * e], r[e], sum[e & 1]);
-        lgs = L::add(lgs, L::lg(L::mul(L::mul(L::mul(w[0], w[1]), L::mul(w[2], w[3])), w[4])));
+        lgs = L::add(lgs, L::lg(all));
     }
 };
 
@@ -972,10 +985,11 @@ __global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const __grid_c
             if (!bad) {
                 tc_fence_after();
                 const CmpStage& S = stage[buf];
+                const unsigned vmask_all = qu.vmask[lane];
 #pragma unroll 1
                 for (int it = 0; it < kCmpEpiItems; ++it) {
                     const int item = part + kCmpEpiParts * it, jl = jl0 + 8 * (item >> 2);
-                    const unsigned vmask = (qu.vmask[lane] >> (2 * it)) & 3u;
+                    const unsigned vmask = (vmask_all >> (2 * it)) & 3u;
                     if (item >= 8) break;
                     const int next = item + kCmpEpiParts < 8 ? item + kCmpEpiParts : part;
                     if (!__any_sync(0xffffffffu, vmask)) {   // k <= j throughout
@@ -1000,9 +1014,19 @@ __global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const __grid_c
                             tc_ld16x2(tb + (uint32_t)(region(2 * (cm ^ 1) + ph) * kN), v[0]);
                             tc_ld16x2(tb + (uint32_t)(region(2 * cm + ph) * kN), v[1]);
                         };
+                        float4 cs, cmn, r0, r1, r2;   // a phase's constants
+                        auto constants = [&](int ph) {
+                            lds128(cs, col + 2 * ph);
+                            lds128(cmn, col + 2 * ph + 1);
+                            lds128(r0, row + 3 * ph);
+                            lds128(r1, row + 3 * ph + 1);
+                            lds128(r2, row + 3 * ph + 2);
+                        };
+                        constants(0);
                         T ds[4], dm[4];   // cells (2, b, z): the (Y, Z) table minus the counted genotypes
 #pragma unroll
                         for (int ph = 0; ph < 3; ++ph) {
+                            if (ph < 2) load(ph);
                             T us[4], um[4];   // cells (b, z) of this first-SNP genotype, index 2 b + z
                             float4 y4[4];
                             if (ph == 2) {
@@ -1010,10 +1034,7 @@ __global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const __grid_c
 #pragma unroll
                                 for (int e = 0; e < 4; ++e) y4[e] = ys[32 * e];
                             }
-                            if (ph < 2) {
-                                load(ph);
-                                tc_wait_ld2(v);
-                            }
+                            if (ph < 2) tc_wait_ld2(v);
 #pragma unroll
                             for (int e = 0; e < 4; ++e) {
                                 if (ph < 2) {
@@ -1030,8 +1051,6 @@ __global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const __grid_c
                                     um[e] = L::sub(L::pick(e & 1 ? make_float2(ym.z, ym.w) : make_float2(ym.x, ym.y), pass), dm[e]);
                                 }
                             }
-                            const float4 cs = col[2 * ph], cmn = col[2 * ph + 1];
-                            const float4 r0 = row[3 * ph], r1 = row[3 * ph + 1], r2 = row[3 * ph + 2];
                             const T cst[9] = {us[0], us[1], us[2], us[3], L::two(r0.x, r0.y), L::two(r1.x, r1.y),
                                               L::pick(make_float2(cs.x, cs.y), pass),
                                               L::pick(make_float2(cs.z, cs.w), pass), L::two(r2.x, r2.y)};
@@ -1058,6 +1077,7 @@ __global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const __grid_c
                             s9[8] = L::sub(L::sub(s9[8], s9[6]), s9[7]);
                             m9[8] = L::sub(L::sub(m9[8], m9[6]), m9[7]);
                             if (ph == 2 && (kPaired || pass == 1)) fetch(next);
+                            if (ph < 2) constants(ph + 1);
                             B.phase(s9, m9);
                         }
                         // ln 2 / 2 (sum of lg2 us) - c (sum of um^2 / us) against the cut
