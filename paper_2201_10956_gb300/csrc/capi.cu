@@ -47,7 +47,8 @@ int cuda_fail(cudaError_t e, const char* what) {
 // EPI3_FAULT=timeout makes the tensor-core scan's MMA issuer wait on a barrier nobody
 // signals, so its bounded wait runs out (1 s) and the scan returns EPI3_ERR_TIMEOUT;
 // EPI3_FAULT=cand starts a handle with a 128-entry candidate list, so scans overflow it and
-// take the retry path with a larger list.
+// take the retry path with a larger list.  EPI3_FAULT=tables asks for more memory than there is
+// for the counted form of the four- to six-SNP scans, which then take the direct form.
 bool inject(const char* what) {
     const char* f = getenv("EPI3_FAULT");
     return f && strcmp(f, what) == 0;
@@ -123,6 +124,7 @@ cudaError_t dev_alloc(void** p, size_t bytes) {
         e = cudaMalloc(p, bytes);
     }
     if (e != cudaSuccess) {
+        (void)cudaGetLastError();  // reported by the return value: a caller that goes on launches kernels
         *p = nullptr;
         return e;
     }
@@ -1504,7 +1506,7 @@ int epi3_scan_order(epi3_handle* h, int32_t order, int32_t top_k, int32_t* out_s
     // sets tie at the k-th score than it rescores; then the direct form
     bool done = false;
     const size_t cnt = set_scan_scratch(h->M, h->N, order);
-    if (cnt && scratch(cnt) == EPI3_OK) {
+    if (cnt && scratch(inject("tables") ? (size_t)1 << 60 : cnt) == EPI3_OK) {
         place(cnt);
         CK(launch_set_scan(h->pl, h->k2.lf64, h->N0, h->N1, order, top_k, h->sm_count, h->d_pair_scratch,
                            h->h_ctrl, d_sets, d_s, &done, h->stream), "k-SNP scan launch");

@@ -48,3 +48,11 @@ def test_thousands_of_equal_sets(order, m):
     g, ph = pins.tiny_data(m, 200, 90, seed=1800 + order)
     g[:] = g[np.arange(m) % 3]
     _check(g, ph, order, 40)
+
+
+@pytest.mark.parametrize("order,m", [(4, 15), (5, 11), (6, 9)])
+def test_direct_form_without_memory_for_the_tables(order, m, monkeypatch):
+    # the failed allocation is not reported by the launches that follow it
+    monkeypatch.setenv("EPI3_FAULT", "tables")
+    g, ph = pins.tiny_data(m, 150, 70, seed=1900 + order)
+    _check(g, ph, order, 12)
