@@ -7,8 +7,8 @@
 // genotypes a of SNP i are counted this way, the two least frequent over all samples; the most
 // frequent one is derived with the other 19 cells (the same genotype in both classes), so the
 // GEMMs run over the smallest share of the samples.  The samples of each of the four sets
-// (c, a) are gathered once per first SNP ("compaction": bit extraction from the packed planes,
-// expansion to FP4 E2M1 0/1 values in the 128B-swizzled shared-memory image), and the scan
+// (c, a) are gathered once per first SNP ("compaction": the samples' genotype bits, transposed and
+// expanded to FP4 E2M1 0/1 values in the 128B-swizzled shared-memory image), and the scan
 // multiplies compacted chunks straight from L2: both MMA operands come from shared memory,
 // filled by bulk copies, with no operand formed on chip and 4 MACs per sample-triplet whose
 // first-SNP genotype is counted.  SNP i's genotypes are relabelled (counted ones 0 and 1, the
@@ -472,8 +472,9 @@ __device__ __forceinline__ void cmp_score(const CmpArgs& a, EpiShared& es, const
 }
 
 // A warp's surviving triplets of an item (mask: bit m, triplet (i, j, k0 + m)) go to its queue, their
-// counted cells read from tensor memory again (t: the item's four sets); before it would overflow, the queue is scored.  Called by a whole warp; with no survivors
-// at all (mask 0 in every lane) it scores what is left.
+// counted cells read from tensor memory again (t: the item's four sets); before it would overflow, the
+// queue is scored.  Called by a whole warp; with no survivors at all (mask 0 in every lane) it scores
+// what is left.
 struct CmpItems {
     uint32_t t[4];
     int i, j, k0;
@@ -535,9 +536,9 @@ __device__ __forceinline__ void cmp_survivors(const CmpArgs& a, EpiShared& es, C
 // Two cells a, b share a denominator that is also their factor of the product:
 //     um_a^2 / us_a + um_b^2 / us_b = (um_a^2 us_b + um_b^2 us_a) / (us_a us_b),
 // six FP32 operations, and two such pairs share a reciprocal (a reciprocal holds its pipe for 8 cycles
-// a warp, a product the FP32 pipe for 2).  The nine cells of a phase go
-// through each operation together: one after the other, every operation would wait for the one
-// before it.  (The us of nine cells sum to at most N + 54, so their product stays in FP32 range.)
+// a warp, a product the FP32 pipe for 2).  The nine cells of a phase go through each operation
+// together: one after the other, every operation would wait for the one before it.  (The us of nine
+// cells sum to at most N + 54: at the 131072 samples a handle takes their product is at most 3.0e37.)
 template <class L>
 struct CmpBound {
     typedef typename L::T T;
@@ -915,10 +916,11 @@ __global__ void __launch_bounds__(kCmpThreads, 1) scan_cmp_kernel(const __grid_c
         // neighbouring registers, as the f32x2 instructions take them.  Items of a quadrant: lane
         // groups G = 2 quad + h (h = 0, 1) x column groups H = 0..3; each warp takes two column
         // groups of one h.
-        // The bound per triplet: 93 FP32 operations for the 27 cells and 76 subtractions for the 19
-        // derived cells in two tables, about 185 lane operations in all (3000 cycles a tile at 128 a
-        // clock), and 18 reciprocals and logs (2300 at 16 a clock).  The form before, phi(us) - phi(u0) - phi(u1) per cell, took 81 logs, and each
-        // thread formed the constants that the stagers now form once a tile.
+        // The bound per triplet: 105 FP32 operations for the 27 cells, 84 additions and subtractions
+        // for the 19 derived cells in two tables, 192 lane operations with the last three (3070 cycles
+        // a tile at 128 a clock), and 12 reciprocals and logs (1540 at 16 a clock).  The form before,
+        // phi(us) - phi(u0) - phi(u1) per cell, took 81 logs, and each thread formed the constants that
+        // the stagers now form once a tile.
         const int tid = threadIdx.x - kCmpEpiWarp0 * 32;     // 0 .. 383
         const int quad = warp & 3, part = (warp - kCmpEpiWarp0) >> 2;
         const int jl0 = 16 * quad + (lane >> 2), tcol = 2 * (lane & 3);
