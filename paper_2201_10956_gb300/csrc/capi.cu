@@ -1835,7 +1835,9 @@ void tune_store(const TuneEntry& e) {
 // The handle tuner: for path "auto", every scan form that supports the shape -- 8-cell POPC,
 // sample-compacted tensor, one-hot tensor in its plain and register-split forms -- is timed
 // on the heaviest pair slice (the first pairs, those with the smallest second SNP: at most 1/16
-// of the pairs and about 3e13 sample-triplets), after a warm-up on a sixteenth of it, and its
+// of the pairs and about 3e13 sample-triplets; the whole of a scan of at most 2e10, a millisecond
+// in the slowest form, whose slice would leave most SMs idle: 200 SNPs x 2500 samples got the one-hot
+// form from it, 298 us where the compacted one takes 229), after a warm-up on a sixteenth of it, and its
 // time is extrapolated to the whole scan by the form's work terms: triplets for the POPC and
 // one-hot forms; for the compacted form its compaction (timed apart, scaled by compacted
 // chunks) and its MMA K-steps, both from the plan of the whole scan.  The lowest wins.  For an explicitly chosen one-hot tensor path with form "auto", only its two forms
@@ -1870,7 +1872,8 @@ int tune_handle(epi3_handle* h) {
             return EPI3_OK;
         }
     const long long np = pairs(h->M - 1);
-    long long pe = std::max(1LL, np / 16);
+    const bool small = (double)triplets_in_pairs(h->M, 0, np) * h->N <= 2e10;
+    long long pe = small ? np : std::max(1LL, np / 16);
     while (pe > 1 && (double)triplets_in_pairs(h->M, 0, pe) * h->N > 3e13) pe /= 2;
     const long long pw = std::max(1LL, pe / 16);
     const double nt_full = (double)triplets_in_pairs(h->M, 0, np);
@@ -1934,6 +1937,10 @@ int tune_handle(epi3_handle* h) {
     return EPI3_OK;
 }
 
+// One-hot tiles an SM below which a batch's cohort shares the one-hot launch (tune_path): 5 is 211
+// SNPs on 152 SMs, just above where the two forms meet.
+constexpr long long kBatchSharedTiles = 5;
+
 int tune_path(epi3_batch* b, epi3_handle* h, int* path_out, float* ms) {
     const char* force = getenv("EPI3_BATCH_PATH");
     if (force && !strcmp(force, "mma")) { *path_out = EPI3_PATH_MMA4; return EPI3_OK; }
@@ -1943,10 +1950,20 @@ int tune_path(epi3_batch* b, epi3_handle* h, int* path_out, float* ms) {
     // timed alone, yet in the batch its tiles share one persistent launch with every other
     // cohort's (its marginal cost there is its tiles' share of that launch, at the
     // throughput-bound rate, several times the POPC forms').  Timing it alone would be biased
-    // against the shared launch, so such cohorts take it; the rest get the handle tuner's
-    // measured choice for their shape (8-cell POPC, the compacted form in launches of its own,
-    // or the shared one-hot launch).
-    if (mma_tile_estimate(h->M) < 64LL * b->sm_count) { *path_out = EPI3_PATH_MMA4; return EPI3_OK; }
+    // against the shared launch, so the choice comes from whole batches of eight equal cohorts:
+    // the smallest take the shared launch; up to 64 tiles an SM the paired compacted form, in
+    // launches of its own, which there is the faster of the two at 1500, 6000 and 18000 samples (ms a
+    // cohort at 6000, one-hot and compacted: 140 SNPs 0.124 and 0.154, 180 SNPs 0.169 and 0.177, 220
+    // SNPs 0.263 and 0.210, 300 SNPs 0.500 and 0.329, 480 SNPs 1.460 and 0.654).  The rest get the
+    // handle tuner's measured choice for their shape.
+    const long long tiles = mma_tile_estimate(h->M);
+    if (tiles < kBatchSharedTiles * b->sm_count) { *path_out = EPI3_PATH_MMA4; return EPI3_OK; }
+    if (tiles < 64LL * b->sm_count) {
+        *path_out = EPI3_PATH_MMA4C;
+        h->tuned_path = h->tuned_form_path = EPI3_PATH_MMA4C;
+        h->tuned_form = 2;
+        return EPI3_OK;
+    }
     const auto t0 = std::chrono::steady_clock::now();
     h->path = EPI3_PATH_AUTO;
     const int rc = tune_handle(h);
