@@ -765,19 +765,44 @@ int start_scan(epi3_handle* h, long long pb, long long pe, int top_k) {
     return EPI3_OK;
 }
 
-// Candidate stage + result read-back shared by all scan forms.  The caller's device outputs are
-// written by the candidate stage itself; the scans of the tuner and of the debug calls keep their
-// answer in the handle's buffers.  Returns 1 to retry with a larger candidate list, EPI3_OK, or an
-// error.
-int finish_scan(epi3_handle* h, int top_k, int attempt, int32_t* out_trip, double* out_scores) {
-    const bool direct = (h->flags & EPI3_DEVICE_PTRS) && !h->tuning && !h->dbg && !h->tsum;
+// How a scan's answer reaches the caller.
+enum class Out {
+    kNone,     // not at all: the scans of the tuner and of the debug calls on device handles
+    kHost,     // read back into pinned memory, copied from there
+    kCopy,     // device outputs, by a copy
+    kKernel,   // device outputs, written by the candidate stage itself
+};
+// The candidate stage stores doubles and ints, so it writes only aligned memory of this device (saves
+// two copies and a wait); everything else that a copy can reach -- other alignments, pinned host
+// memory, another device's -- takes the copy.
+bool stage_can_write(const void* p, size_t align, int device) {
+    if (reinterpret_cast<uintptr_t>(p) % align) return false;
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == device;
+}
+Out out_mode(const epi3_handle* h, const int32_t* out_trip, const double* out_scores) {
+    if (!(h->flags & EPI3_DEVICE_PTRS)) return Out::kHost;
+    if (h->tuning || h->dbg || h->tsum) return Out::kNone;
+    return stage_can_write(out_scores, alignof(double), h->device) &&
+                   stage_can_write(out_trip, alignof(int32_t), h->device)
+               ? Out::kKernel : Out::kCopy;
+}
+
+// Candidate stage + result read-back shared by all scan forms.  Returns 1 to retry with a larger
+// candidate list, EPI3_OK, or an error.
+int finish_scan(epi3_handle* h, int top_k, int attempt, Out mode, int32_t* out_trip, double* out_scores) {
+    const bool direct = mode == Out::kKernel;
     CK(launch_answer(h->pl, h->k2, h->d_ctrl, h->d_cand, h->cand_cap, top_k, h->d_fin,
                      direct ? out_scores : h->d_out_scores, direct ? out_trip : h->d_out_trip, h->stream),
        "candidate stage launch");
     CK(cudaEventRecord(h->ev[3], h->stream), "event");
     CK(cudaMemcpyAsync(h->h_ctrl, h->d_ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream),
        "read status");
-    if (!(h->flags & EPI3_DEVICE_PTRS)) {
+    if (mode == Out::kHost) {
         CK(cudaMemcpyAsync(h->h_scores, h->d_out_scores, sizeof(double) * top_k,
                            cudaMemcpyDeviceToHost, h->stream), "read scores");
         CK(cudaMemcpyAsync(h->h_trip, h->d_out_trip, sizeof(int) * 3 * top_k,
@@ -810,13 +835,20 @@ int finish_scan(epi3_handle* h, int top_k, int attempt, int32_t* out_trip, doubl
     return EPI3_OK;
 }
 
-void copy_out(epi3_handle* h, int32_t* out_trip, double* out_scores, int32_t* n_out) {
+int copy_out(epi3_handle* h, Out mode, int32_t* out_trip, double* out_scores, int32_t* n_out) {
     const int nout = (int)h->h_ctrl->n_out;
-    if (!(h->flags & EPI3_DEVICE_PTRS)) {
+    if (mode == Out::kHost) {
         memcpy(out_scores, h->h_scores, sizeof(double) * nout);
         memcpy(out_trip, h->h_trip, sizeof(int) * 3 * nout);
+    } else if (mode == Out::kCopy) {
+        CK(cudaMemcpyAsync(out_scores, h->d_out_scores, sizeof(double) * nout, cudaMemcpyDeviceToDevice,
+                           h->stream), "copy scores");
+        CK(cudaMemcpyAsync(out_trip, h->d_out_trip, sizeof(int) * 3 * nout, cudaMemcpyDeviceToDevice,
+                           h->stream), "copy triplets");
+        CK(cudaStreamSynchronize(h->stream), "copy outputs");
     }
     if (n_out) *n_out = nout;
+    return EPI3_OK;
 }
 
 // Register-split or plain form of the tensor scan for this handle (option "mma_form").
@@ -871,6 +903,7 @@ int scan_mma_impl(epi3_handle* h, int path, long long pb, long long pe, long lon
     const int kind = kind_of_path(path);
     if (!h->d_cd) CK(dev_alloc((void**)&h->d_cd, sizeof(CohortDev)), "alloc descriptor");
     const int grid = h->sm_count;
+    const Out mode = out_mode(h, out_trip, out_scores);
     for (int attempt = 0;; ++attempt) {
         if (inject("launch")) return fail(EPI3_ERR_CUDA, "injected launch failure");
         CK(cudaEventRecord(h->ev[0], h->stream), "event");
@@ -888,12 +921,13 @@ int scan_mma_impl(epi3_handle* h, int path, long long pb, long long pe, long lon
                            h->profile ? h->d_prof : nullptr, mma_split(h, kind), h->tsum != nullptr),
            "mma scan launch");
         CK(cudaEventRecord(h->ev[2], h->stream), "event");
-        const int rc = finish_scan(h, top_k, attempt, out_trip, out_scores);
+        const int rc = finish_scan(h, top_k, attempt, mode, out_trip, out_scores);
         if (rc == 1) continue;
         if (rc != EPI3_OK) return rc;
         break;
     }
-    copy_out(h, out_trip, out_scores, n_out);
+    const int orc = copy_out(h, mode, out_trip, out_scores, n_out);
+    if (orc != EPI3_OK) return orc;
     epi3_stats& s = h->stats;
     s.n_triplets = nt;
     s.n_candidates = h->h_ctrl->n_cand;
@@ -1108,6 +1142,7 @@ int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int 
         CK(cudaEventCreate(&e), "event create");
         h->cmp_ev.push_back(e);
     }
+    const Out mode = out_mode(h, out_trip, out_scores);
     for (int attempt = 0;; ++attempt) {
         if (inject("launch")) return fail(EPI3_ERR_CUDA, "injected launch failure");
         CK(cudaEventRecord(h->ev[0], h->stream), "event");
@@ -1133,7 +1168,7 @@ int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int 
                "compacted scan launch");
         }
         CK(cudaEventRecord(h->ev[2], h->stream), "event");
-        const int rc = finish_scan(h, top_k, attempt, out_trip, out_scores);
+        const int rc = finish_scan(h, top_k, attempt, mode, out_trip, out_scores);
         if (rc == 1) continue;
         if (rc != EPI3_OK) return rc;
         break;
@@ -1143,7 +1178,8 @@ int scan_cmp_impl(epi3_handle* h, long long pb, long long pe, long long nt, int 
         cudaEventElapsedTime(&ms, h->cmp_ev[2 * r], h->cmp_ev[2 * r + 1]);
         compact_ms += ms;
     }
-    copy_out(h, out_trip, out_scores, n_out);
+    const int orc = copy_out(h, mode, out_trip, out_scores, n_out);
+    if (orc != EPI3_OK) return orc;
     epi3_stats& s = h->stats;
     s.n_triplets = nt;
     s.n_candidates = h->h_ctrl->n_cand;
@@ -1232,6 +1268,7 @@ int scan_impl(epi3_handle* h, long long pb, long long pe, int top_k, int32_t* ou
     const int per_sm = h->ctas_per_sm > 0 && h->ctas_per_sm < occ ? h->ctas_per_sm : occ;
     const int grid = h->sm_count * per_sm;
 
+    const Out mode = out_mode(h, out_trip, out_scores);
     for (int attempt = 0;; ++attempt) {
         if (inject("launch")) return fail(EPI3_ERR_CUDA, "injected launch failure");
         CK(cudaEventRecord(h->ev[0], h->stream), "event");
@@ -1253,12 +1290,13 @@ int scan_impl(epi3_handle* h, long long pb, long long pe, int top_k, int32_t* ou
         if (path == EPI3_PATH_POPC8) CK(launch_scan_popc8(a, grid, block, smem, h->stream), "scan launch");
         else CK(launch_scan_popc(a, grid, block, smem, h->stream), "scan launch");
         CK(cudaEventRecord(h->ev[2], h->stream), "event");
-        const int rc = finish_scan(h, top_k, attempt, out_trip, out_scores);
+        const int rc = finish_scan(h, top_k, attempt, mode, out_trip, out_scores);
         if (rc == 1) continue;
         if (rc != EPI3_OK) return rc;
         break;
     }
-    copy_out(h, out_trip, out_scores, n_out);
+    const int orc = copy_out(h, mode, out_trip, out_scores, n_out);
+    if (orc != EPI3_OK) return orc;
     epi3_stats& s = h->stats;
     s.n_triplets = nt;
     s.n_candidates = h->h_ctrl->n_cand;
