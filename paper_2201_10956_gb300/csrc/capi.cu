@@ -440,65 +440,6 @@ int build_k2_tables(epi3_handle* h) {
     return EPI3_OK;
 }
 
-// The table-free bounds.  With u = count + 1 per cell and class, us = u0 + u1, um the smaller class's
-// u, p = um / us, the entropy H in nats is bounded from below by a parabola that touches it at p0 =
-// (sum um) / (sum us), the same for every table:
-//     H(p) >= H(p0) + H'(p0) (p - p0) - c (p - p0)^2,  c = max over p of KL(p || p0) / (p - p0)^2,
-// and KL(p || p0) / (p - p0)^2 = integral over s in [0, 1] of (1 - s) / (t (1 - t)), t = p0 + s (p -
-// p0), is convex in p, so its largest value is at p = 0 or 1.  Summed with weights us the linear term
-// vanishes; S = sum us = N + 2 cells, sum um = p0 S.
-//
-// Pairs (9 cells): Stirling's form (lf(n) = (n + 1/2) ln(n + 1) - (n + 1) + ln(2 pi)/2 + e(n), 0 < e(n)
-// <= 1/(12 (n + 1))) makes K2 = sum us H + (1/2) sum ln q - cells ln(2 pi)/2 + remainders of at least
-// -1/6 a cell, q = um (us - um) / us, and sum us (p - p0)^2 = S p0 (1 - p0) - sum q, hence
-//     K2 >= c sum q + (1/2) sum ln q - [c S p0 (1 - p0) - S H(p0) + cells (ln(2 pi)/2 + 1/6)].
-//
-// Triplets (27 cells, the compacted scan): a cell's own term K = ln((us - 1)! / ((u0 - 1)! (u1 - 1)!))
-// obeys, for all u0, u1 >= 1,
-//     K >= us [H(p0) + H'(p0) (p - p0) - c (p - p0)^2] + (1/2) ln us + (1/2) ln(p0 (1 - p0)) -
-//          ln(2 pi)/2 - eps,   eps = max(0.125, 0.2346 - p0 / 4):
-// near p0 both sides agree to first order, away from it the parabola's slack grows with us, and the
-// largest excess of the right side without eps lies at um = 1, us p0 about 2 (1.081 - ln(x)/2 - 1/x at
-// x = us p0 for small p0, 0.2345 at x = 2; 0.121 at u0 = u1 = 1 for p0 = 1/2).  With sum us (p - p0)^2 =
-// sum um^2 / us - p0^2 S,
-//     K2 >= (1/2) sum ln us - c sum um^2 / us -
-//           [-S H(p0) - c p0^2 S + 27 (ln(2 pi)/2 - ln(p0 (1 - p0))/2 + eps)].
-//
-// c is the larger of the two p0's (a larger c is a weaker bound).  At the usual class shares it is 1.4 to
-// 1.8 times the parabola's own curvature, which costs a table without association (sum us (p - p0)^2 c
-// / 1.4 ~ 13 nats) 5 to 10 nats: about what the one-hot scan's bound loses to its doubled error term,
-// with half a reciprocal per cell instead of three logs.
-// FP32 rounding, S1 = sum um (q, um^2 / us <= um; p0 <= 1/2, so c S1 <= 1.4 S): every q or quotient
-// within 2^-21 of its um, S1 2^-21 together, c-fold; with q >= 1/2 once more in (1/2) ln q; the sums'
-// additions 27 2^-24 S1, c-fold; c's, the cut's and the last FMA's rounding 2^-24 (4 c S1 + 8 S + 200);
-// logs and products under 0.01; the FP32 score against K2: rel * K + abs as in build_k2_tables.  The
-// rounding terms are doubled.
-void cmp_bound_terms(epi3_handle* h) {
-    const int cm = h->N1 <= h->N0 ? 1 : 0;
-    const double nm = (double)(cm ? h->N1 : h->N0), N = (double)h->N;
-    auto p_of = [&](double cells) { return (nm + cells) / (N + 2.0 * cells); };
-    auto c_of = [](double p) {
-        return std::max(-std::log1p(-p) / (p * p), -std::log(p) / ((1.0 - p) * (1.0 - p)));
-    };
-    auto h_of = [](double p) { return -p * std::log(p) - (1.0 - p) * std::log1p(-p); };
-    const double c = std::max(c_of(p_of(27.0)), c_of(p_of(9.0)));
-    const double u = std::ldexp(1.0, -24), half_ln_2pi = 0.9189385332046727;
-    const double kmax = 27.0 * std::log(N + 2.0) + N * std::log(2.0);
-    const double S1 = nm + 27.0;
-    const double rnd = 8.0 * u * S1 * (c + 1.1) + 27.0 * u * S1 * c + u * (4.0 * c * S1 + 8.0 * N + 200.0) + 0.01 +
-                       (double)h->k2.rel * kmax + (double)h->k2.abs_;
-    const double S = N + 54.0, p = p_of(27.0), eps = std::max(0.125, 0.2346 - 0.25 * p);
-    const double off = -S * h_of(p) - c * p * p * S +
-                       27.0 * (half_ln_2pi - 0.5 * std::log(p * (1.0 - p)) + eps) + 2.0 * rnd;
-    const double S2 = N + 18.0, p2 = p_of(9.0);
-    const double off2 = c * S2 * p2 * (1.0 - p2) - S2 * h_of(p2) + 9.0 * (half_ln_2pi + 1.0 / 6.0) + 2.0 * rnd;
-    h->bound.c = std::nextafter((float)c, INFINITY);
-    h->bound.off = std::nextafter((float)off, INFINITY);
-    h->bound.off2 = std::nextafter((float)off2, INFINITY);
-    h->bound.slack = (float)(27.0 * eps + 2.0 * rnd);
-    h->bound.minor = cm;
-}
-
 int create_impl(epi3_handle* h, const uint8_t* geno, const uint8_t* pheno) {
     const size_t MN = (size_t)h->M * h->N;
     uint8_t* d_geno = nullptr;
@@ -577,7 +518,7 @@ int create_impl(epi3_handle* h, const uint8_t* geno, const uint8_t* pheno) {
     cleanup();
     if (rc != EPI3_OK) return rc;
     if ((rc = build_k2_tables(h)) != EPI3_OK) return rc;
-    cmp_bound_terms(h);
+    h->bound = cmp_bound_terms(h->N0, h->N1, h->k2.rel, h->k2.abs_);
     // FP32 candidate list: the CTAs flush their in-band candidates before the shared threshold
     // tightens, about 10^5 of them on a scan that fills the GPU (a list that overflows costs a
     // whole rescan, in a batch a second replay of every cohort)

@@ -1,6 +1,8 @@
 // Internal declarations shared by the library's translation units.
 #pragma once
 
+#include <algorithm>
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -88,13 +90,79 @@ struct PairTables {
     const float2* margf;
 };
 
-// Constants of the table-free bound by class sizes (cmp_bound_terms in capi.cu).
+// Constants of the table-free bounds by class sizes (cmp_bound_terms).
 struct CmpBoundTerms {
     float c, off;                // K2 >= (sum of ln us) / 2 - c (sum of um^2 / us) - off, 27 cells
     float off2;                  // K2 >= c (sum of q) + (sum of ln q) / 2 - off2, the 9 cells of a pair
     float slack;                 // the part of off that covers Stirling's remainders and rounding
     int minor;                   // the smaller class
 };
+
+// The table-free bounds.  With u = count + 1 per cell and class, us = u0 + u1, um the smaller class's
+// u, p = um / us, the entropy H in nats is bounded from below by a parabola that touches it at p0 =
+// (sum um) / (sum us), the same for every table:
+//     H(p) >= H(p0) + H'(p0) (p - p0) - c (p - p0)^2,  c = max over p of KL(p || p0) / (p - p0)^2,
+// and KL(p || p0) / (p - p0)^2 = integral over s in [0, 1] of (1 - s) / (t (1 - t)), t = p0 + s (p -
+// p0), is convex in p, so its largest value is at p = 0 or 1.  Summed with weights us the linear term
+// vanishes; S = sum us = N + 2 cells, sum um = p0 S.
+//
+// Pairs (9 cells): Stirling's form (lf(n) = (n + 1/2) ln(n + 1) - (n + 1) + ln(2 pi)/2 + e(n), 0 < e(n)
+// <= 1/(12 (n + 1))) makes K2 = sum us H + (1/2) sum ln q - cells ln(2 pi)/2 + remainders of at least
+// -1/6 a cell, q = um (us - um) / us, and sum us (p - p0)^2 = S p0 (1 - p0) - sum q, hence
+//     K2 >= c sum q + (1/2) sum ln q - [c S p0 (1 - p0) - S H(p0) + cells (ln(2 pi)/2 + 1/6)].
+//
+// Triplets (27 cells, the compacted scan): a cell's own term K = ln((us - 1)! / ((u0 - 1)! (u1 - 1)!))
+// obeys, for all u0, u1 >= 1,
+//     K >= us [H(p0) + H'(p0) (p - p0) - c (p - p0)^2] + (1/2) ln us + (1/2) ln(p0 (1 - p0)) -
+//          ln(2 pi)/2 - eps,   eps = max(0.125, 0.2346 - p0 / 4).
+// By Stirling's form the left side minus the right one is D = us [c (p - p0)^2 - KL(p || p0)] + (1/2)
+// ln(p (1 - p) / (p0 (1 - p0))) + m(us) - m(u0) - m(u1) + eps, m(z) = e(z - 1).  At fixed p, D grows
+// with the counts: the first term is not negative, and -z m'(z) lies between 1/(12 z) - 1/(120 z^3)
+// and 1/(12 z), so that scaling the counts up adds at least (0.9 (1/u0 + 1/u1) - 1/us)/12 > 0 per unit
+// of ln us.  So D >= 0 need only hold where the smaller count is 1, in real numbers: u1 = 1 or u0 = 1,
+// us >= 2, K = ln(us - 1), a function of us and p0.  There it is evaluated on a grid over every us and
+// p0 that a data set can have, not solved: its least value is 1.1e-4, at p0 -> 0, um = 1, us p0 = 2,
+// where the grid's steps are worth 1e-6 (tests/test_bound_range.py).  With sum us (p - p0)^2 =
+// sum um^2 / us - p0^2 S,
+//     K2 >= (1/2) sum ln us - c sum um^2 / us -
+//           [-S H(p0) - c p0^2 S + 27 (ln(2 pi)/2 - ln(p0 (1 - p0))/2 + eps)].
+//
+// c is the larger of the two p0's (a larger c is a weaker bound).  At the usual class shares it is 1.4 to
+// 1.8 times the parabola's own curvature, which costs a table without association (sum us (p - p0)^2 c
+// / 1.4 ~ 13 nats) 5 to 10 nats: about what the one-hot scan's bound loses to its doubled error term,
+// with a third of a reciprocal and a ninth of a log per cell instead of three logs.
+// FP32 rounding, S1 = sum um (q, um^2 / us <= um): every q or quotient
+// within 2^-21 of its um, S1 2^-21 together, c-fold; with q >= 1/2 once more in (1/2) ln q; the sums'
+// additions 27 2^-24 S1, c-fold; c's, the cut's and the last FMA's rounding 2^-24 (4 c S1 + 8 S + 200);
+// logs and products under 0.01; the FP32 score against K2: rel * K + abs as in build_k2_tables.  The
+// rounding terms are doubled.
+inline CmpBoundTerms cmp_bound_terms(int n0, int n1, float rel, float abs_) {
+    const int cm = n1 <= n0 ? 1 : 0;
+    const double nm = (double)(cm ? n1 : n0), N = (double)n0 + (double)n1;
+    auto p_of = [&](double cells) { return (nm + cells) / (N + 2.0 * cells); };
+    auto c_of = [](double p) {
+        return std::max(-std::log1p(-p) / (p * p), -std::log(p) / ((1.0 - p) * (1.0 - p)));
+    };
+    auto h_of = [](double p) { return -p * std::log(p) - (1.0 - p) * std::log1p(-p); };
+    const double c = std::max(c_of(p_of(27.0)), c_of(p_of(9.0)));
+    const double u = std::ldexp(1.0, -24), half_ln_2pi = 0.9189385332046727;
+    const double kmax = 27.0 * std::log(N + 2.0) + N * std::log(2.0);
+    const double S1 = nm + 27.0;
+    const double rnd = 8.0 * u * S1 * (c + 1.1) + 27.0 * u * S1 * c + u * (4.0 * c * S1 + 8.0 * N + 200.0) + 0.01 +
+                       (double)rel * kmax + (double)abs_;
+    const double S = N + 54.0, p = p_of(27.0), eps = std::max(0.125, 0.2346 - 0.25 * p);
+    const double off = -S * h_of(p) - c * p * p * S +
+                       27.0 * (half_ln_2pi - 0.5 * std::log(p * (1.0 - p)) + eps) + 2.0 * rnd;
+    const double S2 = N + 18.0, p2 = p_of(9.0);
+    const double off2 = c * S2 * p2 * (1.0 - p2) - S2 * h_of(p2) + 9.0 * (half_ln_2pi + 1.0 / 6.0) + 2.0 * rnd;
+    CmpBoundTerms b;
+    b.c = std::nextafter((float)c, INFINITY);
+    b.off = std::nextafter((float)off, INFINITY);
+    b.off2 = std::nextafter((float)off2, INFINITY);
+    b.slack = (float)(27.0 * eps + 2.0 * rnd);
+    b.minor = cm;
+    return b;
+}
 
 struct ScanArgs {
     Planes pl;
