@@ -219,7 +219,7 @@ int epi3_scan_checksum(epi3_handle* h, int32_t path, uint64_t* out_sum, int64_t*
  * up to 9377 SNPs); the first auto scan of a (n_snps / 64, n_samples / 1024) bucket
  * times each on the heaviest slice of pairs, at most 1/16 of them, and the choice is kept for
  * the process and appended to the file named by the environment variable EPI3_TUNE_CACHE,
- * if set, for later processes) | "popc" | "popc8" | "mma" | "mma16" | "mma4" | "mma4c";
+ * if set, for later processes of the same kernels -- lines of other versions are ignored) | "popc" | "popc8" | "mma" | "mma16" | "mma4" | "mma4c";
  * "autotune" = "1" (default) | "0" (no measuring: auto = EPI3_PATH_MMA4C, form plain);
  * "candidates" = initial length of the FP32 candidate list (64 .. 2^28; default 2^20 from
  * 2^22 triplets on, else 2^16; a scan that overflows it grows it 8x and runs again);

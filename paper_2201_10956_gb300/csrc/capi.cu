@@ -1761,8 +1761,9 @@ void batch_release(epi3_batch* b) {
 // scan kernels are timed on the cohort's heaviest pair slice (pairs with the smallest j,
 // about 1/16 of the pairs) and the lower kernel time per triplet wins.  Results are kept
 // per (M / 64, N / 1024) bucket for the process, and in the file named by EPI3_TUNE_CACHE
-// (lines "device<TAB>SMs<TAB>M/64<TAB>N/1024<TAB>path[<TAB>form<TAB>scope]") across
-// processes.  Scope 0 = a batch cohort's path, 1 = a handle's auto path and form, 2 = the
+// (lines "device kernels-R<TAB>SMs<TAB>M/64<TAB>N/1024<TAB>path[<TAB>form<TAB>scope]") across
+// processes.  R = kTuneKernels counts the changes after which the forms compare differently: a file's
+// lines of another R, or of none, are left alone and their buckets measured again.  Scope 0 = a batch cohort's path, 1 = a handle's auto path and form, 2 = the
 // form of an explicitly chosen tensor path.
 struct TuneEntry {
     std::string dev;
@@ -1777,6 +1778,10 @@ std::string device_name(int dev) {
     if (cudaGetDeviceProperties(&p, dev) != cudaSuccess) return "unknown";
     return p.name;
 }
+
+// Raise it with every change that makes one scan form faster or slower than before.
+constexpr int kTuneKernels = 2;
+std::string tune_device(int dev) { return device_name(dev) + " kernels-" + std::to_string(kTuneKernels); }
 
 void tune_load() {
     if (g_tune_loaded) return;
@@ -1840,7 +1845,7 @@ int tune_handle(epi3_handle* h) {
     }
     const int scope = want_path ? 1 : 2;
     tune_load();
-    const std::string dev = device_name(h->device);
+    const std::string dev = tune_device(h->device);
     const int mb = h->M / 64, nb = h->N / 1024;
     for (const TuneEntry& e : g_tune)
         if (e.dev == dev && e.sms == h->sm_count && e.mb == mb && e.nb == nb && e.scope == scope &&
