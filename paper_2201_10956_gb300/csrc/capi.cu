@@ -2301,18 +2301,22 @@ int epi3_batch_scan(epi3_batch* b, int32_t top_k, int32_t* out_triplets, double*
     if (dev) CK(cudaStreamSynchronize(b->stream), "copy outputs");
     epi3_stats& s = b->stats;
     s = epi3_stats{};
-    int n_mma = 0;
+    // per cohort seed and candidate stage, and its scan's launches: one for POPC, three per range of
+    // first SNPs for the compacted form, one for all one-hot cohorts together
+    s.kernel_launches = 2 * b->n + (b->n_tiles > 0 ? 1 : 0);
+    s.path = b->path[0];
     for (int c = 0; c < b->n; ++c) {
         const long long m = b->h[c]->M;
         s.n_triplets += m * (m - 1) * (m - 2) / 6;
         s.n_candidates += b->h_ctrls[c].n_cand;
         s.n_rescored += b->h_ctrls[c].n_final;
-        n_mma += b->path[c] == EPI3_PATH_MMA4;
+        if (b->path[c] != s.path) s.path = EPI3_PATH_AUTO;   // more than one form
+        if (b->path[c] == EPI3_PATH_MMA4C) s.kernel_launches += 3 * (int)b->h[c]->plan.range_start.size();
+        else if (b->path[c] == EPI3_PATH_POPC8) s.kernel_launches += 1;
     }
-    s.path = n_mma == b->n ? EPI3_PATH_MMA4 : (n_mma == 0 ? EPI3_PATH_POPC8 : EPI3_PATH_AUTO);
     s.grid = b->sm_count;
-    s.block = mma_threads(b->split);
-    s.kernel_launches = b->n + (b->n_tiles > 0 ? 1 : 0) + (b->n - n_mma) + b->n;
+    s.block = b->n_tiles > 0 ? mma_threads(b->split)
+              : s.path == EPI3_PATH_POPC8 ? b->h[0]->threads : scan_cmp_threads();
     // device time of the whole graph replay (scan kernels + candidate stages + read-back);
     // the scan kernels are > 99 % of it
     cudaEventElapsedTime(&s.total_ms, b->ev[0], b->ev[4]);
