@@ -738,7 +738,8 @@ Out out_mode(const epi3_handle* h, const int32_t* out_trip, const double* out_sc
 int finish_scan(epi3_handle* h, int top_k, int attempt, Out mode, int32_t* out_trip, double* out_scores) {
     const bool direct = mode == Out::kKernel;
     CK(launch_answer(h->pl, h->k2, h->d_ctrl, h->d_cand, h->cand_cap, top_k, h->d_fin,
-                     direct ? out_scores : h->d_out_scores, direct ? out_trip : h->d_out_trip, h->stream),
+                     direct ? out_scores : h->d_out_scores, direct ? out_trip : h->d_out_trip, h->sm_count,
+                     h->stream),
        "candidate stage launch");
     CK(cudaEventRecord(h->ev[3], h->stream), "event");
     CK(cudaMemcpyAsync(h->h_ctrl, h->d_ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, h->stream),
@@ -2070,7 +2071,7 @@ int batch_capture(epi3_batch* b, int top_k) {
         epi3_handle* h = b->h[c];
         ok(launch_answer(h->pl, h->k2, h->d_ctrl, h->d_cand, h->cand_cap, top_k, h->d_fin,
                          b->d_scores + (size_t)c * EPI3_MAX_TOPK, b->d_trip + (size_t)c * 3 * EPI3_MAX_TOPK,
-                         b->stream));
+                         b->sm_count, b->stream));
     }
     cur = "read-back";
     cur_c = -1;

@@ -196,7 +196,7 @@ cudaError_t launch_seed(const Planes& pl, const K2Tables& k2, Ctrl* ctrl, Cand* 
                         long long pair_begin, long long pair_end, int top_k, cudaStream_t st);
 // The candidate stage: the answer from the scan's candidates.
 cudaError_t launch_answer(const Planes& pl, const K2Tables& k2, Ctrl* ctrl, const Cand* cand, long long cap,
-                          int top_k, Final* fin, double* out_scores, int* out_trip, cudaStream_t st);
+                          int top_k, Final* fin, double* out_scores, int* out_trip, int sms, cudaStream_t st);
 cudaError_t launch_tables(const Planes& pl, const PairTables* pt, const K2Tables* k2, long long n,
                           const int* trip, int* out_counts, float* out_s32, double* out_s64,
                           Ctrl* ctrl, cudaStream_t st);

@@ -207,7 +207,7 @@ int scan_noalloc(const uint8_t* geno, const uint8_t* pheno, int M, int N, int to
     NA_CK(launch_seed(pl, k2, ctrl, cand, kNoAllocCandCap, 0, a.pair_end, top_k, st), "seed launch");
     if (L.eight) NA_CK(launch_scan_popc8(a, sms * occ, 128, smem, st), "scan launch");
     else NA_CK(launch_scan_popc(a, sms * occ, 128, smem, st), "scan launch");
-    NA_CK(launch_answer(pl, k2, ctrl, cand, kNoAllocCandCap, top_k, fin, out_scores, out_trip, st),
+    NA_CK(launch_answer(pl, k2, ctrl, cand, kNoAllocCandCap, top_k, fin, out_scores, out_trip, sms, st),
           "candidate stage launch");
     NA_CK(cudaMemcpyAsync(&hctrl, ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st), "read status");
     NA_CK(cudaStreamSynchronize(st), "scan");

@@ -10,7 +10,10 @@
 //              candidate inside the band recounts its 2 x 27 table (lanes split the sample groups,
 //              warp-shuffle sums of the 54 counts) and takes its FP64 K2 (Eq. 1, cell order
 //              0..26); the last CTA to finish sorts them by (K2, i, j, k) and writes the first
-//              top_k (Sec. III: the lowest K2 is the solution).
+//              top_k (Sec. III: the lowest K2 is the solution).  One CTA an SM: with 32 in all, 7140
+//              tied triplets of 100 000 samples cost 1093 us a scan instead of 561 (1000 samples: 446
+//              and 370), 512 rows of 131 072 samples 564 instead of 480; the smallest panels' 99 us
+//              are the same either way.
 //   tables   : warp per listed triplet, tables and/or FP32 and FP64 K2.
 #include "epi3_internal.cuh"
 
@@ -19,7 +22,6 @@ namespace epi3 {
 namespace {
 
 constexpr int kAnsThreads = 512;
-constexpr int kAnsCtas = 32;
 constexpr int kSeedThreads = 256;
 constexpr int kSeedMax = 2048;        // seed triplets, at most
 
@@ -392,11 +394,11 @@ cudaError_t launch_seed(const Planes& pl, const K2Tables& k2, Ctrl* ctrl, Cand* 
 }
 
 cudaError_t launch_answer(const Planes& pl, const K2Tables& k2, Ctrl* ctrl, const Cand* cand, long long cap,
-                          int top_k, Final* fin, double* out_scores, int* out_trip, cudaStream_t st) {
+                          int top_k, Final* fin, double* out_scores, int* out_trip, int sms, cudaStream_t st) {
     const size_t smem = (size_t)kFinalCap * sizeof(Final);
     cudaError_t e = cudaFuncSetAttribute(answer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    answer_kernel<<<kAnsCtas, kAnsThreads, smem, st>>>(pl, k2, ctrl, cand, cap, top_k, fin, out_scores, out_trip);
+    answer_kernel<<<sms, kAnsThreads, smem, st>>>(pl, k2, ctrl, cand, cap, top_k, fin, out_scores, out_trip);
     return cudaGetLastError();
 }
 
