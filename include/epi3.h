@@ -140,13 +140,18 @@ int epi3_scan_pairs(epi3_handle* h, int32_t top_k, int32_t* out_pairs, double* o
  * table (cell = the genotypes read as base-3 digits, x_0 most significant: 9 gX + 3 gY + gZ
  * for three) and its K2; the top_k sets by (K2 ascending, then the indices in order) are
  * returned.
- *   order        2 (= epi3_scan_pairs), 3 (= epi3_scan), or 4, 5, 6: every set counted by
- *                AND + POPC over the bit planes (81, 243 or 729 cells, plane 2 by NOR; order 4
- *                one set per thread, orders 5 and 6 one set per warp) and scored in FP64 in
- *                cell order with the rescoring table (needs M >= order, class sizes and M
- *                below 65536, and at most 4 GiB of selection scratch, about
+ *   order        2 (= epi3_scan_pairs), 3 (= epi3_scan), or 4, 5, 6 (needs M >= order, class sizes
+ *                and M below 65536, and at most 4 GiB of selection scratch, about
  *                C(M, order) / 2048 * top_k * 32 bytes); other orders give
- *                EPI3_ERR_UNSUPPORTED.
+ *                EPI3_ERR_UNSUPPORTED.  Every set's exact table comes from its 2^order cells with
+ *                genotypes 0 and 1 (AND + POPC over the bit planes) and the same counts of all
+ *                smaller sets; it is scored in FP32, and the sets within that score's error of the
+ *                k-th best in FP64 in cell order with the rescoring table.  The smaller sets'
+ *                counts take about C(M, order - 1) * 2^(order + 1) bytes of device memory during
+ *                the call, at most 16 GiB and a quarter of what is free; where that is not enough
+ *                all 3^order cells of every set are counted (plane 2 by NOR) and every set is
+ *                scored in FP64, as slow as that is.  Scratch of more than 256 MiB is given back
+ *                before the call returns, less is kept on the handle.
  *   top_k        1..min(EPI3_MAX_TOPK, C(M, order)).
  *   out_snps     [top_k][order] int32, increasing within a row, 0-based.
  *   out_scores   [top_k] FP64 K2, ascending.

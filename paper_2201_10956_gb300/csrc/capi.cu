@@ -48,7 +48,8 @@ int cuda_fail(cudaError_t e, const char* what) {
 // signals, so its bounded wait runs out (1 s) and the scan returns EPI3_ERR_TIMEOUT;
 // EPI3_FAULT=cand starts a handle with a 128-entry candidate list, so scans overflow it and
 // take the retry path with a larger list.  EPI3_FAULT=tables asks for more memory than there is
-// for the counted form of the four- to six-SNP scans, which then take the direct form.
+// for the counted form of the four- to six-SNP scans, which then take the direct form;
+// EPI3_FAULT=lowmem lets that form believe that the device has 1 MB left.
 bool inject(const char* what) {
     const char* f = getenv("EPI3_FAULT");
     return f && strcmp(f, what) == 0;
@@ -1385,6 +1386,41 @@ int epi3_scan_range(epi3_handle* h, int64_t pair_begin, int64_t pair_end, int32_
     return scan_impl(h, pair_begin, pair_end, top_k, out_triplets, out_scores, n_out, false);
 }
 
+}  // extern "C"
+
+namespace {
+
+// Scratch of the pair and the four- to six-SNP scans.  Up to kScratchKept stays on the handle for the
+// next call; a larger one is given back when the call ends, however it ends.
+constexpr size_t kScratchKept = (size_t)256 << 20;
+struct ScratchGuard {
+    epi3_handle* h;
+    ~ScratchGuard() {
+        if (h->pair_scratch_bytes <= kScratchKept) return;
+        dev_free(h->d_pair_scratch);
+        h->d_pair_scratch = nullptr;
+        h->pair_scratch_bytes = 0;
+    }
+};
+
+// The counted form's tables may take a quarter of the memory that is free, so that they never keep
+// the program beside them from its own allocations (small ones are not worth the question).
+bool tables_fit(size_t bytes) {
+    const bool low = inject("lowmem");
+    if (bytes <= kScratchKept && !low) return true;
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    if (low) free_bytes = (size_t)1 << 20;
+    return bytes <= free_bytes / 4;
+}
+
+}  // namespace
+
+extern "C" {
+
 int epi3_scan_pairs(epi3_handle* h, int32_t top_k, int32_t* out_pairs, double* out_scores) {
     g_err.clear();
     (void)cudaGetLastError();  // do not report an earlier call's error as ours
@@ -1396,7 +1432,8 @@ int epi3_scan_pairs(epi3_handle* h, int32_t top_k, int32_t* out_pairs, double* o
     int rc = ensure_pair_tables(h);
     if (rc != EPI3_OK) return rc;
     const size_t outs = sizeof(double) * (size_t)top_k + sizeof(int32_t) * 2 * (size_t)top_k;
-    auto scratch = [&](size_t bytes) -> int {   // kept on the handle; outputs after the first `bytes`
+    ScratchGuard guard{h};
+    auto scratch = [&](size_t bytes) -> int {   // outputs after the first `bytes`
         if (h->pair_scratch_bytes >= bytes + outs) return EPI3_OK;
         dev_free(h->d_pair_scratch);
         h->d_pair_scratch = nullptr;
@@ -1466,7 +1503,8 @@ int epi3_scan_order(epi3_handle* h, int32_t order, int32_t top_k, int32_t* out_s
         return fail(EPI3_ERR_UNSUPPORTED, "%d-SNP scan of %d SNPs with top_k %d needs %zu bytes of "
                     "selection scratch (limit 4 GiB)", order, h->M, top_k, sel);
     const size_t outs = sizeof(double) * (size_t)top_k + sizeof(int32_t) * order * (size_t)top_k;
-    auto scratch = [&](size_t bytes) -> int {   // kept on the handle; outputs after the first `bytes`
+    ScratchGuard guard{h};
+    auto scratch = [&](size_t bytes) -> int {   // outputs after the first `bytes`
         if (h->pair_scratch_bytes >= bytes + outs) return EPI3_OK;
         dev_free(h->d_pair_scratch);
         h->d_pair_scratch = nullptr;
@@ -1482,11 +1520,11 @@ int epi3_scan_order(epi3_handle* h, int32_t order, int32_t top_k, int32_t* out_s
         d_sets = reinterpret_cast<int32_t*>(d_s + top_k);
     };
     CK(cudaEventRecord(h->ev[0], h->stream), "event");
-    // the counted form, unless its tables are too large (or there is no memory for them) or more
+    // the counted form, unless its tables are too large for it or for the memory that is free, or more
     // sets tie at the k-th score than it rescores; then the direct form
     bool done = false;
     const size_t cnt = set_scan_scratch(h->M, h->N, order);
-    if (cnt && scratch(inject("tables") ? (size_t)1 << 60 : cnt) == EPI3_OK) {
+    if (cnt && tables_fit(cnt) && scratch(inject("tables") ? (size_t)1 << 60 : cnt) == EPI3_OK) {
         place(cnt);
         CK(launch_set_scan(h->pl, h->k2.lf64, h->N0, h->N1, order, top_k, h->sm_count, h->d_pair_scratch,
                            h->h_ctrl, d_sets, d_s, &done, h->stream), "k-SNP scan launch");
