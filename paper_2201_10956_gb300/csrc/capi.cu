@@ -47,7 +47,7 @@ int cuda_fail(cudaError_t e, const char* what) {
 // EPI3_FAULT=timeout makes the tensor-core scan's MMA issuer wait on a barrier nobody
 // signals, so its bounded wait runs out (1 s) and the scan returns EPI3_ERR_TIMEOUT;
 // EPI3_FAULT=cand starts a handle with a 128-entry candidate list, so scans overflow it and
-// take the retry path with a larger list.  EPI3_FAULT=tables asks for more memory than there is
+// take the retry path with a larger list, and leaves the scans of other orders a list of 1024.  EPI3_FAULT=tables asks for more memory than there is
 // for the counted form of the four- to six-SNP scans, which then take the direct form;
 // EPI3_FAULT=lowmem lets that form believe that the device has 1 MB left.
 bool inject(const char* what) {
@@ -1417,6 +1417,15 @@ bool tables_fit(size_t bytes) {
     return bytes <= free_bytes / 4;
 }
 
+// Most entries of the candidate list of a pair or four- to six-SNP scan.
+unsigned most_cands() { return inject("cand") ? 1024u : ~0u; }
+
+// A block of device memory for the rest of a call.
+struct TempBlock {
+    void* p = nullptr;
+    ~TempBlock() { dev_free(p); }
+};
+
 }  // namespace
 
 extern "C" {
@@ -1452,15 +1461,15 @@ int epi3_scan_pairs(epi3_handle* h, int32_t top_k, int32_t* out_pairs, double* o
     if ((rc = scratch(flt)) != EPI3_OK) return rc;
     place(flt);
     CK(cudaEventRecord(h->ev[0], h->stream), "event");
-    bool done = false;
-    CK(launch_pair_filter(h->ptab, h->k2.lf64, h->M, top_k, h->bound, h->sm_count, h->d_pair_scratch, h->h_ctrl,
-                          d_pairs, d_s, &done, h->stream), "pair scan launch");
-    if (!done) {   // thousands of pairs tie at the k-th score: every pair sorted
+    ThresholdInfo info{};
+    CK(launch_pair_filter(h->ptab, h->k2.lf64, h->M, top_k, h->bound, h->sm_count, most_cands(), h->d_pair_scratch,
+                          h->h_ctrl, d_pairs, d_s, &info, h->stream), "pair scan launch");
+    if (!info.done) {   // more pairs tie at the k-th score than the list holds: every pair scored
         const size_t sel = (pair_scan_scratch(np, top_k) + 255) & ~(size_t)255;
         if ((rc = scratch(sel)) != EPI3_OK) return rc;
         place(sel);
-        CK(launch_pair_scan(h->ptab, h->k2.lf64, h->M, top_k, h->d_pair_scratch, d_pairs, d_s,
-                            h->stream), "pair scan launch");
+        CK(launch_pair_scan(h->ptab, h->k2.lf64, h->M, info.thr, top_k, h->d_pair_scratch, d_pairs, d_s,
+                            &info.launches, h->stream), "pair scan launch");
     }
     CK(cudaEventRecord(h->ev[1], h->stream), "event");
     const cudaMemcpyKind kind =
@@ -1471,8 +1480,9 @@ int epi3_scan_pairs(epi3_handle* h, int32_t top_k, int32_t* out_pairs, double* o
     CK(cudaStreamSynchronize(h->stream), "pair scan");
     epi3_stats& s = h->stats;
     s.n_triplets = np;  // pairs scored
-    s.n_candidates = 0;
-    s.n_rescored = np;
+    s.n_candidates = info.n_cand;
+    s.n_rescored = info.done ? info.n_final : np;
+    s.kernel_launches = info.launches;
     s.path = EPI3_PATH_AUTO;
     cudaEventElapsedTime(&s.scan_kernel_ms, h->ev[0], h->ev[1]);
     s.total_ms = s.scan_kernel_ms;
@@ -1520,14 +1530,23 @@ int epi3_scan_order(epi3_handle* h, int32_t order, int32_t top_k, int32_t* out_s
         d_sets = reinterpret_cast<int32_t*>(d_s + top_k);
     };
     CK(cudaEventRecord(h->ev[0], h->stream), "event");
-    // the counted form, unless its tables are too large for it or for the memory that is free, or more
-    // sets tie at the k-th score than it rescores; then the direct form
+    // the counted form, unless its tables are too large for it or for the memory that is free; where
+    // more sets tie at the k-th score than its list holds, every set is scored: four SNPs from its
+    // tables, five and six by the direct form
+    ThresholdInfo info{};
+    TempBlock sorted;
     bool done = false;
     const size_t cnt = set_scan_scratch(h->M, h->N, order);
     if (cnt && tables_fit(cnt) && scratch(inject("tables") ? (size_t)1 << 60 : cnt) == EPI3_OK) {
         place(cnt);
-        CK(launch_set_scan(h->pl, h->k2.lf64, h->N0, h->N1, order, top_k, h->sm_count, h->d_pair_scratch,
-                           h->h_ctrl, d_sets, d_s, &done, h->stream), "k-SNP scan launch");
+        CK(launch_set_scan(h->pl, h->k2.lf64, h->N0, h->N1, order, top_k, h->sm_count, most_cands(), h->d_pair_scratch,
+                           h->h_ctrl, d_sets, d_s, &info, h->stream), "k-SNP scan launch");
+        done = info.done;
+        if (!done && order == 4 && dev_alloc(&sorted.p, sel) == cudaSuccess) {
+            CK(launch_quad_tied(h->pl, h->k2.lf64, h->N0, h->N1, info.thr, top_k, h->d_pair_scratch, sorted.p, d_sets,
+                                d_s, &info.launches, h->stream), "four-SNP scan launch");
+            done = true;
+        }
     }
     if (!done) {
         g_err.clear();
@@ -1536,10 +1555,10 @@ int epi3_scan_order(epi3_handle* h, int32_t order, int32_t top_k, int32_t* out_s
         place(sel);
         if (order == 4)
             CK(launch_quad_scan(h->pl, h->k2.lf64, h->N0, h->N1, top_k, h->d_pair_scratch, d_sets, d_s,
-                                h->stream), "four-SNP scan launch");
+                                &info.launches, h->stream), "four-SNP scan launch");
         else
-            CK(launch_order_scan(h->pl, h->k2.lf64, order, top_k, h->d_pair_scratch, d_sets, d_s, h->stream),
-               "k-SNP scan launch");
+            CK(launch_order_scan(h->pl, h->k2.lf64, order, top_k, h->d_pair_scratch, d_sets, d_s, &info.launches,
+                                 h->stream), "k-SNP scan launch");
     }
     CK(cudaEventRecord(h->ev[1], h->stream), "event");
     const cudaMemcpyKind kind =
@@ -1550,8 +1569,9 @@ int epi3_scan_order(epi3_handle* h, int32_t order, int32_t top_k, int32_t* out_s
     CK(cudaStreamSynchronize(h->stream), "k-SNP scan");
     epi3_stats& s = h->stats;
     s.n_triplets = nq;  // sets scored
-    s.n_candidates = 0;
-    s.n_rescored = nq;
+    s.n_candidates = info.n_cand;
+    s.n_rescored = info.done ? info.n_final : nq;
+    s.kernel_launches = info.launches;
     s.path = EPI3_PATH_POPC;
     cudaEventElapsedTime(&s.scan_kernel_ms, h->ev[0], h->ev[1]);
     s.total_ms = s.scan_kernel_ms;

@@ -203,33 +203,44 @@ cudaError_t launch_tables(const Planes& pl, const PairTables* pt, const K2Tables
 cudaError_t launch_reset(Ctrl* ctrl, cudaStream_t st);
 // Pairwise scan (Eq. 1 for two SNPs): the k best pairs by (FP64 K2, i, j) from the pair tables.
 size_t pair_scan_scratch(long long n_pairs, int k);
-cudaError_t launch_pair_scan(const PairTables& pt, const double* lf64, int M, int k,
-                             void* scratch, int32_t* out_pairs, double* out_s, cudaStream_t st);
-// The same by a threshold from a sample of the pairs and a table-free bound; *done false: the direct
-// form must answer (thousands of pairs tie at the k-th score).  Reads a few words back into h_ctrl
-// (pinned) and synchronises.
+// Pairs above thr are left out: an upper bound of the k-th score, or +inf.  *launches: kernels added.
+cudaError_t launch_pair_scan(const PairTables& pt, const double* lf64, int M, float thr, int k,
+                             void* scratch, int32_t* out_pairs, double* out_s, int* launches, cudaStream_t st);
+// What a thresholded scan says of itself.
+struct ThresholdInfo {
+    bool done;                   // false: more items tie at the threshold than the list holds
+    float thr;                   // upper bound of the k-th score
+    long long n_cand, n_final;   // candidates of the last pass, and those scored in FP64
+    int launches;
+};
+// The same by a threshold from a sample of the pairs and a table-free bound, through a list of at most
+// cap candidates (k at least; more than the scratch has room for are not used).  Reads a few words back
+// into h_ctrl (pinned) and synchronises.
 size_t pair_filter_scratch(long long n_pairs);
 cudaError_t launch_pair_filter(const PairTables& pt, const double* lf64, int M, int k, const CmpBoundTerms& bound,
-                               int sms, void* scratch, void* h_ctrl, int32_t* out_pairs, double* out_s, bool* done,
-                               cudaStream_t st);
+                               int sms, unsigned cap, void* scratch, void* h_ctrl, int32_t* out_pairs, double* out_s,
+                               ThresholdInfo* info, cudaStream_t st);
 // Four-SNP scan (Eq. 1 for four SNPs, 81 cells): the k best sets by (FP64 K2, i, j, k, l) from
 // the bit planes; needs both class sizes below 65536 and M below 65536.
 // orders 5 and 6: every set by AND + POPC (one warp per set), FP64 K2 in cell order
 long long order_count(int M, int order);
 size_t order_scan_scratch(int M, int order, int k);
 cudaError_t launch_order_scan(const Planes& pl, const double* lf64, int order, int k, void* scratch,
-                              int32_t* out_snps, double* out_s, cudaStream_t st);
-// The counted form of orders 4 to 6: scratch bytes (0: not for this size); *done false: more sets tie
-// at the k-th score than it rescores (the direct form answers).  Reads a few words back into h_ctrl
-// (pinned, at least 16 bytes) and synchronises.
+                              int32_t* out_snps, double* out_s, int* launches, cudaStream_t st);
+// The counted form of orders 4 to 6: scratch bytes (0: not for this size); cap, h_ctrl and info as
+// launch_pair_filter.
 size_t set_scan_scratch(int M, int N, int order);
 cudaError_t launch_set_scan(const Planes& pl, const double* lf64, int n0, int n1, int order, int k, int sms,
-                            void* scratch, void* h_ctrl, int32_t* out_snps, double* out_s, bool* done,
-                            cudaStream_t st);
+                            unsigned cap, void* scratch, void* h_ctrl, int32_t* out_snps, double* out_s,
+                            ThresholdInfo* info, cudaStream_t st);
+// Four SNPs, where that was not done: every set in FP64 from the counted form's tables, which
+// launch_set_scan left in `tables`; those above thr are left out.  scratch: as launch_quad_scan's.
+cudaError_t launch_quad_tied(const Planes& pl, const double* lf64, int n0, int n1, float thr, int k, void* tables,
+                             void* scratch, int32_t* out_snps, double* out_s, int* launches, cudaStream_t st);
 long long quad_count(int M);
 size_t quad_scan_scratch(int M, int k);
 cudaError_t launch_quad_scan(const Planes& pl, const double* lf64, int n0, int n1, int k,
-                             void* scratch, int32_t* out_snps, double* out_s, cudaStream_t st);
+                             void* scratch, int32_t* out_snps, double* out_s, int* launches, cudaStream_t st);
 // max over n in [0, n_lf) of (n + 1/2) |lg2_hw(n + 1) - log2(n + 1)| (FP64) into *out (device).
 cudaError_t launch_approx_error(const double* lf64, int n_lf, double* out, cudaStream_t st);
 cudaError_t launch_pair_tables(const Planes& pl, int4* pt, int2* marg, long long n_pairs,

@@ -10,8 +10,10 @@
 // from the same FP64 log-factorial table as the triplet rescoring, so it equals the oracle's
 // bit for bit.  The thresholded form (launch_pair_filter) bounds every pair from below without a
 // table and scores only those in FP64 whose bound does not exceed the threshold: 4096 SNPs x 4096
-// samples, k = 64, 1852 -> 223 us (pair tables read once, 268 MB).  The direct form scores and sorts
-// every pair; it answers where thousands of pairs tie at the k-th score.
+// samples, k = 64, 1852 -> 292 us (pair tables read once, 268 MB).  The direct form scores every pair
+// and sorts every 2048 of them that reach the threshold; it answers where more pairs tie at the k-th
+// score than the list of candidates holds (2500 of the 4096 SNPs without a variant: 1896 -> 1421 us;
+// all of them, where there is nothing to leave out: 1909 -> 2039 us).
 //
 // Four SNPs, the direct form: every set i < j < k < l gets its 3^4 = 81-cell table by AND + POPC over the bit
 // planes (plane 2 by NOR, pad bits land in cell 80 and are subtracted), built as a product
@@ -27,7 +29,9 @@
 // both classes in one register and one three-input subtraction per cell: 4 SNPs of 120 with 2000
 // samples 13.9 -> 2.41 ms, 5 of 48 with 1500 59.2 -> 1.37 ms.  The direct forms
 // (81, 243 or 729 cells counted, every set scored in FP64) serve what the counted form refuses:
-// tables of the smaller sets past kSubsetBytes, or more sets tied at the k-th score than it rescores.
+// tables of the smaller sets past kSubsetBytes, or, with five and six SNPs, more sets tied at the k-th
+// score than the list of candidates holds; with four, every set is then counted the same way and
+// scored in FP64 (launch_quad_tied).
 //
 // Selection (pairs and the direct forms): each block scores 2048 consecutive items and keeps its k best (bitonic
 // sort in shared memory); further passes merge 2048 survivors per block until one block
@@ -113,13 +117,14 @@ __device__ __forceinline__ double pair_score(const int (&r)[2][9], const double*
     return s;
 }
 
-// Pass 1 of the direct form: score pairs [b * 2048, (b + 1) * 2048), keep the block's k best in
-// out[b * k ..].
+// Pass 1 of the direct form: score pairs [b * 2048, (b + 1) * 2048), keep the block's k best of those
+// at or below thr in out[b * k ..] (a block without any sorts nothing).
 __global__ void __launch_bounds__(kPairThreads)
 pair_score_kernel(PairTables pt, const double* __restrict__ lf64, int M, long long n_pairs,
-                  int k, Item* __restrict__ out) {
+                  float thr, int k, Item* __restrict__ out) {
     __shared__ Item it[kPairBlock];
     const long long p0 = (long long)blockIdx.x * kPairBlock;
+    bool any = false;
     for (int t = threadIdx.x; t < kPairBlock; t += kPairThreads) {
         const long long p = p0 + t;
         it[t] = pad_item();
@@ -127,10 +132,13 @@ pair_score_kernel(PairTables pt, const double* __restrict__ lf64, int M, long lo
         int i, j, r[2][9];
         decode_pair(p, &i, &j);
         // exact counts cannot be negative; a corrupt table is ranked last, never looked up
-        if (pair_cells(pt, M, p, i, j, r)) it[t] = Item{pair_score(r, lf64), (long long)i * M + j};
+        if (!pair_cells(pt, M, p, i, j, r)) continue;
+        const double s = pair_score(r, lf64);
+        if (!(s <= (double)thr)) continue;
+        it[t] = Item{s, (long long)i * M + j};
+        any = true;
     }
-    __syncthreads();
-    sort_items(it);
+    if (__syncthreads_or(any)) sort_items(it);
     for (int t = threadIdx.x; t < k; t += kPairThreads) out[(long long)blockIdx.x * k + t] = it[t];
 }
 
@@ -146,8 +154,39 @@ pair_merge_kernel(const Item* __restrict__ in, long long n, int k, Item* __restr
     for (int t = threadIdx.x; t < k; t += kPairThreads) out[(long long)blockIdx.x * k + t] = it[t];
 }
 
-__global__ void pair_emit_kernel(const Item* __restrict__ best, int k, int M,
+// The k best of n items, k from each 2048, in passes over the buffers a and b until one block is left;
+// *best: where they are.  Items in `in` (which may be a).
+cudaError_t merge_items(const Item* in, long long n, int k, Item* a, Item* b, const Item** best, int* launches,
+                        cudaStream_t st) {
+    while (n > k) {
+        const long long blocks = (n + kPairBlock - 1) / kPairBlock;
+        Item* const out = in == a ? b : a;
+        pair_merge_kernel<<<(unsigned)blocks, kPairThreads, 0, st>>>(in, n, k, out);
+        ++*launches;
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        in = out;
+        n = blocks * k;
+    }
+    *best = in;
+    return cudaSuccess;
+}
+
+// Control block of the thresholded forms.
+struct SetCtrl {
+    float thr, last;             // threshold, and the one before
+    unsigned n_cand, n_final;    // candidates met (the list holds the first `cap`), rescored ones
+    unsigned tied;               // the sample says that more tie at the threshold than the list holds
+};
+// The answer is in fin[0 .. n_final), to be sorted by one block.
+__device__ __forceinline__ bool in_one_block(const SetCtrl* ctrl, unsigned cap) {
+    return ctrl->n_cand <= cap && ctrl->n_final <= (unsigned)kPairBlock;
+}
+
+// (ctrl: null, or nothing is written unless its answer is in one block)
+__global__ void pair_emit_kernel(const Item* __restrict__ best, int k, int M, const SetCtrl* ctrl, unsigned cap,
                                  int32_t* __restrict__ out_pairs, double* __restrict__ out_s) {
+    if (ctrl && !in_one_block(ctrl, cap)) return;
     for (int t = threadIdx.x; t < k; t += blockDim.x) {
         const Item e = best[t];
         out_pairs[2 * t] = (int32_t)(e.key / M);
@@ -427,10 +466,13 @@ order_score_kernel(Planes pl, const double* __restrict__ lf64, long long n_sets,
 }
 
 template <int K>
-__global__ void order_emit_kernel(const Item* __restrict__ best, int k, int M,
+__global__ void order_emit_kernel(const Item* __restrict__ best, int k, int M, const SetCtrl* ctrl, unsigned cap,
                                   int32_t* __restrict__ out_snps, double* __restrict__ out_s) {
+    if (ctrl && !in_one_block(ctrl, cap)) return;
+    const long long n_sets = choose_ll(M, K);
     for (int t = threadIdx.x; t < k; t += blockDim.x) {
         const Item e = best[t];
+        if ((unsigned long long)e.key >= (unsigned long long)n_sets) continue;   // no rank: nothing to decode
         int x[K];
         decode_lex<K>(e.key, M, x);
 #pragma unroll
@@ -441,25 +483,17 @@ __global__ void order_emit_kernel(const Item* __restrict__ best, int k, int M,
 
 template <int K>
 cudaError_t order_scan_k(const Planes& pl, const double* lf64, int k, void* scratch,
-                         int32_t* out_snps, double* out_s, cudaStream_t st) {
+                         int32_t* out_snps, double* out_s, int* launches, cudaStream_t st) {
     const long long n_sets = choose_ll(pl.M, K);
-    long long blocks = (n_sets + kPairBlock - 1) / kPairBlock;
-    Item* a = static_cast<Item*>(scratch);
-    Item* b = a + blocks * k;
+    const long long blocks = (n_sets + kPairBlock - 1) / kPairBlock;
+    Item* const a = static_cast<Item*>(scratch);
     order_score_kernel<K><<<(unsigned)blocks, kOrdThreads, 0, st>>>(pl, lf64, n_sets, k, a);
     cudaError_t e = cudaGetLastError();
-    long long n = blocks * k;
-    while (e == cudaSuccess && blocks > 1) {
-        blocks = (n + kPairBlock - 1) / kPairBlock;
-        pair_merge_kernel<<<(unsigned)blocks, kPairThreads, 0, st>>>(a, n, k, b);
-        e = cudaGetLastError();
-        n = blocks * k;
-        Item* tmp = a;
-        a = b;
-        b = tmp;
-    }
+    const Item* best = nullptr;
+    if (e == cudaSuccess) e = merge_items(a, blocks * k, k, a, a + blocks * k, &best, launches, st);
     if (e != cudaSuccess) return e;
-    order_emit_kernel<K><<<1, 512, 0, st>>>(a, k, pl.M, out_snps, out_s);
+    order_emit_kernel<K><<<1, 512, 0, st>>>(best, k, pl.M, nullptr, 0u, out_snps, out_s);
+    *launches += 2;
     return cudaGetLastError();
 }
 
@@ -481,10 +515,6 @@ struct SetCand {
     long long q;                 // rank
     float s;
 };
-struct SetCtrl {
-    float thr;
-    unsigned n_cand, n_final;
-};
 
 __device__ __forceinline__ long long binom_at(const SetArgs& a, int x, int t) {
     return __ldg(a.binom + (size_t)t * (a.pl.M + 1) + x);
@@ -505,6 +535,15 @@ __device__ __forceinline__ void decode_colex(const SetArgs& a, long long q, int*
         x[t - 1] = lo;
         hi = lo;
     }
+}
+
+// Its rank in lexicographic order, the tie key.
+template <int K>
+__device__ __forceinline__ long long lex_rank(const SetArgs& a, const int* x) {
+    long long lex = a.n_sets - 1;
+#pragma unroll
+    for (int t = 0; t < K; ++t) lex -= binom_at(a, a.pl.M - 1 - x[t], K - t);
+    return lex;
 }
 
 __global__ void set_tables_kernel(int M, const double* __restrict__ lf64, int n_lf,
@@ -690,12 +729,59 @@ __device__ __forceinline__ void outer_cells(const SetArgs& a, const int* x, cons
     }
 }
 
+// add(27 cells) for the whole table of a set, in cell order; own: its own counts (count_cells).
+template <int K, class Add>
+__device__ __forceinline__ void all_cells(const SetArgs& a, const int* x, const uint32_t* own, Add add) {
+#pragma unroll 1
+    for (int outer = 0; outer < (K == 4 ? 1 : K == 5 ? 3 : 9); ++outer) {
+        // position K - 4: genotypes 0 and 1, then 2 as what is left of any
+        uint32_t any[27], g[27];
+        auto step = [&](int o) {
+            outer_cells<K>(a, x, own, o, 2, any);
+#pragma unroll
+            for (int mid = 0; mid < 2; ++mid) {
+                outer_cells<K>(a, x, own, o, mid, g);
+                add(g);
+#pragma unroll
+                for (int e = 0; e < 27; ++e) any[e] -= g[e];
+            }
+            add(any);
+        };
+        if (K == 4) step(0);
+        else if (K == 5) {
+            if (outer == 0) step(0);
+            else if (outer == 1) step(1);
+            else step(2);
+        } else {
+            switch (outer) {
+                case 0: step(0); break;
+                case 1: step(1); break;
+                case 2: step(2); break;
+                case 3: step(3); break;
+                case 4: step(4); break;
+                case 5: step(5); break;
+                case 6: step(6); break;
+                case 7: step(7); break;
+                default: step(8); break;
+            }
+        }
+    }
+}
 // Adds the 27 cells' K2 terms in FP32.
 __device__ __forceinline__ float add_terms(const float* lf, const uint32_t* g, float s) {
 #pragma unroll
     for (int e = 0; e < 27; ++e) {
         const uint32_t r0 = g[e] & 0xFFFFu, r1 = g[e] >> 16;
         s += (lf[r0 + r1 + 1] - lf[r0]) - lf[r1];
+    }
+    return s;
+}
+// The same in FP64, every operation that of the direct forms.
+__device__ __forceinline__ double add_terms64(const double* __restrict__ lf64, const uint32_t* g, double s) {
+#pragma unroll 3
+    for (int e = 0; e < 27; ++e) {
+        const uint32_t r0 = g[e] & 0xFFFFu, r1 = g[e] >> 16;
+        s = __dadd_rn(s, __dsub_rn(__dsub_rn(lf64[r0 + r1 + 1], lf64[r0]), lf64[r1]));
     }
     return s;
 }
@@ -715,6 +801,7 @@ set_scan_kernel(const SetArgs a, long long stride, long long n, float* __restric
         __syncthreads();
     }
     const float* const lf = kSmemLf ? s_lf : a.lf;
+    if (!sample && ctrl->n_cand > cap) return;   // full: the sample says so, or this pass so far
     const float thr = sample ? 0.f : ctrl->thr;
     for (long long t = (long long)blockIdx.x * kSetThreads + threadIdx.x; t < n;
          t += (long long)gridDim.x * kSetThreads) {
@@ -724,40 +811,7 @@ set_scan_kernel(const SetArgs a, long long stride, long long n, float* __restric
         uint32_t own[1 << K];
         count_cells<K>(a.pl, x, own);
         float s = 0.f;
-#pragma unroll 1
-        for (int outer = 0; outer < (K == 4 ? 1 : K == 5 ? 3 : 9); ++outer) {
-            // position K - 4: genotypes 0 and 1, then 2 as what is left of any
-            uint32_t any[27], g[27];
-            auto step = [&](int o) {
-                outer_cells<K>(a, x, own, o, 2, any);
-#pragma unroll
-                for (int mid = 0; mid < 2; ++mid) {
-                    outer_cells<K>(a, x, own, o, mid, g);
-                    s = add_terms(lf, g, s);
-#pragma unroll
-                    for (int e = 0; e < 27; ++e) any[e] -= g[e];
-                }
-                s = add_terms(lf, any, s);
-            };
-            if (K == 4) step(0);
-            else if (K == 5) {
-                if (outer == 0) step(0);
-                else if (outer == 1) step(1);
-                else step(2);
-            } else {
-                switch (outer) {
-                    case 0: step(0); break;
-                    case 1: step(1); break;
-                    case 2: step(2); break;
-                    case 3: step(3); break;
-                    case 4: step(4); break;
-                    case 5: step(5); break;
-                    case 6: step(6); break;
-                    case 7: step(7); break;
-                    default: step(8); break;
-                }
-            }
-        }
+        all_cells<K>(a, x, own, [&](const uint32_t* g) { s = add_terms(lf, g, s); });
         s = fmaxf(s, 0.f);
         if (sample) {
             sample[t] = s;
@@ -770,13 +824,18 @@ set_scan_kernel(const SetArgs a, long long stride, long long n, float* __restric
 
 // The k-th smallest score (scores are not negative: their bit patterns sort like them) of n floats
 // `step` floats apart; ctrl->thr becomes that + 2 delta, rounded up: no set of the answer scores
-// higher.  One block.
+// higher.  One block.  Of the list (n_dev) its first `cap` candidates; of a sample of every `stride`-th
+// item also whether the items that tie at the k-th score alone would overflow the list, which is then
+// marked full before the scan begins.
 __global__ void __launch_bounds__(1024)
 set_threshold_kernel(const float* __restrict__ v, int step, long long n, const unsigned* __restrict__ n_dev,
-                     int k, float delta, SetCtrl* ctrl) {
+                     int k, float delta, long long stride, unsigned cap, SetCtrl* ctrl) {
     __shared__ unsigned hist[256];
-    __shared__ unsigned s_prefix, s_rank;
-    if (n_dev) n = min(n, (long long)*n_dev);
+    __shared__ unsigned s_prefix, s_rank, s_ties;
+    if (n_dev) {
+        if (ctrl->tied) return;
+        n = min(n, (long long)*n_dev);
+    }
     const int tid = threadIdx.x, lane = tid & 31;
     if (tid == 0) {
         s_prefix = 0u;
@@ -807,6 +866,7 @@ set_threshold_kernel(const float* __restrict__ v, int step, long long n, const u
                 int b = 0;
                 while (before + c[b] < rank) before += c[b++];
                 s_rank = rank - before;
+                s_ties = c[b];
                 s_prefix = prefix | ((unsigned)(8 * lane + b) << shift);
             }
         }
@@ -814,22 +874,26 @@ set_threshold_kernel(const float* __restrict__ v, int step, long long n, const u
         __syncthreads();
     }
     if (tid == 0) {
+        if (n_dev) ctrl->last = ctrl->thr;
+        else {
+            const bool tied = (double)s_ties * (double)stride > (double)cap;
+            ctrl->tied = tied ? 1u : 0u;
+            ctrl->n_cand = tied ? cap + 1u : 0u;
+        }
         ctrl->thr = __fadd_ru(__uint_as_float(s_prefix), 2.f * delta);
-        if (!n_dev) ctrl->n_cand = 0u;
         ctrl->n_final = 0u;
     }
 }
 
-// FP64 scores of the candidates inside the threshold, one warp each.
+// FP64 scores of the candidates inside the threshold, one warp each (none if the list overflowed).
 template <int K>
 __global__ void __launch_bounds__(kOrdThreads)
 set_rescore_kernel(const SetArgs a, const double* __restrict__ lf64, SetCtrl* ctrl,
-                   const SetCand* __restrict__ cand, unsigned cap, Item* __restrict__ fin, unsigned fin_cap) {
+                   const SetCand* __restrict__ cand, unsigned cap, Item* __restrict__ fin) {
     uint32_t code[(Pow3<K>::v + 31) / 32];
     lane_codes<K>(code);
-    const unsigned n = min(ctrl->n_cand, cap);
+    const unsigned n = ctrl->n_cand <= cap ? ctrl->n_cand : 0u;
     const float thr = ctrl->thr;
-    const int M = a.pl.M;
     for (unsigned e = blockIdx.x * (kOrdThreads / 32) + (threadIdx.x >> 5); e < n;
          e += gridDim.x * (kOrdThreads / 32)) {
         const SetCand cd = cand[e];
@@ -839,25 +903,51 @@ set_rescore_kernel(const SetArgs a, const double* __restrict__ lf64, SetCtrl* ct
         const double sc = set_score<K>(a.pl, lf64, x, code);
         if ((threadIdx.x & 31) == 0) {
             const unsigned pos = atomicAdd(&ctrl->n_final, 1u);
-            long long lex = a.n_sets - 1;      // rank in lexicographic order, the tie key
-#pragma unroll
-            for (int t = 0; t < K; ++t) lex -= binom_at(a, M - 1 - x[t], K - t);
-            if (pos < fin_cap) fin[pos] = Item{sc, lex};
+            fin[pos] = Item{sc, lex_rank<K>(a, x)};   // at most one per candidate
         }
     }
 }
 
-// The k best of at most kPairBlock rescored sets, sorted.
+// The k best of at most kPairBlock rescored sets, sorted (more are merged, pair_merge_kernel).
 __global__ void __launch_bounds__(kPairThreads)
-set_final_kernel(const SetCtrl* ctrl, const Item* __restrict__ fin, int k, Item* __restrict__ out) {
+set_final_kernel(const SetCtrl* ctrl, unsigned cap, const Item* __restrict__ fin, int k, Item* __restrict__ out) {
     __shared__ Item it[kPairBlock];
-    const int n = min(ctrl->n_final, (unsigned)kPairBlock);
+    if (!in_one_block(ctrl, cap)) return;
+    const int n = (int)ctrl->n_final;
     int n2 = 64;
     while (n2 < n || n2 < k) n2 <<= 1;
     for (int t = threadIdx.x; t < n2; t += kPairThreads) it[t] = t < n ? fin[t] : pad_item();
     __syncthreads();
     sort_items(it, n2);
     for (int t = threadIdx.x; t < k; t += kPairThreads) out[t] = it[t];
+}
+
+// Where more sets lie at the threshold than the list holds: every set scored in FP64 from its counted
+// table, a block's k best of 2048 consecutive ranks at or below thr into out[b * k ..], merged like the
+// direct form's.  Four SNPs only: there the passes before it are a sixth of the direct form's time
+// (60 SNPs x 1000 samples), with five and six a thirtieth.
+constexpr int kTiedThreads = 512;     // four sets each: with 128 threads 50 SNPs, fewer blocks than SMs, took 521 us for 421
+template <int K>
+__global__ void __launch_bounds__(kTiedThreads)
+set_tied_kernel(const SetArgs a, const double* __restrict__ lf64, float thr, int k, Item* __restrict__ out) {
+    __shared__ Item it[kPairBlock];
+    bool any = false;
+    for (int t = threadIdx.x; t < kPairBlock; t += kTiedThreads) {
+        const long long q = (long long)blockIdx.x * kPairBlock + t;
+        it[t] = pad_item();
+        if (q >= a.n_sets) continue;
+        int x[K];
+        decode_colex<K>(a, q, x);
+        uint32_t own[1 << K];
+        count_cells<K>(a.pl, x, own);
+        double s = 0.0;
+        all_cells<K>(a, x, own, [&](const uint32_t* g) { s = add_terms64(lf64, g, s); });
+        if (!(s <= (double)thr)) continue;
+        it[t] = Item{s, lex_rank<K>(a, x)};
+        any = true;
+    }
+    if (__syncthreads_or(any)) sort_items(it);
+    for (int t = threadIdx.x; t < k; t += kTiedThreads) out[(long long)blockIdx.x * k + t] = it[t];
 }
 
 // ---------------------------------------------------------------- pairs, thresholded form
@@ -880,6 +970,9 @@ pair_sample_kernel(PairTables pt, const double* __restrict__ lf64, int M, long l
 __global__ void __launch_bounds__(256)
 pair_filter_kernel(PairTables pt, const double* __restrict__ lf64, int M, float bound_c, float bound_off,
                    int minor, SetCtrl* ctrl, SetCand* __restrict__ cand, unsigned cap) {
+    // the list is full: the sample says so, or this pass so far (a load past L1 for every block cost 110
+    // us of 280)
+    if (ctrl->n_cand > cap) return;
     const float thr = ctrl->thr, cut = __fadd_ru(thr, bound_off);
     for (int j = 1 + blockIdx.y; j < M; j += gridDim.y) {
         const int i = blockIdx.x * 256 + threadIdx.x;
@@ -905,8 +998,8 @@ pair_filter_kernel(PairTables pt, const double* __restrict__ lf64, int M, float 
 }
 __global__ void __launch_bounds__(256)
 pair_rescore_kernel(PairTables pt, const double* __restrict__ lf64, int M, SetCtrl* ctrl,
-                    const SetCand* __restrict__ cand, unsigned cap, Item* __restrict__ fin, unsigned fin_cap) {
-    const unsigned n = min(ctrl->n_cand, cap);
+                    const SetCand* __restrict__ cand, unsigned cap, Item* __restrict__ fin) {
+    const unsigned n = ctrl->n_cand <= cap ? ctrl->n_cand : 0u;
     const float thr = ctrl->thr;
     for (unsigned e = blockIdx.x * 256 + threadIdx.x; e < n; e += gridDim.x * 256) {
         const SetCand cd = cand[e];
@@ -915,15 +1008,27 @@ pair_rescore_kernel(PairTables pt, const double* __restrict__ lf64, int M, SetCt
         decode_pair(cd.q, &i, &j);
         pair_cells(pt, M, cd.q, i, j, r);
         const unsigned pos = atomicAdd(&ctrl->n_final, 1u);
-        if (pos < fin_cap) fin[pos] = Item{pair_score(r, lf64), (long long)i * M + j};
+        fin[pos] = Item{pair_score(r, lf64), (long long)i * M + j};   // at most one per candidate
     }
 }
 
 constexpr unsigned kSetCand = 1u << 18;          // candidate list
 constexpr size_t kSubsetBytes = (size_t)16 << 30;   // counts of the smaller sets, at most
+// items of one of the two buffers that merge the rescored candidates
+constexpr size_t kMergeItems = (size_t)(kSetCand / kPairBlock) * EPI3_MAX_TOPK;
+
+// Entries of the list that a scan of n items uses.  A candidate of a pair or four-SNP scan costs some
+// ten times an item of the form that answers when the list overflows (230 300 tied sets of 50 SNPs x 500
+// samples: 1975 us through the list, 388 by the direct form), so an eighth of the items at most; with
+// five and six SNPs it costs the same.
+unsigned list_cap(long long n, int order, unsigned most) {
+    long long cap = kSetCand;
+    if (order <= 4 && n / 8 < cap) cap = n / 8 < kPairBlock ? kPairBlock : n / 8;
+    return cap < most ? (unsigned)cap : most;
+}
 
 struct SetLayout {
-    size_t binom, lf, ctrl, cand, fin, best, sample, sub[6], total;
+    size_t binom, lf, ctrl, cand, fin, best, merge, sample, sub[6], total;
     long long n_sample;
 };
 SetLayout set_layout(int M, int N, int order) {
@@ -940,8 +1045,9 @@ SetLayout set_layout(int M, int N, int order) {
     L.lf = take(sizeof(float) * ((size_t)N + 2));
     L.ctrl = take(sizeof(SetCtrl));
     L.cand = take(sizeof(SetCand) * kSetCand);
-    L.fin = take(sizeof(Item) * kPairBlock);
+    L.fin = take(sizeof(Item) * kSetCand);
     L.best = take(sizeof(Item) * EPI3_MAX_TOPK);
+    L.merge = take(sizeof(Item) * 2 * kMergeItems);
     L.sample = take(sizeof(float) * (size_t)L.n_sample);
     for (int t = 1; t < order; ++t) L.sub[t] = take((sizeof(uint32_t) << t) * (size_t)choose_ll(M, t));
     L.total = o;
@@ -956,18 +1062,59 @@ cudaError_t count_subsets(const SetArgs& a, int grid, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// Passes over the items until the list of candidates holds all of them, or cannot: *done false.  A
+// pass (`scan`) fills the list, `rescore` scores the candidates inside the list's own threshold in FP64
+// into fin, `emit` writes the answer.  One wait a pass.
+template <class Scan, class Rescore, class Emit>
+cudaError_t threshold_passes(int k, float delta, unsigned cap, char* base, size_t ctrl_at, size_t cand_at, size_t fin_at,
+                             size_t best_at, size_t merge_at, SetCtrl* h_ctrl, ThresholdInfo* info, cudaStream_t st,
+                             Scan scan, Rescore rescore, Emit emit) {
+    SetCtrl* const ctrl = reinterpret_cast<SetCtrl*>(base + ctrl_at);
+    SetCand* const cand = reinterpret_cast<SetCand*>(base + cand_at);
+    Item* const fin = reinterpret_cast<Item*>(base + fin_at);
+    Item* const best = reinterpret_cast<Item*>(base + best_at);
+    Item* const merge = reinterpret_cast<Item*>(base + merge_at);
+    info->done = false;
+    for (int attempt = 0;; ++attempt) {
+        scan(ctrl, cand);
+        // the threshold from the candidates themselves (any k of them bound the k-th)
+        set_threshold_kernel<<<1, 1024, 0, st>>>(&cand->s, sizeof(SetCand) / sizeof(float), cap, &ctrl->n_cand, k,
+                                                 delta, 1, cap, ctrl);
+        rescore(ctrl, cand, fin);
+        set_final_kernel<<<1, kPairThreads, 0, st>>>(ctrl, cap, fin, k, best);
+        emit(best, ctrl);
+        info->launches += 5;
+        cudaError_t e = cudaMemcpyAsync(h_ctrl, ctrl, sizeof(SetCtrl), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e == cudaSuccess) e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        info->thr = h_ctrl->thr;
+        info->n_cand = h_ctrl->n_cand;
+        info->n_final = h_ctrl->n_final;
+        if (h_ctrl->n_cand <= cap) {
+            info->done = true;
+            if (h_ctrl->n_final <= (unsigned)kPairBlock) return cudaSuccess;
+            const Item* top = nullptr;   // thousands at the k-th score
+            e = merge_items(fin, h_ctrl->n_final, k, merge, merge + kMergeItems, &top, &info->launches, st);
+            if (e != cudaSuccess) return e;
+            emit(top, nullptr);
+            ++info->launches;
+            return cudaGetLastError();
+        }
+        // the list overflowed: once more with the threshold of what it holds, if that is lower
+        if (h_ctrl->tied || !(h_ctrl->thr < h_ctrl->last) || attempt == 2) return cudaSuccess;
+        e = cudaMemsetAsync(&ctrl->n_cand, 0, sizeof(unsigned), st);
+        if (e != cudaSuccess) return e;
+    }
+}
+
 template <int K>
 cudaError_t set_scan_k(const SetArgs& a, const SetLayout& L, const double* lf64, int sms, int k, float delta,
-                       char* base, SetCtrl* h_ctrl, int32_t* out_snps, double* out_s, bool* done,
-                       cudaStream_t st) {
-    *done = false;
+                       unsigned cap, char* base, SetCtrl* h_ctrl, int32_t* out_snps, double* out_s,
+                       ThresholdInfo* info, cudaStream_t st) {
     const bool smem = a.n_lf <= kSetLfMax;
     const size_t bytes = smem ? sizeof(float) * (size_t)a.n_lf : 0;
-    SetCtrl* const ctrl = reinterpret_cast<SetCtrl*>(base + L.ctrl);
-    SetCand* const cand = reinterpret_cast<SetCand*>(base + L.cand);
     float* const sample = reinterpret_cast<float*>(base + L.sample);
-    Item* const fin = reinterpret_cast<Item*>(base + L.fin);
-    Item* const best = reinterpret_cast<Item*>(base + L.best);
     const int grid = 16 * sms;
     cudaError_t e = cudaSuccess;
     e = count_subsets<1>(a, grid, st);
@@ -976,38 +1123,28 @@ cudaError_t set_scan_k(const SetArgs& a, const SetLayout& L, const double* lf64,
     if (e == cudaSuccess && K > 4) e = count_subsets<4>(a, grid, st);
     if (e == cudaSuccess && K > 5) e = count_subsets<5>(a, grid, st);
     if (e != cudaSuccess) return e;
-    auto scan = [&](long long stride, long long n, float* smp) {
+    auto scan = [&](long long stride, long long n, float* smp, SetCtrl* ctrl, SetCand* cand) {
         const long long blocks = (n + kSetThreads - 1) / kSetThreads;
         const unsigned g = (unsigned)(blocks < grid ? blocks : grid);
-        if (smem) set_scan_kernel<K, true><<<g, kSetThreads, bytes, st>>>(a, stride, n, smp, ctrl, cand, kSetCand);
-        else set_scan_kernel<K, false><<<g, kSetThreads, 0, st>>>(a, stride, n, smp, ctrl, cand, kSetCand);
-        return cudaGetLastError();
+        if (smem) set_scan_kernel<K, true><<<g, kSetThreads, bytes, st>>>(a, stride, n, smp, ctrl, cand, cap);
+        else set_scan_kernel<K, false><<<g, kSetThreads, 0, st>>>(a, stride, n, smp, ctrl, cand, cap);
     };
-    e = scan(a.n_sets / L.n_sample, L.n_sample, sample);
+    SetCtrl* const ctrl = reinterpret_cast<SetCtrl*>(base + L.ctrl);
+    const long long stride = a.n_sets / L.n_sample;
+    scan(stride, L.n_sample, sample, ctrl, nullptr);
+    set_threshold_kernel<<<1, 1024, 0, st>>>(sample, 1, L.n_sample, nullptr, k, delta, stride, cap, ctrl);
+    info->launches += K + 1;
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    set_threshold_kernel<<<1, 1024, 0, st>>>(sample, 1, L.n_sample, nullptr, k, delta, ctrl);
-    for (int attempt = 0; attempt < 4; ++attempt) {
-        e = scan(1, a.n_sets, nullptr);
-        if (e != cudaSuccess) return e;
-        // the threshold from the candidates themselves (any set of k of them bounds the k-th)
-        set_threshold_kernel<<<1, 1024, 0, st>>>(&cand->s, sizeof(SetCand) / sizeof(float), kSetCand,
-                                                 &ctrl->n_cand, k, delta, ctrl);
-        set_rescore_kernel<K><<<4 * sms, kOrdThreads, 0, st>>>(a, lf64, ctrl, cand, kSetCand, fin, kPairBlock);
-        set_final_kernel<<<1, kPairThreads, 0, st>>>(ctrl, fin, k, best);
-        order_emit_kernel<K><<<1, 512, 0, st>>>(best, k, a.pl.M, out_snps, out_s);
-        e = cudaMemcpyAsync(h_ctrl, ctrl, sizeof(SetCtrl), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e == cudaSuccess) e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        if (h_ctrl->n_cand <= kSetCand) {
-            *done = h_ctrl->n_final <= (unsigned)kPairBlock;
-            return cudaSuccess;
-        }
-        // the list overflowed: once more with the threshold of what it holds
-        e = cudaMemsetAsync(&ctrl->n_cand, 0, sizeof(unsigned), st);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    return threshold_passes(
+        k, delta, cap, base, L.ctrl, L.cand, L.fin, L.best, L.merge, h_ctrl, info, st,
+        [&](SetCtrl* c, SetCand* cand) { scan(1, a.n_sets, nullptr, c, cand); },
+        [&](SetCtrl* c, const SetCand* cand, Item* fin) {
+            set_rescore_kernel<K><<<4 * sms, kOrdThreads, 0, st>>>(a, lf64, c, cand, cap, fin);
+        },
+        [&](const Item* top, const SetCtrl* c) {
+            order_emit_kernel<K><<<1, 512, 0, st>>>(top, k, a.pl.M, c, cap, out_snps, out_s);
+        });
 }
 
 }  // namespace
@@ -1024,20 +1161,27 @@ size_t set_scan_scratch(int M, int N, int order) {
     return set_layout(M, N, order).total;
 }
 
-cudaError_t launch_set_scan(const Planes& pl, const double* lf64, int n0, int n1, int order, int k, int sms,
-                            void* scratch, void* h_ctrl, int32_t* out_snps, double* out_s, bool* done,
-                            cudaStream_t st) {
-    const int N = n0 + n1;
-    const SetLayout L = set_layout(pl.M, N, order);
-    char* const base = static_cast<char*>(scratch);
+// The kernels' view of the counted form's scratch.
+static SetArgs set_args(const Planes& pl, int n0, int n1, int order, const SetLayout& L, char* base) {
     SetArgs a{};
     a.pl = pl;
     a.binom = reinterpret_cast<const long long*>(base + L.binom);
     a.lf = reinterpret_cast<const float*>(base + L.lf);
-    a.n_lf = N + 2;
+    a.n_lf = n0 + n1 + 2;
     for (int t = 1; t < order; ++t) a.sub[t] = reinterpret_cast<uint32_t*>(base + L.sub[t]);
     a.total = (uint32_t)n0 + ((uint32_t)n1 << 16);
     a.n_sets = choose_ll(pl.M, order);
+    return a;
+}
+
+cudaError_t launch_set_scan(const Planes& pl, const double* lf64, int n0, int n1, int order, int k, int sms,
+                            unsigned cap, void* scratch, void* h_ctrl, int32_t* out_snps, double* out_s,
+                            ThresholdInfo* info, cudaStream_t st) {
+    const int N = n0 + n1;
+    const SetLayout L = set_layout(pl.M, N, order);
+    char* const base = static_cast<char*>(scratch);
+    const SetArgs a = set_args(pl, n0, n1, order, L, base);
+    cap = list_cap(a.n_sets, order, cap);
     // |FP32 score - K2|: the table's entries and the two subtractions round by 2^-24 of lf(r + 1) at
     // most, and the cells' lf(r + 1) sum to at most lf(N + 3^K); each addition rounds by 2^-24 of the
     // score.  Both with a margin, plus the subtraction's own rounding of small terms.
@@ -1047,12 +1191,28 @@ cudaError_t launch_set_scan(const Planes& pl, const double* lf64, int n0, int n1
     const float delta = (float)(std::ldexp(1.0, -24) * (6.0 * top + cells * score) * 1.1 + 0.01);
     set_tables_kernel<<<sms, 256, 0, st>>>(pl.M, lf64, N + 2, reinterpret_cast<long long*>(base + L.binom),
                                            reinterpret_cast<float*>(base + L.lf));
+    info->launches = 1;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     SetCtrl* const hc = static_cast<SetCtrl*>(h_ctrl);
-    if (order == 4) return set_scan_k<4>(a, L, lf64, sms, k, delta, base, hc, out_snps, out_s, done, st);
-    if (order == 5) return set_scan_k<5>(a, L, lf64, sms, k, delta, base, hc, out_snps, out_s, done, st);
-    return set_scan_k<6>(a, L, lf64, sms, k, delta, base, hc, out_snps, out_s, done, st);
+    if (order == 4) return set_scan_k<4>(a, L, lf64, sms, k, delta, cap, base, hc, out_snps, out_s, info, st);
+    if (order == 5) return set_scan_k<5>(a, L, lf64, sms, k, delta, cap, base, hc, out_snps, out_s, info, st);
+    return set_scan_k<6>(a, L, lf64, sms, k, delta, cap, base, hc, out_snps, out_s, info, st);
+}
+
+cudaError_t launch_quad_tied(const Planes& pl, const double* lf64, int n0, int n1, float thr, int k, void* tables,
+                             void* scratch, int32_t* out_snps, double* out_s, int* launches, cudaStream_t st) {
+    const SetArgs a = set_args(pl, n0, n1, 4, set_layout(pl.M, n0 + n1, 4), static_cast<char*>(tables));
+    const long long blocks = (a.n_sets + kPairBlock - 1) / kPairBlock;
+    Item* const items = static_cast<Item*>(scratch);
+    set_tied_kernel<4><<<(unsigned)blocks, kTiedThreads, 0, st>>>(a, lf64, thr, k, items);
+    cudaError_t e = cudaGetLastError();
+    const Item* best = nullptr;
+    if (e == cudaSuccess) e = merge_items(items, blocks * k, k, items, items + blocks * k, &best, launches, st);
+    if (e != cudaSuccess) return e;
+    order_emit_kernel<4><<<1, 512, 0, st>>>(best, k, a.pl.M, nullptr, 0u, out_snps, out_s);
+    *launches += 2;
+    return cudaGetLastError();
 }
 
 long long order_count(int M, int order) { return choose_ll(M, order); }
@@ -1063,9 +1223,9 @@ size_t order_scan_scratch(int M, int order, int k) {
 }
 
 cudaError_t launch_order_scan(const Planes& pl, const double* lf64, int order, int k, void* scratch,
-                              int32_t* out_snps, double* out_s, cudaStream_t st) {
-    if (order == 5) return order_scan_k<5>(pl, lf64, k, scratch, out_snps, out_s, st);
-    if (order == 6) return order_scan_k<6>(pl, lf64, k, scratch, out_snps, out_s, st);
+                              int32_t* out_snps, double* out_s, int* launches, cudaStream_t st) {
+    if (order == 5) return order_scan_k<5>(pl, lf64, k, scratch, out_snps, out_s, launches, st);
+    if (order == 6) return order_scan_k<6>(pl, lf64, k, scratch, out_snps, out_s, launches, st);
     return cudaErrorInvalidValue;
 }
 
@@ -1077,31 +1237,23 @@ size_t quad_scan_scratch(int M, int k) {
 }
 
 cudaError_t launch_quad_scan(const Planes& pl, const double* lf64, int n0, int n1, int k,
-                             void* scratch, int32_t* out_snps, double* out_s, cudaStream_t st) {
+                             void* scratch, int32_t* out_snps, double* out_s, int* launches, cudaStream_t st) {
     const long long n_sets = choose_ll(pl.M, 4);
-    long long blocks = (n_sets + kPairBlock - 1) / kPairBlock;
-    Item* a = static_cast<Item*>(scratch);
-    Item* b = a + blocks * k;
+    const long long blocks = (n_sets + kPairBlock - 1) / kPairBlock;
+    Item* const a = static_cast<Item*>(scratch);
     quad_score_kernel<<<(unsigned)blocks, kQuadThreads, 0, st>>>(pl, lf64, n0, n1, n_sets, k, a);
     cudaError_t e = cudaGetLastError();
-    long long n = blocks * k;
-    while (e == cudaSuccess && blocks > 1) {
-        blocks = (n + kPairBlock - 1) / kPairBlock;
-        pair_merge_kernel<<<(unsigned)blocks, kPairThreads, 0, st>>>(a, n, k, b);
-        e = cudaGetLastError();
-        n = blocks * k;
-        Item* t = a;
-        a = b;
-        b = t;
-    }
+    const Item* best = nullptr;
+    if (e == cudaSuccess) e = merge_items(a, blocks * k, k, a, a + blocks * k, &best, launches, st);
     if (e != cudaSuccess) return e;
-    quad_emit_kernel<<<1, 512, 0, st>>>(a, k, out_snps, out_s);
+    quad_emit_kernel<<<1, 512, 0, st>>>(best, k, out_snps, out_s);
+    *launches += 2;
     return cudaGetLastError();
 }
 
 namespace {
 struct PairLayout {
-    size_t ctrl, cand, fin, best, sample, total;
+    size_t ctrl, cand, fin, best, merge, sample, total;
     long long n_sample;
 };
 PairLayout pair_layout(long long n) {
@@ -1116,8 +1268,9 @@ PairLayout pair_layout(long long n) {
     L.n_sample = n < 32768 ? n : 32768;
     L.ctrl = take(sizeof(SetCtrl));
     L.cand = take(sizeof(SetCand) * kSetCand);
-    L.fin = take(sizeof(Item) * kPairBlock);
+    L.fin = take(sizeof(Item) * kSetCand);
     L.best = take(sizeof(Item) * EPI3_MAX_TOPK);
+    L.merge = take(sizeof(Item) * 2 * kMergeItems);
     L.sample = take(sizeof(float) * (size_t)L.n_sample);
     L.total = o;
     return L;
@@ -1127,40 +1280,31 @@ PairLayout pair_layout(long long n) {
 size_t pair_filter_scratch(long long n_pairs) { return pair_layout(n_pairs).total; }
 
 cudaError_t launch_pair_filter(const PairTables& pt, const double* lf64, int M, int k, const CmpBoundTerms& bound,
-                               int sms, void* scratch, void* h_ctrl, int32_t* out_pairs, double* out_s, bool* done,
-                               cudaStream_t st) {
+                               int sms, unsigned cap, void* scratch, void* h_ctrl, int32_t* out_pairs, double* out_s,
+                               ThresholdInfo* info, cudaStream_t st) {
     const PairLayout L = pair_layout(pt.n_pairs);
     char* const base = static_cast<char*>(scratch);
-    SetCtrl* const ctrl = reinterpret_cast<SetCtrl*>(base + L.ctrl);
-    SetCand* const cand = reinterpret_cast<SetCand*>(base + L.cand);
-    Item* const fin = reinterpret_cast<Item*>(base + L.fin);
-    Item* const best = reinterpret_cast<Item*>(base + L.best);
     float* const sample = reinterpret_cast<float*>(base + L.sample);
-    SetCtrl* const hc = static_cast<SetCtrl*>(h_ctrl);
-    *done = false;
-    pair_sample_kernel<<<(unsigned)((L.n_sample + 255) / 256), 256, 0, st>>>(pt, lf64, M, pt.n_pairs / L.n_sample,
-                                                                             L.n_sample, sample);
-    set_threshold_kernel<<<1, 1024, 0, st>>>(sample, 1, L.n_sample, nullptr, k, 0.f, ctrl);
+    cap = list_cap(pt.n_pairs, 2, cap);
+    const long long stride = pt.n_pairs / L.n_sample;
+    pair_sample_kernel<<<(unsigned)((L.n_sample + 255) / 256), 256, 0, st>>>(pt, lf64, M, stride, L.n_sample, sample);
+    set_threshold_kernel<<<1, 1024, 0, st>>>(sample, 1, L.n_sample, nullptr, k, 0.f, stride, cap,
+                                             reinterpret_cast<SetCtrl*>(base + L.ctrl));
+    info->launches = 2;
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
     const dim3 grid((M + 255) / 256, M < 8192 ? M : 8192);
-    for (int attempt = 0; attempt < 4; ++attempt) {
-        pair_filter_kernel<<<grid, 256, 0, st>>>(pt, lf64, M, bound.c, bound.off2, bound.minor, ctrl, cand, kSetCand);
-        set_threshold_kernel<<<1, 1024, 0, st>>>(&cand->s, sizeof(SetCand) / sizeof(float), kSetCand,
-                                                 &ctrl->n_cand, k, 0.f, ctrl);
-        pair_rescore_kernel<<<sms, 256, 0, st>>>(pt, lf64, M, ctrl, cand, kSetCand, fin, kPairBlock);
-        set_final_kernel<<<1, kPairThreads, 0, st>>>(ctrl, fin, k, best);
-        pair_emit_kernel<<<1, 512, 0, st>>>(best, k, M, out_pairs, out_s);
-        cudaError_t e = cudaMemcpyAsync(hc, ctrl, sizeof(SetCtrl), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e == cudaSuccess) e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        if (hc->n_cand <= kSetCand) {
-            *done = hc->n_final <= (unsigned)kPairBlock;
-            return cudaSuccess;
-        }
-        e = cudaMemsetAsync(&ctrl->n_cand, 0, sizeof(unsigned), st);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
+    return threshold_passes(
+        k, 0.f, cap, base, L.ctrl, L.cand, L.fin, L.best, L.merge, static_cast<SetCtrl*>(h_ctrl), info, st,
+        [&](SetCtrl* c, SetCand* cand) {
+            pair_filter_kernel<<<grid, 256, 0, st>>>(pt, lf64, M, bound.c, bound.off2, bound.minor, c, cand, cap);
+        },
+        [&](SetCtrl* c, const SetCand* cand, Item* fin) {
+            pair_rescore_kernel<<<sms, 256, 0, st>>>(pt, lf64, M, c, cand, cap, fin);
+        },
+        [&](const Item* top, const SetCtrl* c) {
+            pair_emit_kernel<<<1, 512, 0, st>>>(top, k, M, c, cap, out_pairs, out_s);
+        });
 }
 
 size_t pair_scan_scratch(long long n_pairs, int k) {
@@ -1168,26 +1312,18 @@ size_t pair_scan_scratch(long long n_pairs, int k) {
     return (size_t)2 * (size_t)blocks * (size_t)k * sizeof(Item);
 }
 
-cudaError_t launch_pair_scan(const PairTables& pt, const double* lf64, int M, int k,
-                             void* scratch, int32_t* out_pairs, double* out_s, cudaStream_t st) {
+cudaError_t launch_pair_scan(const PairTables& pt, const double* lf64, int M, float thr, int k,
+                             void* scratch, int32_t* out_pairs, double* out_s, int* launches, cudaStream_t st) {
     const long long n_pairs = pt.n_pairs;
-    long long blocks = (n_pairs + kPairBlock - 1) / kPairBlock;
-    Item* a = static_cast<Item*>(scratch);
-    Item* b = a + blocks * k;
-    pair_score_kernel<<<(unsigned)blocks, kPairThreads, 0, st>>>(pt, lf64, M, n_pairs, k, a);
+    const long long blocks = (n_pairs + kPairBlock - 1) / kPairBlock;
+    Item* const a = static_cast<Item*>(scratch);
+    pair_score_kernel<<<(unsigned)blocks, kPairThreads, 0, st>>>(pt, lf64, M, n_pairs, thr, k, a);
     cudaError_t e = cudaGetLastError();
-    long long n = blocks * k;
-    while (e == cudaSuccess && blocks > 1) {
-        blocks = (n + kPairBlock - 1) / kPairBlock;
-        pair_merge_kernel<<<(unsigned)blocks, kPairThreads, 0, st>>>(a, n, k, b);
-        e = cudaGetLastError();
-        n = blocks * k;
-        Item* t = a;
-        a = b;
-        b = t;
-    }
+    const Item* best = nullptr;
+    if (e == cudaSuccess) e = merge_items(a, blocks * k, k, a, a + blocks * k, &best, launches, st);
     if (e != cudaSuccess) return e;
-    pair_emit_kernel<<<1, 512, 0, st>>>(a, k, M, out_pairs, out_s);
+    pair_emit_kernel<<<1, 512, 0, st>>>(best, k, M, nullptr, 0u, out_pairs, out_s);
+    *launches += 2;
     return cudaGetLastError();
 }
 
