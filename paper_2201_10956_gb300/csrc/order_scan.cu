@@ -28,8 +28,8 @@
 //     #(.., 2, ..) = #(.., any, ..) - #(.., 0, ..) - #(.., 1, ..),
 // both classes in one register and one three-input subtraction per cell: 4 SNPs of 120 with 2000
 // samples 13.9 -> 2.41 ms, 5 of 48 with 1500 59.2 -> 1.37 ms.  The direct forms
-// (81, 243 or 729 cells counted, every set scored in FP64) serve what the counted form refuses:
-// tables of the smaller sets past kSubsetBytes, or, with five and six SNPs, more sets tied at the k-th
+// (81, 243 or 729 cells counted, every set scored in FP64) serve what the counted form refuses: a few
+// sets, tables of the smaller sets past kSubsetBytes, or, with five and six SNPs, more sets tied at the k-th
 // score than the list of candidates holds; with four, every set is then counted the same way and
 // scored in FP64 (launch_quad_tied).
 //
@@ -1152,6 +1152,10 @@ cudaError_t set_scan_k(const SetArgs& a, const SetLayout& L, const double* lf64,
 // Scratch bytes of the counted form, 0 if it does not serve the size.
 size_t set_scan_scratch(int M, int N, int order) {
     if (order < 4 || order > 6 || M < order) return 0;
+    // A few sets take the direct form: up to one a thread (four SNPs) or one a warp of its first block
+    // it needs two launches instead of eleven and more (4 SNPs of 10 with 2000 samples, 210 sets: 153 us,
+    // counted 178; of 11, 330 sets: 195 and 176; 6 of 7: 402 and 661; 5 of 7, 21 sets: 384 and 275).
+    if (choose_ll(M, order) <= (order == 4 ? kQuadThreads : kOrdThreads / 32)) return 0;
     double sub = 0.0, c = 1.0;
     for (int t = 1; t < order; ++t) {
         c = c * (M - t + 1) / t;
