@@ -41,3 +41,10 @@ def test_forms_in_turn():
     for m, n, n1, k in [(700, 80, 30, 12), (50, 900, 400, 300), (690, 64, 64, 7), (30, 128, 0, 9)]:
         g, ph = pins.tiny_data(m, n, n1, seed=2500 + m)
         _check(g, ph, k)
+
+
+@pytest.mark.parametrize("m", [3, 4, 9, 10, 11, 12])
+@pytest.mark.parametrize("n,n1", [(60, 25), (65536, 30001)])
+def test_few_snps(m, n, n1):
+    g, ph = pins.tiny_data(m, n, n1, seed=2450 + m)
+    _check(g, ph, min(7, m * (m - 1) * (m - 2) // 6))
