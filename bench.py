@@ -48,6 +48,9 @@ L2_FLUSH_BYTES = 512 << 20    # > 129 MB L2
 # an entry is removed whenever that kernel changes.
 TRAFFIC = {
     ("mma4", "large"): 567.59e6 + 7.07e6,   # scan_mma_kernel<e2m1> (plain form), 2048 x 16384
+    # scan_cmp_kernel (paired form), 2048 x 16384: one scan's seven range launches (the unit `achieved`
+    # is taken over), each of its 14.2 GB of chunks read twice on average
+    ("mma4c", "large"): 30.57e9 + 5.5e6,
 }
 FP32_PER_SM_CLK = 128         # FP32 lane operations per SM per clock
 EPILOGUE_OPS = 192            # of them per triplet in the compacted scan's table-free bound

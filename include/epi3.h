@@ -124,9 +124,10 @@ int epi3_scan_range(epi3_handle* h, int64_t pair_begin, int64_t pair_end, int32_
 /*
  * Pairwise (second-order) scan: Eq. 1 applied to two SNPs (3^2 cells x {control, case},
  * cell = 3 gX + gY; the paper states the score for any number of interacting SNPs).  Every
- * pair i < j is scored in FP64 from its exact table, summed in cell order 0..8 with the same
- * log-factorial table as the triplet rescoring; the top_k pairs by (K2 ascending, then i, j)
- * are returned.
+ * pair i < j is bounded from below from its exact table in FP32; the pairs whose bound does not
+ * exceed an upper bound of the k-th score are scored in FP64, summed in cell order 0..8 with
+ * the same log-factorial table as the triplet rescoring (every pair where more tie at the k-th
+ * score than a list holds); the top_k pairs by (K2 ascending, then i, j) are returned.
  *   top_k        1..min(EPI3_MAX_TOPK, C(M,2)).
  *   out_pairs    [top_k][2] int32, i < j, 0-based;  out_scores [top_k] FP64 K2, ascending.
  * Outputs are host memory unless the handle was created with EPI3_DEVICE_PTRS.  Returns
@@ -265,10 +266,12 @@ typedef struct {
        issuer spent issuing tcgen05.mma / commit instructions */
     float wait_loader, wait_mma_operands, wait_mma_accum, wait_producers, wait_epilogue;
     float wait_producers_tmem, mma_issue;
-    /* tensor-core scan: a table whose approximate K2 (Stirling's form with the hardware log,
-       no table lookups) exceeds the candidate threshold by more than this proven bound is
-       skipped without its exact FP32 score; the bound comes from the approximation's error
-       measured on the device for every count 0..N+1 */
+    /* tensor-core scans skip a table without its exact FP32 score where a bound from below, found
+       without table lookups, lies above the candidate threshold.  One-hot form: K2 by Stirling's
+       form with the hardware log, less this figure, which comes from the approximation's error
+       measured on the device for every count 0..N+1.  EPI3_PATH_MMA4C: a parabola below the
+       binary entropy plus the logs of the cell sizes; this figure is the part of its constant
+       that covers Stirling's remainders and rounding (the parabola's own slack comes on top) */
     float k2_prune_bound;
     /* sample-compacted form (EPI3_PATH_MMA4C): device time of the compaction kernels, a part
        of scan_kernel_ms (0 for the other forms) */
@@ -297,13 +300,12 @@ int epi3_get_stats(const epi3_handle* h, epi3_stats* out);
  *   top_k, out_triplets, out_scores   as epi3_scan, but the outputs are device pointers.
  *   cuda_stream            stream to run on (NULL = the legacy default stream).
  *
- * It counts with the 8-cell POPC scan (EPI3_PATH_POPC8, about 18 T sample-triplets/s on
- * GB300) where the pair tables fit the scratch too (up to some 600 SNPs), with the 27-cell one
- * (EPI3_PATH_POPC, about 5 T) beyond, not with the tensor-core form epi3_scan uses by default,
- * and its candidate list has a
- * fixed 65536 entries with no retry: a data set with more near-tied FP32 candidates gives
- * EPI3_ERR_OVERFLOW where epi3_scan would grow the list.  The answer is the one epi3_scan
- * gives.
+ * It counts with the 8-cell POPC scan (EPI3_PATH_POPC8) where the pair tables fit the scratch
+ * too (11 to some 600 SNPs; the whole call does 13.6 T sample-triplets/s at 400 x 5003 on
+ * GB300), with the 27-cell one (EPI3_PATH_POPC, about 5 T) elsewhere, not with the tensor-core
+ * form epi3_scan uses by default, and its candidate list has a fixed 65536 entries with no
+ * retry: a data set with more near-tied FP32 candidates gives EPI3_ERR_OVERFLOW where
+ * epi3_scan would grow the list.  The answer is the one epi3_scan gives.
  *
  * All scratch lives in one file-scope __device__ array of EPI3_NOALLOC_SCRATCH_BYTES that
  * every GPU loading the library holds until the process exits.  The first call on a device
@@ -321,9 +323,10 @@ int epi3_scan_noalloc(const uint8_t* genotypes, const uint8_t* phenotype, int32_
 
 /*
  * Batches: many independent data sets ("cohorts") of uneven size scanned together.  Each
- * cohort is packed like epi3_create; a cohort too small to fill the GPU alone joins the
- * shared one-hot tensor launch, every other one gets the handle tuner's measured choice for its
- * shape (8-cell POPC, the compacted tensor form in launches of its own, or the shared one-hot
+ * cohort is packed like epi3_create; the smallest (up to some 210 SNPs) join the shared one-hot
+ * tensor launch, those of up to some 490 SNPs take the compacted tensor form in launches of
+ * their own, larger ones get the handle tuner's measured choice for their
+ * shape (8-cell POPC, the compacted form, or the shared one-hot
  * launch; per M/64, N/1024 bucket; persisted in the file named by EPI3_TUNE_CACHE;
  * EPI3_BATCH_PATH = mma | mma4c | popc8 forces one).  The one-hot tensor cohorts share ONE
  * persistent tcgen05 launch over all their tiles; the whole scan + candidate stages + read-back is captured once in a CUDA graph and
@@ -348,7 +351,8 @@ int epi3_batch_create(epi3_batch** b, int32_t n_cohorts, const epi3_cohort* coho
 int epi3_batch_scan(epi3_batch* b, int32_t top_k, int32_t* out_triplets, double* out_scores);
 int epi3_batch_destroy(epi3_batch* b);
 /* Figures of the last epi3_batch_scan: scan_kernel_ms = total_ms = device time of the graph
- * replay; pack_ms holds the tuner's time at create. */
+ * replay; pack_ms holds the tuner's time at create; path = the cohorts' common path, or
+ * EPI3_PATH_AUTO where they differ. */
 int epi3_batch_get_stats(const epi3_batch* b, epi3_stats* out);
 /* The path the tuner chose for each cohort: EPI3_PATH_MMA4 (the shared one-hot tensor launch),
  * EPI3_PATH_MMA4C (compaction + compacted scan launches of its own in the graph) or
@@ -356,8 +360,8 @@ int epi3_batch_get_stats(const epi3_batch* b, epi3_stats* out);
  * one for every cohort. */
 int epi3_batch_get_paths(const epi3_batch* b, int32_t* out_paths);
 /* The tensor-scan form of each cohort: 0 = not a tensor cohort, 1 = plain, 2 = register-split
- * (one-hot) or paired (compacted), -1 = not measured yet.  Compacted cohorts take the handle
- * tuner's form for their shape.  All one-hot cohorts share one persistent launch and so one form,
+ * (one-hot) or paired (compacted), -1 = not measured yet.  Compacted cohorts are paired, or take
+ * the handle tuner's form where it chose their path.  All one-hot cohorts share one persistent launch and so one form,
  * measured on the first epi3_batch_scan by replaying the batch in both forms (the environment
  * variable EPI3_BATCH_FORM = "plain" | "split" forces one).  The tile (128 rows (j, b) x 256
  * columns (k, z) of the one-hot operands) is the kernel's only one: the tensor-memory budget

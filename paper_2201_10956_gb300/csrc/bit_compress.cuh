@@ -1,5 +1,5 @@
-// Bit extraction for the sample compaction of the tensor scan, usable from host and device code
-// (the host tests check it against a plain bit loop).
+// Bit extraction, usable from host and device code (the host tests check it against a plain bit
+// loop).  No kernel includes it: the sample compaction gathers samples and transposes their bits.
 #pragma once
 
 #include <cstdint>

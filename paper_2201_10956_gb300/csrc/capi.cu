@@ -311,7 +311,7 @@ struct epi3_handle {
     Ctrl* h_ctrl = nullptr;       // pinned
     double* h_scores = nullptr;   // pinned [EPI3_MAX_TOPK]
     int* h_trip = nullptr;        // pinned [EPI3_MAX_TOPK * 3]
-    int path = EPI3_PATH_AUTO;          // scan path (option "path"); auto = E2M1 tensor form
+    int path = EPI3_PATH_AUTO;          // scan path (option "path"); auto = the tuner's choice
     int threads = 128;
     int ctas_per_sm = 0;
     bool timing = false;
@@ -1993,12 +1993,13 @@ int tune_path(epi3_batch* b, epi3_handle* h, int* path_out, float* ms) {
     // timed alone, yet in the batch its tiles share one persistent launch with every other
     // cohort's (its marginal cost there is its tiles' share of that launch, at the
     // throughput-bound rate, several times the POPC forms').  Timing it alone would be biased
-    // against the shared launch, so the choice comes from whole batches of eight equal cohorts:
+    // against the shared launch, so the choice comes from whole batches of equal cohorts:
     // the smallest take the shared launch; up to 64 tiles an SM the paired compacted form, in
-    // launches of its own, which there is the faster of the two at 1500, 6000 and 18000 samples (ms a
-    // cohort at 6000, one-hot and compacted: 140 SNPs 0.124 and 0.154, 180 SNPs 0.169 and 0.177, 220
-    // SNPs 0.263 and 0.210, 300 SNPs 0.500 and 0.329, 480 SNPs 1.460 and 0.654).  The rest get the
-    // handle tuner's measured choice for their shape.
+    // launches of its own, which there takes 0.32 to 0.79 of the one-hot launch's time in batches of 1,
+    // 2, 4, 8 and 16 cohorts of 64 to 60000 samples (ms of a batch of one and of 16, one-hot and
+    // compacted: 211 SNPs x 500 samples 0.29 and 0.23, 3.7 and 2.7, the closest; 340 x 6000 1.07 and
+    // 0.42, 14.6 and 5.9; 480 x 60000 8.0 and 2.9, 125 and 44).  The rest get the handle tuner's
+    // measured choice for their shape.
     const long long tiles = mma_tile_estimate(h->M);
     if (tiles < kBatchSharedTiles * b->sm_count) { *path_out = EPI3_PATH_MMA4; return EPI3_OK; }
     if (tiles < 64LL * b->sm_count) {

@@ -365,7 +365,9 @@ __host__ __device__ __forceinline__ int2 relabel_marg(int2 m, int nc, int d) {
     return d == 0 ? make_int2(m.y, n2) : d == 1 ? make_int2(m.x, n2) : m;
 }
 // The same for the FP32 pair-table row (X, Z) (+ 3 each, index 2 a + z) with Z's marginal + 9
-// (exact: integers below 2^24).
+// (exact: integers below 2^24), and below the cells' way back: no kernel takes these two since the
+// stagers relabel integers and cmp_score walks the genotypes in order; the host check of the
+// relabelling is written with them.
 __host__ __device__ __forceinline__ float4 relabel_xz(float4 x, float2 mz9, int d) {
     if (d == 2) return x;
     const float r0 = (mz9.x - x.x) - x.z, r1 = (mz9.y - x.y) - x.w;

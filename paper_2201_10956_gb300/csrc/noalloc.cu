@@ -4,9 +4,9 @@
 // budget, and frameworks whose caching allocator owns the device memory (a raw
 // cudaMalloc/cudaFree there can fail or implicitly synchronise the device).  For them this
 // entry point runs the class split, the packing, a POPC scan (8 cells counted and 19 derived where
-// the pair tables fit the scratch beside the rest -- up to some 600 SNPs --, about 18 T
-// sample-triplets/s on GB300; else all 27 cells, about 5 T; not the tensor-core form that
-// epi3_scan picks by default), the candidate band, FP64 rescoring and the final order, with
+// the pair tables fit the scratch beside the rest -- 11 to some 600 SNPs; the whole call does 13.6 T
+// sample-triplets/s at 400 SNPs x 5003 samples on GB300 --; else all 27 cells, about 5 T; not the
+// tensor-core form that epi3_scan picks by default), the candidate band, FP64 rescoring and the final order, with
 // every piece of scratch memory (class counts, packed bit planes, pair tables, log-factorial
 // tables, control block, candidate lists) in one file-scope device array of kScratchBytes;
 // the log-factorial tables are staged in file-scope host arrays.  The caller passes device

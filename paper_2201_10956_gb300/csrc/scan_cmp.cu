@@ -36,10 +36,10 @@
 // is bounded; on timeout the kernel records kStTimeout, waits for its own copies and MMAs, frees
 // tensor memory and returns.
 //
-// Measured (GB300, scan kernel without the compaction): 2048 SNPs x 4096 samples 46.0 -> 21.4 ms,
-// 2048 x 16384 50.2 -> 31.4 ms.  At 4096 samples a tile takes 8800 cycles, of which the FP32 pipe
-// is busy 3800 (the bound); at 16 384 it takes 12 900, of which the tensor pipe's operand reads and
-// the ring's hand-offs alone take 10 300.
+// Measured (GB300, scan kernel without the compaction): 2048 SNPs x 4096 samples 46.0 -> 18.6 ms,
+// 2048 x 16384 50.2 -> 29.5 ms.  At 4096 samples a tile takes 7600 cycles, of which the bound's
+// operations take the FP32 pipe 3070; at 16 384 it takes 12 100, of which the tensor pipe's operand
+// reads and the ring's hand-offs alone take 10 300.
 #include <algorithm>
 #include <atomic>
 #include <type_traits>

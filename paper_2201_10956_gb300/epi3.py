@@ -217,7 +217,7 @@ class Handle:
         return pairs, sc
 
     def scan_order(self, order: int, top_k: int):
-        """Scan of interaction order 2, 3 or 4 (Eq. 1 for that many SNPs): top-k SNP sets
+        """Scan of interaction order 2 to 6 (Eq. 1 for that many SNPs): top-k SNP sets
         (int32 [k, order]) and FP64 K2 ([k])."""
         sets = self._alloc((top_k, order), np.int32)
         sc = self._alloc((top_k,), np.float64)
@@ -367,8 +367,8 @@ def scan_noalloc(genotypes, phenotype, top_k: int, stream=None):
 
     For callers that cannot allocate (fixed memory budgets, foreign allocators); the
     outputs are allocated here by torch, the scratch is the library's static device array
-    (8 MiB).  It runs the 27-cell POPC scan and synchronises the stream, so it is not for
-    a capturing stream.  Returns (triplets int32 [k, 3], scores float64 [k]) on the device.
+    (8 MiB).  It runs a POPC scan (8 cells counted where the pair tables fit the scratch, else 27)
+    and synchronises the stream, so it is not for a capturing stream.  Returns (triplets int32 [k, 3], scores float64 [k]) on the device.
     """
     import torch
     m, n = genotypes.shape
